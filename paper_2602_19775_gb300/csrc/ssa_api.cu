@@ -33,12 +33,12 @@ cudaError_t launch_backward_thread(const AdjParams &p, int readout, int block, s
                                    cudaStream_t st);
 cudaError_t launch_reduce_partials(const float *partial, int64_t nblk, int M, const int *rate_index, int P,
                                    float *dA_tmp, float *dtheta, cudaStream_t st);
-cudaError_t launch_forward_warp(const FwdParams &p, int readout, bool record, int warps, size_t smem, cudaStream_t st);
+cudaError_t launch_forward_warp(const FwdParams &p, int readout, bool record, int warps, size_t limit, cudaStream_t st);
 cudaError_t launch_forward_warp_soft(const FwdParams &p, int readout, bool record, int warps, size_t smem,
                                      cudaStream_t st);
 cudaError_t launch_backward_warp_soft(const AdjParams &p, const int *upd, uint32_t upd_words, int readout, int warps,
                                       size_t smem, int64_t grid, cudaStream_t st);
-cudaError_t launch_backward_warp(const AdjParams &p, int readout, int warps, size_t smem, int64_t grid,
+cudaError_t launch_backward_warp(const AdjParams &p, int readout, int warps, size_t limit, int64_t grid,
                                  cudaStream_t st);
 int thread_kernel_mc(int M);
 cudaError_t launch_exp_variates(const uint32_t *words, int64_t n, float *out, cudaStream_t st);
@@ -293,7 +293,7 @@ extern "C" ssa_status ssa_create_network(int32_t n_species, int32_t n_reactions,
     std::vector<std::vector<int>> upd_by_species(n_species);
     for (int j = 0; j < n_reactions; ++j)
         for (int e = stoich_ptr[j]; e < stoich_ptr[j + 1]; ++e)
-            upd_by_species[stoich_species[e]].push_back((((j + 1) & 3) * nb_warp + ((j + 1) >> 2)) << 8 |
+            upd_by_species[stoich_species[e]].push_back(jpos(j, nb_warp) << 8 |
                                                         (stoich_delta[e] & 0xff));
     const int upd_ptr_pad = (n_species + 1 + 3) / 4 * 4;
     std::vector<int> upd(upd_ptr_pad, 0);
@@ -303,6 +303,47 @@ extern "C" ssa_status ssa_create_network(int32_t n_species, int32_t n_reactions,
     }
     for (int sp = n_species + 1; sp < upd_ptr_pad; ++sp) upd[sp] = upd[n_species];
     upd.resize((upd.size() + 3) / 4 * 4, 0);
+    // the warp kernels' second table region (WarpTab): the entries of v_j by wide position, and per species the
+    // reactions it reacts in, homodimers last. Networks past these sizes are refused by those kernels (shared
+    // memory).
+    const bool has_wtab = n_species <= kEntMaxSpecies && n_reactions <= kEntMaxReactions;
+    const int wtab_ent = 4 * wide_len(n_reactions);
+    std::vector<int> wtab(has_wtab ? wtab_ent + 4 * (n_species + 1) : 0, 0);
+    auto list_entry = [&](int j) { return jpos(j, nb_warp) << 16 | wpos(j); };
+    if (has_wtab) {
+        std::fill(wtab.begin(), wtab.begin() + wtab_ent, (int)((uint32_t)n_species << 18));
+        for (int j = 0; j < n_reactions; ++j) {
+            int *en = &wtab[4 * wpos(j)];
+            const int cnt = stoich_ptr[j + 1] - stoich_ptr[j];
+            if (cnt > 4) {
+                en[0] = kEntMany;
+                wtab[wtab_ent + 4 * n_species + 3] = 1;
+            }
+            for (int e = 0; e < cnt && cnt <= 4; ++e) {
+                const float d = (float)stoich_delta[stoich_ptr[j] + e];  // at most 7 bits: exact in bf16
+                uint32_t bits;
+                memcpy(&bits, &d, 4);
+                en[e] = (int)(bits >> 16 | (uint32_t)stoich_species[stoich_ptr[j] + e] << 18);
+            }
+        }
+        std::vector<std::vector<int>> plain(n_species), homo(n_species);
+        for (int j = 0; j < n_reactions; ++j) {
+            if (rx[j].x < 0) continue;
+            (rx[j].x == rx[j].y ? homo : plain)[rx[j].x].push_back(list_entry(j));
+            if (rx[j].y >= 0 && rx[j].y != rx[j].x) plain[rx[j].y].push_back(list_entry(j));
+        }
+        std::vector<int> list;
+        for (int sp = 0; sp < n_species; ++sp) {
+            int *c = &wtab[wtab_ent + 4 * sp];
+            c[0] = (int)list.size();
+            list.insert(list.end(), plain[sp].begin(), plain[sp].end());
+            c[1] = (int)list.size();
+            list.insert(list.end(), homo[sp].begin(), homo[sp].end());
+            c[2] = (int)list.size();
+        }
+        wtab.insert(wtab.end(), list.begin(), list.end());
+    }
+    wtab.resize((wtab.size() + 3) / 4 * 4, 0);
     const int inc_ptr_pad = (n_species + 1 + 3) / 4 * 4;
     const int inc_list_pad = ((int)inc_list.size() + 3) / 4 * 4;
     inc_ptr.resize(inc_ptr_pad, inc_ptr[n_species]);
@@ -322,7 +363,9 @@ extern "C" ssa_status ssa_create_network(int32_t n_species, int32_t n_reactions,
     // blob = [tables][rate_index: int Mp][tables again, with rx in the warp kernels' lane-major order]
     //        [species-major update list of the warp soft forward]
     net->upd_words = (uint32_t)upd.size();
-    const size_t bytes = 2 * (size_t)net->tab_bytes + (size_t)Mp * 4 + 4 * (size_t)net->upd_words;
+    net->wtab_bytes = (uint32_t)(4 * wtab.size());
+    const size_t bytes =
+        2 * (size_t)net->tab_bytes + (size_t)Mp * 4 + 4 * (size_t)net->upd_words + (size_t)net->wtab_bytes;
     cudaError_t e = cudaMalloc(&net->d_blob, bytes);
     if (e != cudaSuccess) {
         delete net;
@@ -345,10 +388,12 @@ extern "C" ssa_status ssa_create_network(int32_t n_species, int32_t n_reactions,
     if (e == cudaSuccess) e = cudaMemcpy(net->d_rx_warp, net->d_rx, net->tab_bytes, cudaMemcpyDeviceToDevice);
     net->d_upd = reinterpret_cast<int *>(b + 2 * (size_t)net->tab_bytes + (size_t)Mp * 4);
     if (e == cudaSuccess) e = cudaMemcpy(net->d_upd, upd.data(), 4 * (size_t)net->upd_words, cudaMemcpyHostToDevice);
+    net->d_wtab = reinterpret_cast<int4 *>(net->d_upd + net->upd_words);  // every part before it is a multiple of 16
+    if (e == cudaSuccess) e = cudaMemcpy(net->d_wtab, wtab.data(), net->wtab_bytes, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         const int nb = (n_reactions + 4) >> 2;
         std::vector<int4> rxp(Mp, make_int4(-1, -1, 0, 0));
-        for (int j = 0; j < n_reactions; ++j) rxp[((j + 1) & 3) * nb + ((j + 1) >> 2)] = rx[j];
+        for (int j = 0; j < n_reactions; ++j) rxp[jpos(j, nb)] = rx[j];
         e = cudaMemcpy(net->d_rx_warp, rxp.data(), 16 * (size_t)Mp, cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
@@ -475,6 +520,8 @@ static ssa_status forward_impl(const ssa_network *net, const float *log_rates, i
     p.invT = opts->selector == SSA_SELECT_SOFT ? 1.0f / opts->temperature : 0.0f;
     p.upd = net->d_upd;
     p.upd_words = net->upd_words;
+    p.wtab = net->d_wtab;
+    p.wtab_bytes = net->wtab_bytes;
     p.obs_out = obs_out;
     p.draws = reinterpret_cast<int *>(ws + L.draws);
     p.status = reinterpret_cast<int *>(ws + L.status);
@@ -501,7 +548,7 @@ static ssa_status forward_impl(const ssa_network *net, const float *log_rates, i
         CUDA_TRY(launch_forward_warp_soft(p, opts->readout, opts->record != 0, kWarpsPerBlock, fwd_warp_soft_smem(net),
                                           st));
     else
-        CUDA_TRY(launch_forward_warp(p, opts->readout, opts->record != 0, kWarpsPerBlock, fwd_warp_smem(net), st));
+        CUDA_TRY(launch_forward_warp(p, opts->readout, opts->record != 0, kWarpsPerBlock, limit, st));
     if (n_traj > 0 && draws_out) CUDA_TRY(cudaMemcpyAsync(draws_out, p.draws, (size_t)n_traj * 4, cudaMemcpyDeviceToDevice, st));
     if (n_traj > 0 && status_out) CUDA_TRY(cudaMemcpyAsync(status_out, p.status, (size_t)n_traj * 4, cudaMemcpyDeviceToDevice, st));
     if (run_out) {
@@ -597,6 +644,8 @@ static ssa_status backward_setup(ssa_run *run, const float *dl_dobs, int64_t dl_
     p.Mp = net->Mp;
     p.inc_off = net->inc_off;
     p.inc_list_off = net->inc_list_off;
+    p.wtab = net->d_wtab;
+    p.wtab_bytes = net->wtab_bytes;
     p.nnz = net->nnz;
     p.n_traj = run->n_traj;
     p.traj_offset = run->traj_offset;
@@ -650,7 +699,7 @@ extern "C" ssa_status ssa_backward(ssa_run *run, const float *dl_dobs, int64_t d
         CUDA_TRY(launch_backward_warp_soft(p, net->d_upd, net->upd_words, run->opts.readout, kWarpsPerBlock,
                                            adj_warp_soft_smem(net), grid, st));
     else
-        CUDA_TRY(launch_backward_warp(p, run->opts.readout, kWarpsPerBlock, adj_warp_smem(net), grid, st));
+        CUDA_TRY(launch_backward_warp(p, run->opts.readout, kWarpsPerBlock, smem_limit(), grid, st));
     CUDA_TRY(launch_reduce_partials(p.partial, grid, net->M, net->d_rate_index, net->P,
                                     reinterpret_cast<float *>(ws + run->L.dA), dl_dlog_rates, st));
     return SSA_OK;

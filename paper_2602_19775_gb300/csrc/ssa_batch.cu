@@ -56,9 +56,11 @@ struct BatchUnit {
 constexpr int kBatchWarps = 4;
 constexpr int kBatchThreadMaxN = 16;  // thread variant inside a batch: N <= 16 and M <= 16
 // Resident blocks per SM the warp-unit kernels are compiled for (a tuning constant: more blocks hide more
-// latency, fewer leave more of the SM's 256 KB to L1, through which the batch kernels read their tables).
+// latency, fewer let each trajectory run faster, which counts where one long trajectory ends a launch, and leave
+// more of the SM's 256 KB to L1, through which the batch kernels read their tables). 24 networks, 9,468
+// trajectories with up to 32,768 draws: 6 blocks 380 ms, 5 300, 4 240, 3 221.
 #ifndef SSA_BATCH_WARP_BLOCKS
-#define SSA_BATCH_WARP_BLOCKS 5
+#define SSA_BATCH_WARP_BLOCKS 4
 #endif
 constexpr int kBatchWarpBlocks = SSA_BATCH_WARP_BLOCKS;
 constexpr int kBatchWarpUnit = 1;     // trajectories per warp-variant unit (one: the finest grain for the tail)
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
     extern __shared__ __align__(16) int bsm[];
     BatchItem *s_items = reinterpret_cast<BatchItem *>(bsm);
     const int wib = threadIdx.x >> 5;
-    int *Xw = bsm + kItemWords * kBatchWarps + wib * x_words;
+    int *Xw = bsm + kItemWords * (blockDim.x >> 5) + wib * x_words;
     int cached = -1;
     for (;;) {
         const int ui = next_unit(counter);
@@ -165,9 +167,10 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
             }
         } else {
             const FwdParams &p = b.f;
-            const int *st = reinterpret_cast<const int *>(reinterpret_cast<const unsigned char *>(p.rx) + 16 * p.Mp);
+            const WarpTab tab = warp_tab(p, p.rx, p.wtab, p.k_rates);
+            float *a = reinterpret_cast<float *>(Xw) + ((p.N + 3) & ~3);
             for (int c = 0; c < u.count; ++c) {
-                warp_fwd_body<READOUT, true>(p, p.rx, st, p.k_rates, Xw, u.traj_begin + c);
+                warp_fwd_body<READOUT, true>(p, tab, Xw, a, u.traj_begin + c);
                 __syncwarp();
             }
         }
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
     extern __shared__ __align__(16) float bsa[];
     BatchItem *s_items = reinterpret_cast<BatchItem *>(bsa);
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    float *wsm = bsa + kItemWords * kBatchWarps + wib * w_words;
+    float *wsm = bsa + kItemWords * (blockDim.x >> 5) + wib * w_words;
     int cached = -1;
     for (;;) {
         const int ui = next_unit(counter);
@@ -230,12 +233,12 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
             const AdjParams &p = b.a;
             const int Npad = (p.N + 3) & ~3;
             const int4 *rx = p.rx;
-            const unsigned char *tb = reinterpret_cast<const unsigned char *>(p.rx);
-            const int *st = reinterpret_cast<const int *>(tb + 16 * p.Mp);
-            const int *inc_ptr = reinterpret_cast<const int *>(tb + p.inc_off);
-            const int *inc = reinterpret_cast<const int *>(tb + p.inc_list_off);
             float *dA;
             if constexpr (SOFT) {
+                const unsigned char *tb = reinterpret_cast<const unsigned char *>(p.rx);
+                const int *st = reinterpret_cast<const int *>(tb + 16 * p.Mp);
+                const int *inc_ptr = reinterpret_cast<const int *>(tb + p.inc_off);
+                const int *inc = reinterpret_cast<const int *>(tb + p.inc_list_off);
                 // the soft forward's gradient: Xs [kSoftK][Npad], lam, dX [Npad]; a, h, y, c1, c2, dA [Mp]
                 float *Xs = wsm;
                 float *lam = Xs + kSoftK * Npad;
@@ -260,22 +263,24 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
                 int *X = reinterpret_cast<int *>(wsm);
                 float *lam = wsm + Npad;
                 float *aj = lam + Npad;
-                float *lj = aj + p.Mp;
-                float *ct = lj + p.Mp;
-                dA = ct + p.Mp;
-                for (int j = lane; j < p.Mp; j += 32) dA[j] = 0.0f;
+                const int Mw = wide_len(p.M);
+                float *lj = aj + Mw;
+                float *ct = lj + Mw;
+                dA = ct + Mw;
+                const WarpTab tab = warp_tab(p, rx, p.wtab, p.k_rates);
+                for (int j = lane; j < Mw; j += 32) dA[j] = 0.0f;
                 __syncwarp();
                 for (int c = 0; c < u.count; ++c) {
                     const int64_t i = u.traj_begin + c;
                     const int stt = p.status[i];
                     if (stt == SSA_TRAJ_OK || stt == SSA_TRAJ_ABSORBED || stt == SSA_TRAJ_STEP_CAP)
-                        warp_adj_body<READOUT>(p, rx, st, inc_ptr, inc, p.k_rates, X, lam, aj, lj, ct, dA, i, stt);
+                        warp_adj_body<READOUT>(p, tab, X, lam, aj, lj, ct, dA, i, stt);
                     __syncwarp();
                 }
             }
             float *slot = p.partial + b.slot_off + (int64_t)u.slot * p.M;
             const int nb = (p.M + 4) >> 2;
-            for (int j = lane; j < p.M; j += 32) slot[j] = dA[jpos(j, nb)];
+            for (int j = lane; j < p.M; j += 32) slot[j] = dA[SOFT ? jpos(j, nb) : wpos(j)];
         }
         __syncwarp();
     }
@@ -340,6 +345,7 @@ struct ssa_batch {
     int x_words[2] = {0, 0}, w_words[2] = {0, 0};
     int fwd_blocks[2] = {0, 0}, adj_blocks[2] = {0, 0};
     size_t fwd_smem[2] = {0, 0}, adj_smem[2] = {0, 0};
+    int warps[2] = {0, 0};  // per block
     std::vector<BatchItem> h_items;
     cudaGraphExec_t graph = nullptr;
     bool ready = false;
@@ -613,6 +619,8 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
         p.invT = bt->soft ? a.invT : 0.0f;  // the soft forward's T is the gradient's
         p.upd = net->d_upd;
         p.upd_words = net->upd_words;
+        p.wtab = a.wtab = net->d_wtab;
+        p.wtab_bytes = a.wtab_bytes = net->wtab_bytes;
         a.partial = partial;
         a.mismatch = flag + 2;
         a.err = flag + 1;
@@ -684,12 +692,12 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
     for (int it = 0; it < n_items; ++it)
         if (bt->variant[it] != 1) {
             maxNw = std::max(maxNw, bt->items[it].net->N);
-            maxMpw = std::max(maxMpw, bt->items[it].net->Mp);
+            maxMpw = std::max(maxMpw, bt->soft ? bt->items[it].net->Mp : wide_len(bt->items[it].net->M));
         }
     const int maxNpad = (maxNw + 3) & ~3;
     bt->x_words[0] = kBatchThreadMaxN * 32;
     bt->w_words[0] = 3 * kBatchThreadMaxN * 32;
-    bt->x_words[1] = bt->soft ? 2 * maxNpad + maxMpw : maxNpad;
+    bt->x_words[1] = bt->soft ? 2 * maxNpad + maxMpw : maxNpad + maxMpw;
     bt->w_words[1] = bt->soft ? (kSoftK + 2) * maxNpad + 6 * maxMpw : 2 * maxNpad + 4 * maxMpw;
     int dev = 0, sms = 0, limit = 0;
     CUDA_TRY_B(cudaGetDevice(&dev));
@@ -712,19 +720,24 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
                             : (ro == 0 ? (const void *)batch_adj_kernel<0, 32>
                                        : ro == 1 ? (const void *)batch_adj_kernel<1, 32> : (const void *)batch_adj_kernel<2, 32>)};
     for (int v = 0; v < 2; ++v) {
-        bt->fwd_smem[v] = (size_t)kBatchWarps * (kItemWords + bt->x_words[v]) * 4;
-        bt->adj_smem[v] = (size_t)kBatchWarps * (kItemWords + bt->w_words[v]) * 4;
+        // a block of four warps, of fewer where the arrays of the largest network leave no room for four
+        const size_t words = kItemWords + (size_t)std::max(bt->x_words[v], bt->w_words[v]);
+        bt->warps[v] = kBatchWarps;
+        if (v == 1 && !bt->soft)
+            while (bt->warps[v] > 1 && bt->warps[v] * words * 4 > (size_t)limit) --bt->warps[v];
+        bt->fwd_smem[v] = (size_t)bt->warps[v] * (kItemWords + bt->x_words[v]) * 4;
+        bt->adj_smem[v] = (size_t)bt->warps[v] * (kItemWords + bt->w_words[v]) * 4;
         if (bt->n_units[v] == 0) continue;
         if (bt->fwd_smem[v] > (size_t)limit || bt->adj_smem[v] > (size_t)limit)
             return set_error(SSA_ERR_UNSUPPORTED, "a network in the batch is too large for the batch kernels");
         int per_sm_f = 0, per_sm_a = 0;
         CUDA_TRY_B(cudaFuncSetAttribute(fk[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bt->fwd_smem[v]));
         CUDA_TRY_B(cudaFuncSetAttribute(ak[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bt->adj_smem[v]));
-        CUDA_TRY_B(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, fk[v], 32 * kBatchWarps, bt->fwd_smem[v]));
-        CUDA_TRY_B(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, ak[v], 32 * kBatchWarps, bt->adj_smem[v]));
+        CUDA_TRY_B(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_f, fk[v], 32 * bt->warps[v], bt->fwd_smem[v]));
+        CUDA_TRY_B(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_a, ak[v], 32 * bt->warps[v], bt->adj_smem[v]));
         if (per_sm_f < 1 || per_sm_a < 1) return set_error(SSA_ERR_UNSUPPORTED, "batch kernels do not fit on an SM");
         // one persistent wave, never more warps than units
-        const int64_t need_blocks = (bt->n_units[v] + kBatchWarps - 1) / kBatchWarps;
+        const int64_t need_blocks = (bt->n_units[v] + bt->warps[v] - 1) / bt->warps[v];
         bt->fwd_blocks[v] = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm_f, need_blocks));
         bt->adj_blocks[v] = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * per_sm_a, need_blocks));
     }
@@ -737,7 +750,7 @@ template <int R>
 static void batch_launch_kernels(const ssa_batch *bt, cudaStream_t st)
 {
     const BatchUnit *u0 = bt->d_units + bt->unit_begin[0], *u1 = bt->d_units + bt->unit_begin[1];
-    const dim3 blk(32 * kBatchWarps);
+    const dim3 blk(32 * bt->warps[0]), blkw(32 * bt->warps[1]);
     if (bt->n_units[0] > 0) {  // thread units: forward then adjoint
         batch_fwd_kernel<R, 1><<<bt->fwd_blocks[0], blk, bt->fwd_smem[0], st>>>(bt->d_items, u0, bt->n_units[0],
                                                                               bt->d_counters, bt->x_words[0]);
@@ -745,14 +758,14 @@ static void batch_launch_kernels(const ssa_batch *bt, cudaStream_t st)
                                                                               bt->d_counters + 1, bt->w_words[0]);
     }
     if (bt->n_units[1] > 0 && bt->soft) {  // warp units of a soft batch
-        batch_fwd_kernel<R, 32, true><<<bt->fwd_blocks[1], blk, bt->fwd_smem[1], st>>>(
+        batch_fwd_kernel<R, 32, true><<<bt->fwd_blocks[1], blkw, bt->fwd_smem[1], st>>>(
             bt->d_items, u1, bt->n_units[1], bt->d_counters + 2, bt->x_words[1]);
-        batch_adj_kernel<R, 32, true><<<bt->adj_blocks[1], blk, bt->adj_smem[1], st>>>(
+        batch_adj_kernel<R, 32, true><<<bt->adj_blocks[1], blkw, bt->adj_smem[1], st>>>(
             bt->d_items, u1, bt->n_units[1], bt->d_counters + 3, bt->w_words[1]);
     } else if (bt->n_units[1] > 0) {  // warp units
-        batch_fwd_kernel<R, 32><<<bt->fwd_blocks[1], blk, bt->fwd_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
+        batch_fwd_kernel<R, 32><<<bt->fwd_blocks[1], blkw, bt->fwd_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
                                                                                bt->d_counters + 2, bt->x_words[1]);
-        batch_adj_kernel<R, 32><<<bt->adj_blocks[1], blk, bt->adj_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
+        batch_adj_kernel<R, 32><<<bt->adj_blocks[1], blkw, bt->adj_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
                                                                                bt->d_counters + 3, bt->w_words[1]);
     }
 }

@@ -31,6 +31,12 @@ __device__ __forceinline__ float int2f(int x)
     return __int2float_rn(x);
 }
 
+// the same for an x known to lie in [0, 2^23)
+__device__ __forceinline__ float small2f(int x)
+{
+    return __fsub_rn(__uint_as_float(0x4B000000u | (unsigned)x), 8388608.0f);
+}
+
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw, SC'11): ten rounds, two 32x32->64 products each,
 // round keys bumped by the two Weyl increments.
 __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1)
@@ -96,7 +102,7 @@ __device__ __forceinline__ float mass_action_h_sel(const int4 rx, const int *X)
     const int xr2 = X[rx.y >= 0 ? rx.y : 0];
     const int x2 = homo ? max(x1 - 1, 0) : (rx.y >= 0 ? xr2 : 1);
     if ((unsigned)(x1 | x2) >= (1u << 23)) return mass_action_h(rx, X, 1);
-    const float h = __fmul_rn(int2f(x1), int2f(x2));
+    const float h = __fmul_rn(small2f(x1), small2f(x2));
     return homo ? h * 0.5f : h;
 }
 
@@ -139,6 +145,48 @@ __device__ __forceinline__ int stoich_delta(int e) { return (int)(signed char)(e
 // Exponential variate E = -ln u of a uniform u in (0, 1), the one function every kernel draws its
 // waiting times and race variates with (CUDA's logf, within one unit in the last place).
 __device__ __forceinline__ float neg_log_unit(float u) { return -logf(u); }
+
+// 1/v for a normal v, 2 ulp; log2 and exp2 of the special function unit without the handling of subnormals
+__device__ __forceinline__ float rcp_approx(float v)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float lg2_approx(float v)
+{
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+__device__ __forceinline__ float ex2_approx(float v)
+{
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+// 1/E = -1/ln u of the uniform of a Philox word, for the adjoints' soft weights (the forward's clock and race use
+// neg_log_unit). With v = 1 - u, 1/E = 1/v - P(v) where P = 1/v + 1/ln(1 - v) is smooth (1/2 + v/12 + v^2/24 + ...):
+// below v = 1/2 a degree-6 fit of P (weighted least squares towards the smallest relative error of 1/E, 2^-25.9)
+// and one approximate reciprocal; above it ln u is away from 0 and the hardware log2 is accurate in relative terms.
+// 16 issue slots against 32 of logf and a division.
+__device__ __forceinline__ float inv_exp_of_word(uint32_t x)
+{
+    const float v = u01(~x);
+    float p = 0x1.7ce56ep-4f;
+    p = __fmaf_rn(p, v, -0x1.4636e4p-4f);
+    p = __fmaf_rn(p, v, 0x1.0f75e4p-4f);
+    p = __fmaf_rn(p, v, 0x1.c8f8ccp-7f);
+    p = __fmaf_rn(p, v, 0x1.63387p-5f);
+    p = __fmaf_rn(p, v, 0x1.54e3ecp-4f);
+    p = __fmaf_rn(p, v, 0x1.00004ep-1f);
+    const float near = rcp_approx(v) - p, far = rcp_approx(lg2_approx(1.0f - v) * -0x1.62e430p-1f);
+    float r;  // a select, never a branch
+    asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %3, 0f3F000000;\n\tselp.f32 %0, %1, %2, p;\n\t}"
+        : "=f"(r) : "f"(near), "f"(far), "f"(v));
+    return r;
+}
 
 // Exponential variates of one step, E[q] = -ln u_q for the first NQ words of the step's Philox
 // stream (q = 0 drives the waiting time, q = 1 + j reaction j). They do not depend on the state,
@@ -416,6 +464,8 @@ struct FwdParams {
     float invT;       // soft forward (Eq. 4): 1/T of its soft sample
     const int *upd;   // warp soft forward: species-major update list (ssa_network::d_upd), upd_words ints
     uint32_t upd_words;
+    const int4 *wtab;  // warp kernels' second table region (ssa_network::d_wtab), wtab_bytes long
+    uint32_t wtab_bytes;
     void *obs_out;
     int *draws, *status;
     const int *flag;  // workspace error flags (bad sample times -> every trajectory BAD_INPUT)
@@ -469,6 +519,8 @@ struct AdjParams {
     // several temperatures in one walk (network-specialised kernels): 1/T_t, t < the kernel's count; the
     // block sums of temperature t go to partial + t gridDim.x M
     float invT_multi[4];
+    const int4 *wtab;  // as in FwdParams
+    uint32_t wtab_bytes;
 };
 
 

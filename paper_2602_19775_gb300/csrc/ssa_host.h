@@ -21,6 +21,9 @@ struct ssa_network {
     // [upd_ptr: int N+1, padded to 4][upd_list: (jpos(j) << 8) | (delta & 0xff), reactions in increasing j]
     int *d_upd;
     uint32_t upd_words;
+    // second table region of the warp kernels (WarpTab): [ent: int4 Mp][inc: int4 N+1][list: int, padded to 4]
+    int4 *d_wtab;
+    uint32_t wtab_bytes;
     int *d_stoich;
     int *d_rate_index;
     uint32_t tab_bytes;

@@ -22,11 +22,34 @@ struct NetTables {
     uint32_t tab_bytes;  // 16 * M + 4 * nnz_pad, a multiple of 16
 };
 
-// Per-warp view of a step's inputs (warp-per-trajectory kernels).
-struct FwdParamsView {
-    const int4 *s_rx;
-    const float *s_k;
-    int M, nb;
+// What a warp-per-trajectory kernel reads of the network, in shared or global memory. Its per-reaction values live
+// at wide positions (wpos): round c, word q and lane l of reaction j's word at 128 c + 32 q + l, so that a lane's
+// addresses differ by constants and the lanes of an access lie side by side.
+//   rx, k     reactants and rates, lane-major (jpos)
+//   ent[w]    by wide position, up to four entries (species, change) of v_j, each (4 species << 16) | bf16 bits of
+//             the change; an absent entry is species N with change 0, whose list in inc is empty and whose lambda
+//             slot holds 0; a reaction with more entries is marked by ent[w].x = kEntMany and read from
+//             st[rx.z .. rx.w)
+//   inc[s]    {begin, first homodimer, end} of species s in list: the reactions it reacts in, each
+//             (jpos << 16) | wpos; inc[N].w: whether any reaction is marked
+struct WarpTab {
+    const int4 *rx;
+    const int *st;
+    const int4 *ent;
+    const int4 *inc;
+    const int *list;
+    const float *k;
+    int M, nb, rounds;  // reactions, Philox blocks per step, blocks per lane rounded up
+    bool many;
+};
+constexpr int kEntMany = 0xffff;  // species 0, a change that is no number
+constexpr int kEntMaxSpecies = 0x3ffe, kEntMaxReactions = 0x7000;
+__device__ __forceinline__ int ent_offset(int e) { return (int)((unsigned)e >> 16); }  // bytes into an array by species
+__device__ __forceinline__ int ent_species(int e) { return (int)((unsigned)e >> 18); }
+__device__ __forceinline__ float ent_change(int e) { return __int_as_float(e << 16); }
+
+// Per-trajectory constants of the noise.
+struct WarpNoise {
     uint32_t c2, c3, key0, key1;
 };
 
@@ -34,7 +57,15 @@ struct FwdParamsView {
 // driven by word q = (j + 1) % 4 of Philox block b = (j + 1) / 4, which lane b % 32 draws; storing it
 // at q * nb + b (nb = number of blocks) puts the entries the 32 lanes read for one word q side by
 // side, so those shared-memory accesses are free of bank conflicts.
-__device__ __forceinline__ int jpos(int j, int nb) { return ((j + 1) & 3) * nb + ((j + 1) >> 2); }
+__host__ __device__ __forceinline__ int jpos(int j, int nb) { return ((j + 1) & 3) * nb + ((j + 1) >> 2); }
+
+__host__ __device__ __forceinline__ int wpos(int j)
+{
+    const int b = (j + 1) >> 2;
+    return ((b >> 5) << 7) + (((j + 1) & 3) << 5) + (b & 31);
+}
+// length of an array by wide position
+__host__ __device__ __forceinline__ int wide_len(int M) { return ((((M + 4) >> 2) + 31) >> 5) << 7; }
 
 // Warp reductions shared by the warp-per-trajectory kernels (butterfly: every lane gets the same
 // bits; the race keeps the lowest j on equal products).
@@ -68,6 +99,12 @@ __device__ __forceinline__ float warp_max(float v)
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
     return v;
+}
+
+// largest of 32 values under the order of their bit patterns (non-negative floats order like their bits)
+__device__ __forceinline__ float warp_max_nonneg(float v)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
 }
 
 // ------------------------------------------------------------------------------------------
@@ -125,18 +162,20 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t phase,
 constexpr uint32_t kWaitLimit = 1u << 24;
 
 
-// Stage `tab_bytes` of tables and `k_bytes` of rate constants (both multiples of 16, both
-// 16-byte aligned) into s_tab / s_k. Every thread of the block must call this. Returns false
+// Stage `tab_bytes` of tables, `k_bytes` of rate constants and `more_bytes` of a second table region (multiples
+// of 16, 16-byte aligned; the last may be 0) into s_tab / s_k / s_more. Every thread of the block must call this. Returns false
 // (and sets err_flag) if the copy did not complete within the bound.
 __device__ __forceinline__ bool stage_tables(void *s_tab, const void *g_tab, uint32_t tab_bytes, void *s_k,
                                              const void *g_k, uint32_t k_bytes, uint64_t *bar,
-                                             int *s_ok, int *err_flag)
+                                             int *s_ok, int *err_flag, void *s_more = nullptr,
+                                             const void *g_more = nullptr, uint32_t more_bytes = 0)
 {
     if (threadIdx.x == 0) {
         mbar_init(bar, 1);
-        mbar_arrive_expect_tx(bar, tab_bytes + k_bytes);
+        mbar_arrive_expect_tx(bar, tab_bytes + k_bytes + more_bytes);
         bulk_copy_g2s(s_tab, g_tab, tab_bytes, bar);
         bulk_copy_g2s(s_k, g_k, k_bytes, bar);
+        if (more_bytes) bulk_copy_g2s(s_more, g_more, more_bytes, bar);
         bool ok = mbar_wait_bounded(bar, 0, kWaitLimit);
         if (!ok) {
             atomicOr(err_flag, kErrStageTimeout);

@@ -2,78 +2,207 @@
 // the single-network kernels and the batch kernel.
 #pragma once
 
-#include "ssa_adj_body.cuh"
+#include <type_traits>
 
-// Philox blocks a lane draws together in the adjoint's first pass (the forward draws four); a tuning
-// constant: more blocks give the scheduler more independent work but keep more registers live.
-#ifndef SSA_WARP_ADJ_CHUNK
-#define SSA_WARP_ADJ_CHUNK 1
-#endif
+#include "ssa_adj_body.cuh"
 
 namespace ssa {
 
-// One step's propensities, a0 and race over this lane's Philox blocks b = lane, lane + 32, ...
-// Returns E_0 on lane 0. If aj / lj are given, stores a_j and log2(a_j / E_j) (or -inf) for this
-// lane's reactions. The forward takes the lane's blocks four at a time: their Philox words and
-// variates are drawn first (four independent dependency chains for the scheduler to interleave), then
-// the reactions are evaluated in increasing j, so the sums and the race see the same values in the
-// same order as the adjoint's one-block-at-a-time loop (which keeps fewer values live).
-template <bool STORE>
-__device__ __forceinline__ void warp_step_eval(const FwdParamsView &v, int k, const int *X, float &a0, float &E0,
-                                               float &ab, float &Eb, int &jb, float *aj, float *lj, float &lmax)
+// The network's tables for one launch: rx (then st) and the second region, both in shared or both in global
+// memory.
+template <class P>
+__device__ __forceinline__ WarpTab warp_tab(const P &p, const int4 *rx, const int4 *wtab, const float *k)
 {
-    constexpr int CH = STORE ? SSA_WARP_ADJ_CHUNK : 4;
+    const int4 *inc = wtab + wide_len(p.M);
+    const int nb = (p.M + 4) >> 2;
+    return WarpTab{rx, reinterpret_cast<const int *>(rx + p.Mp), wtab, inc, reinterpret_cast<const int *>(inc + p.N + 1),
+                   k, p.M, nb, (nb + 31) >> 5, inc[p.N].w != 0};
+}
+
+// ------------------------------------------------------------------------------------------
+// Propensities kept between steps. An event changes a few species and so a few propensities; a warp keeps all
+// of them in shared memory by lane-major position and forms again, from the new counts, those of the reactions
+// its event touches (the same expression, so the same bits as forming every one each step). On a 301-reaction
+// network with 11 species an event touches ~50 reactions.
+// SIGNED (the adjoint): where a_j = 0 the array holds -D_j instead, D_j = k_j dh_j/dX for the reactant at zero
+// (the waiting-time path's derivative there, with k_j times the other count; homodimers, whose derivative
+// needs no other count, hold 0), so that a_j = max(value, 0).
+// ------------------------------------------------------------------------------------------
+template <bool SIGNED>
+__device__ __forceinline__ float warp_propensity(const WarpTab &t, int pos, const int *X)
+{
+    const int4 rx = t.rx[pos];
+    const float k = t.k[pos];
+    if (!SIGNED) return __fmul_rn(k, mass_action_h_sel(rx, X));
+    const bool homo = rx.y >= 0 && rx.y == rx.x;
+    const int x1 = rx.x >= 0 ? X[rx.x >= 0 ? rx.x : 0] : 1;
+    const int xr2 = X[rx.y >= 0 ? rx.y : 0];
+    const int x2 = homo ? max(x1 - 1, 0) : (rx.y >= 0 ? xr2 : 1);
+    float d = small2f(max(x1, x2));
+    float h = __fmul_rn(small2f(x1), small2f(x2));
+    if ((unsigned)(x1 | x2) >= (1u << 23)) {
+        h = mass_action_h(rx, X, 1);
+        d = __int2float_rn(max(x1, x2));
+    } else if (homo) {
+        h *= 0.5f;
+    }
+    const float a = __fmul_rn(k, h);
+    return a > 0.0f ? a : (homo ? 0.0f : -(k * d));
+}
+
+template <bool SIGNED>
+__device__ __forceinline__ void warp_propensities_all(const WarpTab &t, const int *X, float *a)
+{
     const int lane = threadIdx.x & 31;
-    float a0p = 0.0f;
-    E0 = 0.0f;
-    ab = 0.0f;
-    Eb = 1.0f;
-    jb = -1;
-    lmax = -CUDART_INF_F;
-    const int n_rounds = (v.nb + 31) >> 5;  // blocks per lane, rounded up
-    for (int t0 = 0; t0 < n_rounds; t0 += CH) {
-        float E[CH][4];
-#pragma unroll
-        for (int t = 0; t < CH; ++t) {
-            const int b = lane + 32 * (t0 + t);
-            if (b < v.nb) {
-                const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, v.c2, v.c3), v.key0, v.key1);
-                E[t][0] = neg_log_unit(u01(r.x));
-                E[t][1] = neg_log_unit(u01(r.y));
-                E[t][2] = neg_log_unit(u01(r.z));
-                E[t][3] = neg_log_unit(u01(r.w));
-            }
+    for (int c = 0; c < t.rounds; ++c)
+        for (int q = 0; q < 4; ++q) {
+            const int b = 32 * c + lane;
+            a[128 * c + 32 * q + lane] = b < t.nb ? warp_propensity<SIGNED>(t, q * t.nb + b, X) : 0.0f;
         }
-#pragma unroll
-        for (int t = 0; t < CH; ++t) {
-            const int b = lane + 32 * (t0 + t);
-            if (b >= v.nb) break;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                // predicated rather than branched: word 0 of lane 0's first block (j = -1) drives the waiting
-                // time, and its table slot, like the padded ones (j >= M), has rate 0, so it adds 0 to a0, never
-                // wins the race (a_j E_b > a_b E_j fails for a_j = 0) and its key is -inf (log2 0)
-                const int j = 4 * b + q - 1;
-                if (q == 0 && j < 0) E0 = E[t][0];
-                const int pos = q * v.nb + b;
-                const float a = __fmul_rn(v.s_k[pos], mass_action_h_sel(v.s_rx[pos], X));
-                a0p = __fadd_rn(a0p, a);
-                race(a, E[t][q], j, ab, Eb, jb);
-                if (STORE) {
-                    const float l = __log2f(a) - __log2f(E[t][q]);
-                    lmax = fmaxf(lmax, l);
-                    if (j >= 0 && j < v.M) {
-                        aj[pos] = a;
-                        lj[pos] = l;
-                    }
-                }
-            }
+    __syncwarp();
+}
+
+// after a change of the species named by four entries: the reactions on their lists, one lane each
+template <bool SIGNED>
+__device__ __forceinline__ void warp_propensities_touched(const WarpTab &t, const int4 en, const int *X, float *a)
+{
+    const int4 c0 = t.inc[ent_species(en.x)], c1 = t.inc[ent_species(en.y)], c2 = t.inc[ent_species(en.z)],
+               c3 = t.inc[ent_species(en.w)];
+    const int o1 = c0.z - c0.x, o2 = o1 + c1.z - c1.x, o3 = o2 + c2.z - c2.x, tot = o3 + c3.z - c3.x;
+    for (int q = threadIdx.x & 31; q < tot; q += 32) {
+        const int e = q < o1 ? c0.x + q : q < o2 ? c1.x + (q - o1) : q < o3 ? c2.x + (q - o2) : c3.x + (q - o3);
+        const int le = t.list[e];
+        a[le & 0xffff] = warp_propensity<SIGNED>(t, le >> 16, X);
+    }
+}
+
+// X += sign v_j, then the touched propensities; all lanes
+template <bool SIGNED>
+__device__ __forceinline__ void warp_apply(const WarpTab &t, int j, int sign, int *X, float *a)
+{
+    const int lane = threadIdx.x & 31;
+    const int4 en = t.ent[wpos(j)];
+    if (!t.many || en.x != kEntMany) {
+        const int e = lane == 0 ? en.x : lane == 1 ? en.y : lane == 2 ? en.z : en.w;
+        const int d = (int)ent_change(e);
+        if (lane < 4 && d != 0) X[ent_species(e)] += sign * d;  // the entries of one reaction name distinct species
+        __syncwarp();
+        warp_propensities_touched<SIGNED>(t, en, X, a);
+    } else {
+        const int4 rj = t.rx[jpos(j, t.nb)];
+        for (int e = rj.z + lane; e < rj.w; e += 32) X[stoich_species(t.st[e])] += sign * stoich_delta(t.st[e]);
+        __syncwarp();
+        for (int e = rj.z; e < rj.w; ++e) {
+            const int4 c = t.inc[stoich_species(t.st[e])];
+            for (int q = c.x + lane; q < c.z; q += 32)
+                a[t.list[q] & 0xffff] = warp_propensity<SIGNED>(t, t.list[q] >> 16, X);
         }
     }
-    a0 = warp_sum(a0p);
+    __syncwarp();
+}
+
+// ------------------------------------------------------------------------------------------
+// The Gumbel-max choice without its logarithms. The race argmax_j a_j / E_j, E_j = -ln(1 - v_j) with
+// v_j = 1 - u_j, has a key K_j = a_j / E_j with
+//     a_j (1/v_j - 1/2 - v_j/2)  <=  K_j  <=  a_j (1/v_j - 1/2) =: B_j
+// (1/v + 1/ln(1 - v) = 1/2 + v/12 + v^2/24 + ... has positive coefficients: convex, from 1/2 at v = 0 to 1 at
+// v = 1). Each lane keeps its two largest B_j (one approximate reciprocal each, the slot's number in the six low
+// bits); the largest lower bound over the warp is the threshold. If a single B_j reaches it, less a margin far
+// above every rounding here and in the exact comparison (2^-13 against 2^-16), that reaction wins the race as the
+// binary32 comparisons of E decide it; else the race is run on the variates themselves (warp_race_exact). One
+// logarithm per step remains, E_0's. A logarithm costs 32 issue slots and B_j with its bookkeeping 8.
+// The bounds assume a0 in [2^-40, 2^100] (no B_j of interest is subnormal or overflows) and the slot number
+// six bits, i.e. up to 16 rounds of blocks (M <= 2047); other steps take the exact race.
+// ------------------------------------------------------------------------------------------
+struct WarpTop {
+    float m1, m2;  // the two largest B_j of this lane, low bits replaced
+};
+
+__device__ __forceinline__ void warp_top_add(WarpTop &top, float a, uint32_t x, int slot)
+{
+    const float v = u01(~x);  // 1 - u, exact
+    const float B = a * (rcp_approx(v) - 0.5f);
+    const float key = __uint_as_float((__float_as_uint(B) & ~63u) | (uint32_t)slot);
+    top.m2 = fmaxf(top.m2, fminf(top.m1, key));
+    top.m1 = fmaxf(top.m1, key);
+}
+
+// the winner's lane and slot if it is certain; a_of(slot): this lane's propensity in that slot
+template <class AF>
+__device__ __forceinline__ bool warp_top_decide(const WarpTop &top, float a0, const AF &a_of, int &src, int &slot)
+{
+    const int mine = (int)(__float_as_uint(top.m1) & 63u);
+    const float a1 = a_of(mine);
+    const float half = 0.5f * a1;
+    // a v / 2 with v from B = a (1/v - 1/2)
+    const float width = half * a1 * rcp_approx(top.m1 + half + 1e-30f);
+    const float thr = warp_max_nonneg(fmaxf(top.m1 - width - 0x1p-13f * top.m1, 0.0f));
+    const unsigned c1 = __ballot_sync(0xffffffffu, top.m1 >= thr), c2 = __ballot_sync(0xffffffffu, top.m2 >= thr);
+    src = __ffs(c1) - 1;
+    slot = __shfl_sync(0xffffffffu, mine, src);
+    return c2 == 0 && (c1 & (c1 - 1)) == 0 && a0 >= 0x1p-40f && a0 <= 0x1p100f;
+}
+
+// the race itself over this lane's blocks, with the accurate variates; returns the winner (-1: no positive key)
+static __device__ __noinline__ int warp_race_exact(int rounds, const float *a, int k, WarpNoise z)
+{
+    const int lane = threadIdx.x & 31;
+    float ab = 0.0f, Eb = 1.0f;
+    int jb = -1;
+    for (int c = 0; c < rounds; ++c) {
+        const int b = 32 * c + lane;
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            race(fmaxf(a[128 * c + 32 * q + lane], 0.0f), neg_log_unit(u01(word_of(r, q))), 4 * b + q - 1, ab, Eb, jb);
+    }
     warp_race_combine(ab, Eb, jb);
-    E0 = __shfl_sync(0xffffffffu, E0, 0);
-    if (STORE) lmax = warp_max(lmax);
+    return jb;
+}
+
+// One step of the forward: a0 over this lane's blocks b = lane, lane + 32, ... in increasing j and a butterfly over
+// the lanes, E_0, and the choice. The lane's blocks are drawn four at a time (independent chains for the
+// scheduler).
+__device__ __forceinline__ void warp_step_eval(int n_rounds, int k, const WarpNoise &z, const float *a, float &a0, float &E0,
+                                               int &jb)
+{
+    const int lane = threadIdx.x & 31;
+    float a0p = 0.0f;
+    uint32_t x0 = 0;
+    WarpTop top{0.0f, 0.0f};
+    // C rounds from t0 on; a lane past its last block draws one all the same and finds propensities of 0
+    auto rounds = [&](auto count, int t0) {
+        constexpr int C = decltype(count)::value;
+        uint4 r[C];
+#pragma unroll
+        for (int t = 0; t < C; ++t)
+            r[t] = philox4x32_10(make_uint4((uint32_t)(lane + 32 * (t0 + t)), (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
+        if (t0 == 0) x0 = r[0].x;
+#pragma unroll
+        for (int t = 0; t < C; ++t) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                // the waiting-time word's slot (j = -1) and the padded ones have rate 0: they add 0 to a0 and
+                // never win
+                const float aq = a[128 * (t0 + t) + 32 * q + lane];
+                a0p = __fadd_rn(a0p, aq);
+                warp_top_add(top, aq, word_of(r[t], q), 4 * (t0 + t) + q);
+            }
+        }
+    };
+    int t0 = 0;
+    for (; t0 + 4 <= n_rounds; t0 += 4) rounds(std::integral_constant<int, 4>{}, t0);
+    if (n_rounds & 2) {
+        rounds(std::integral_constant<int, 2>{}, t0);
+        t0 += 2;
+    }
+    if (n_rounds & 1) rounds(std::integral_constant<int, 1>{}, t0);
+    a0 = warp_sum(a0p);
+    E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
+    int src, slot;
+    const bool sure = warp_top_decide(top, a0, [&](int s) { return a[min(s, 4 * n_rounds - 1) * 32 + lane]; }, src, slot);
+    if (sure && n_rounds <= 16) jb = 4 * (src + 32 * (slot >> 2)) + (slot & 3) - 1;
+    else jb = warp_race_exact(n_rounds, a, k, z);
 }
 
 // Bin readout (Section 4.4) on a warp-per-trajectory forward. Every lane runs the same bookkeeping on the
@@ -148,13 +277,12 @@ __device__ __forceinline__ void warp_bin_tail(const FwdParams &p, int64_t i, int
     if (RECORD && (threadIdx.x & 31) == 0) p.brk_tail[i] = slots;
 }
 
-// Per-trajectory body of the warp forward (all 32 lanes of one warp); X = this warp's counts.
+// Per-trajectory body of the warp forward (all 32 lanes of one warp); X, a = this warp's counts and propensities.
 template <int READOUT, bool RECORD>
-__device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const int4 *s_rx, const int *s_st, const float *s_k,
-                                              int *X, const int64_t i)
+__device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const WarpTab &tab, int *X, float *a, const int64_t i)
 {
     const int lane = threadIdx.x & 31;
-    const int N = p.N, M = p.M;
+    const int N = p.N;
     const int64_t n = p.n_traj;
 
     const int *x0 = p.x0 + (p.x0_per_traj ? i * N : 0);
@@ -167,8 +295,8 @@ __device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const int4 *s_
     const bool bad_input = __any_sync(0xffffffffu, neg) || (*p.flag & (kErrBadSamples | kErrBadObs)) != 0;
     __syncwarp();
     const uint64_t gid = p.traj_offset + (uint64_t)i;
-    FwdParamsView v{s_rx, s_k, M, (M + 4) >> 2, (uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed,
-                    (uint32_t)(p.seed >> 32)};
+    const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
+    if (!bad_input) warp_propensities_all<false>(tab, X, a);
 
     double t = 0.0;
     int s = 0;
@@ -189,27 +317,33 @@ __device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const int4 *s_
 
     while (!bad_input) {
         if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
-        float a0, E0, ab, Eb, lmax;
+        float a0, E0;
         int jb;
-        warp_step_eval<false>(v, k, X, a0, E0, ab, Eb, jb, nullptr, nullptr, lmax);
+        warp_step_eval(tab.rounds, k, noise, a, a0, E0, jb);
         if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
         if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
         if (jb < 0) { status = SSA_TRAJ_BAD_RATE; break; }
         const float tau = waiting_time(E0, a0);
         const double t_next = t + f2d_pos(tau);
-        const int4 rj = s_rx[jpos(jb, v.nb)];
+        const int jpb = jpos(jb, tab.nb);
+        const int4 rj = tab.rx[jpb];
         const bool slow = gt_nonneg(t_next, thr);
         const bool cross = slow && gt_nonneg(t_next, p.t_end);
         if (!cross) {
             bool bad_neg = false, bad_ovf = false;
-            for (int e = rj.z + lane; e < rj.w; e += 32) {
-                const int st = s_st[e];
+            if (rj.w - rj.z <= 4) {
+                const int e = reinterpret_cast<const int *>(tab.ent + wpos(jb))[lane & 3];
+                const int x = X[min(ent_species(e), N - 1)], d = (int)ent_change(e);
+                bad_neg = x + d < 0 && d < 0;
+                bad_ovf = d > 0 && x > 2147483647 - d;
+            } else for (int e = rj.z + lane; e < rj.w; e += 32) {
+                const int st = tab.st[e];
                 const int x = X[stoich_species(st)], d = stoich_delta(st);
                 bad_neg |= d < 0 && x + d < 0;
                 bad_ovf |= d > 0 && x > 2147483647 - d;
             }
-            if (__any_sync(0xffffffffu, bad_neg)) status = SSA_TRAJ_NEG_COUNT;
-            else if (__any_sync(0xffffffffu, bad_ovf)) status = SSA_TRAJ_OVERFLOW;
+            if (__any_sync(0xffffffffu, bad_neg || bad_ovf))
+                status = __any_sync(0xffffffffu, bad_neg) ? SSA_TRAJ_NEG_COUNT : SSA_TRAJ_OVERFLOW;
         }
         if (RECORD) {
             e0 = __funnelshift_r(e0, e1, 16);
@@ -241,7 +375,7 @@ __device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const int4 *s_
                         const int sp = p.obs_sp[c];
                         int dv = 0;
                         for (int e = rj.z; e < rj.w; ++e)
-                            if (stoich_species(s_st[e]) == sp) dv += stoich_delta(s_st[e]);
+                            if (stoich_species(tab.st[e]) == sp) dv += stoich_delta(tab.st[e]);
                         o[c] = __fmaf_rn(alpha, (float)dv, (float)X[sp]);
                     }
                     if (RECORD && lane == 0) p.brk_a[(int64_t)s * n + i] = alpha;
@@ -253,11 +387,7 @@ __device__ __forceinline__ void warp_fwd_body(const FwdParams &p, const int4 *s_
             if (cross) break;
         }
         __syncwarp();
-        for (int e = rj.z + lane; e < rj.w; e += 32) {
-            const int st = s_st[e];
-            X[stoich_species(st)] += stoich_delta(st);  // the entries of one reaction name distinct species
-        }
-        __syncwarp();
+        warp_apply<false>(tab, jb, 1, X, a);
         t = t_next;
         ++k;
         if (RECORD && --ck_left == 0) {
@@ -695,16 +825,44 @@ __device__ __forceinline__ void warp_soft_adj_body(const AdjParams &p, const int
     if (lane == 0 && mism) atomicAdd(p.mismatch, mism);
 }
 
-// Per-trajectory body of the warp adjoint (all 32 lanes). X, lam, aj, lj, ct, dA are this warp's buffers;
+// Two keys within this of each other, relatively, count as a possible tie (a key is a few units in the last place
+// off, and so is the comparison of products that decides the race).
+constexpr float kTieMargin = 0x1p-15f;
+
+// The keys of a step whose a0 lies where a_j / E_j could leave the binary32 range, scaled by a power of two (all
+// that follows uses ratios of keys); returns the largest.
+static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *ad, int k, WarpNoise z, float a0, float *rj)
+{
+    const float sc = a0 > 1.0f ? 0x1p-60f : 0x1p100f;
+    const int lane = threadIdx.x & 31;
+    float rmax = 0.0f;
+    for (int c = 0; c < rounds; ++c) {
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)(32 * c + lane), (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int w = 128 * c + 32 * q + lane;
+            const float key = (fmaxf(ad[w], 0.0f) * sc) * inv_exp_of_word(word_of(r, q));
+            rmax = fmaxf(rmax, key);
+            rj[w] = key;
+        }
+    }
+    return warp_max_nonneg(rmax);
+}
+
+// Per-trajectory body of the warp adjoint (all 32 lanes). X, lam [Npad], ad, rj, ct, dA [wide_len] are this warp's
+// buffers, contiguous in that order (lam[N] is read as 0: a padding word, or ad[0], the waiting-time word's slot);
 // dA accumulates over every trajectory the warp processes.
+// Per step: the keys (pass 1), soft weights and w_j = v_j . lambda (pass 2), the per-reaction
+// adjoints g_j = psi_j + dL/da0 a_j (pass 3), which are also all that the state adjoint needs: a_j is
+// proportional to the count of each plain reactant, so lambda_s += (1/X_s) sum g_j over the reactions of s, a
+// homodimer's share carries (2 X - 1) / (X (X - 1)), and where a reactant is absent (a_j = 0) only the
+// waiting-time path remains, dL/da0 D_j. One division per species replaces two per reaction.
 template <int READOUT>
-__device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_rx, const int *s_st,
-                                              const int *s_inc_ptr, const int *s_inc, const float *s_k, int *X,
-                                              float *lam, float *aj, float *lj, float *ct, float *dA, const int64_t i,
-                                              const int st)
+__device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab &tab, int *X, float *lam, float *ad,
+                                              float *rj, float *ct, float *dA, const int64_t i, const int st)
 {
     const int lane = threadIdx.x & 31;
-    const int N = p.N, M = p.M;
+    const int N = p.N, nb = tab.nb, n_rounds = tab.rounds;
     const int64_t n = p.n_traj;
     const int d = p.draws[i];
     const int L = (st == SSA_TRAJ_OK) ? d - 1 : d;
@@ -712,17 +870,22 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
         X[s] = p.xfinal[(int64_t)s * n + i];
         lam[s] = 0.0f;
     }
+    for (int s = N + lane; s < ((N + 3) & ~3); s += 32) lam[s] = 0.0f;
     __syncwarp();
+    warp_propensities_all<true>(tab, X, ad);
     const uint64_t gid = p.traj_offset + (uint64_t)i;
-    FwdParamsView v{s_rx, s_k, M, (M + 4) >> 2, (uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed,
-                    (uint32_t)(p.seed >> 32)};
+    const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
     const float invT = p.invT;
     const float *gl = p.dl_dobs + i * p.dl_stride;
     int row_cached = -1;
-    uint4 row = make_uint4(0, 0, 0, 0);
+    uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
     auto event_at = [&](int kk) -> int {
         const int r = kk >> 3;
-        if (r != row_cached) { row = p.ev[(int64_t)r * n + i]; row_cached = r; }
+        if (r != row_cached) {
+            row = (r == row_cached - 1) ? row_below : p.ev[(int64_t)r * n + i];
+            row_cached = r;
+            if (r > 0) row_below = p.ev[(int64_t)(r - 1) * n + i];
+        }
         const int slot = kk & 7;
         const uint32_t w = word_of(row, slot >> 1);
         return (slot & 1) ? (int)(w >> 16) : (int)(w & 0xffff);
@@ -749,18 +912,12 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
     float mu = 0.0f;
     int mism = 0;
     int ck_row = L / p.K, ck_off = L - ck_row * p.K;
-    // passes 2 and 3 read only shared memory, so the lanes take the 4 nb slots one at a time, 32 per round
-    // (slot pos = q nb + b holds reaction 4 b + q - 1): ceil(4 nb / 32) rounds instead of ceil(nb / 32)
-    // rounds of four slots (at nb = 76, 95% of the lanes busy instead of 79%; below nb = 32, up to four times
-    // fewer rounds). A lane's first slot, as (q, b); it then advances by 32 slots.
-    const int q_first = lane / v.nb, b_first = lane - q_first * v.nb;
-    auto next_slot = [&](int &q, int &b) {
-        b += 32;
-        while (b >= v.nb) {
-            b -= v.nb;
-            ++q;
-        }
-    };
+    // species groups of the state adjoint: with N <= 32 each species gets 32 / 2^ceil(log2 N) lanes that stride over
+    // its list and combine by a butterfly inside the group; with more species each lane takes whole species
+    int pow2 = 1;
+    while (pow2 < N && pow2 < 32) pow2 <<= 1;
+    const int gsz = N <= 32 ? 32 / pow2 : 1;
+    const int g_first = lane / gsz, g_lane = lane % gsz, g_step = 32 / gsz;
 
     for (int k = L; k >= 0; --k) {
         const bool draw = (k < L) || (st == SSA_TRAJ_OK);
@@ -781,13 +938,35 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
         float tau_k = 0.0f;
         if (draw) {
             const int jk = event_at(k);
-            float a0, E0, ab, Eb, lmax;
-            int jb;
-            warp_step_eval<true>(v, k, X, a0, E0, ab, Eb, jb, aj, lj, lmax);
-            mism += (jb != jk);
+            // pass 1: a0, E_0 and the race's keys r_j = a_j / E_j over this lane's blocks; the waiting-time word's
+            // slot and the padded ones have rate 0: they add 0 and have key 0
+            float a0p = 0.0f, rmax = 0.0f;
+            uint32_t x0 = 0;
+            for (int c = 0; c < n_rounds; ++c) {
+                const uint4 r = philox4x32_10(make_uint4((uint32_t)(lane + 32 * c), (uint32_t)k, noise.c2, noise.c3),
+                                              noise.key0, noise.key1);
+                if (c == 0) x0 = r.x;
+                const float *al = ad + 128 * c + lane;
+                float *rl = rj + 128 * c + lane;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float a = fmaxf(al[32 * q], 0.0f);
+                    a0p = __fadd_rn(a0p, a);
+                    const float key = a * inv_exp_of_word(word_of(r, q));
+                    rmax = fmaxf(rmax, key);
+                    rl[32 * q] = key;
+                }
+            }
+            const float a0 = warp_sum(a0p);
+            const float E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
+            rmax = warp_max_nonneg(rmax);
+            if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, rj);
+            __syncwarp();
+            const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
+            const bool k_tops = rj[wpos(jk)] * inv_rmax >= 1.0f - kTieMargin;
             const float tau = waiting_time(E0, a0);
             tau_k = tau;
-            const int4 rk = s_rx[jpos(jk, v.nb)];
+            const int4 rk = tab.rx[jpos(jk, nb)];
             // BIN: t_{k+1} ends this interval and starts the next, in the bin of gq
             if (kBin) mu -= bin_transition(xobs, xo, gq, p.n_obs);
             float dt_dir = 0.0f, dtau_dir = 0.0f;
@@ -804,7 +983,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
                             lam[sp] += alpha * g;
                             int dv = 0;
                             for (int e = rk.z; e < rk.w; ++e)
-                                if (stoich_species(s_st[e]) == sp) dv += stoich_delta(s_st[e]);
+                                if (stoich_species(tab.st[e]) == sp) dv += stoich_delta(tab.st[e]);
                             c += g * (float)dv;
                         }
                         const float c_tau = __fdividef(c, tau);
@@ -818,95 +997,92 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
             __syncwarp();
             const float dtau = mu + dtau_dir;
             const float dLda0 = -dtau * tau / a0;
-            // pass 2: weights and w_j over this lane's reactions
+            // pass 2: soft-sample weights q_j = (r_j / r_max)^(1/T) and w_j
             float Zp = 0.0f, Wp = 0.0f;
-            for (int pos = lane, q = q_first, b = b_first; pos < 4 * v.nb; pos += 32, next_slot(q, b)) {
-                {
-                    // predicated rather than branched (the lanes hold reactions with 1 to 4 stoichiometric
-                    // entries); the slots of j = -1 and j >= M hold no entries, and their weight is 0
-                    const int j = 4 * b + q - 1;
-                    const bool live = j >= 0 && j < M;
-                    const float l = live ? lj[pos] : -CUDART_INF_F;
-                    const float qv = l == -CUDART_INF_F ? 0.0f : exp2f((l - lmax) * invT);
-                    const int4 rx = s_rx[pos];
-                    float w = 0.0f;
-                    if (rx.w - rx.z <= 4) {
+            int near = 0;  // keys within the tie margin of the largest
+            auto at = [&](int e) { return *reinterpret_cast<const float *>(reinterpret_cast<const char *>(lam) + ent_offset(e)); };
+            auto weights = [&](auto many) {
+                for (int c = 0; c < n_rounds; ++c) {
+                    float *rl = rj + 128 * c + lane, *cl = ct + 128 * c + lane;
+                    const int4 *el = tab.ent + 128 * c + lane;
 #pragma unroll
-                        for (int t = 0; t < 4; ++t)
-                            if (rx.z + t < rx.w) {
-                                const int se = s_st[rx.z + t];
-                                w += (float)stoich_delta(se) * lam[stoich_species(se)];
-                            }
-                    } else {
-                        for (int e = rx.z; e < rx.w; ++e) w += (float)stoich_delta(s_st[e]) * lam[stoich_species(s_st[e])];
+                    for (int q = 0; q < 4; ++q) {
+                        const float rel = rl[32 * q] * inv_rmax;
+                        near += rel >= 1.0f - kTieMargin;
+                        const float qv = ex2_approx(lg2_approx(rel) * invT);
+                        const int4 en = el[32 * q];
+                        float w = ent_change(en.x) * at(en.x);
+                        w = __fmaf_rn(ent_change(en.y), at(en.y), w);
+                        w = __fmaf_rn(ent_change(en.z), at(en.z), w);
+                        w = __fmaf_rn(ent_change(en.w), at(en.w), w);
+                        if (decltype(many)::value && en.x == kEntMany) {
+                            const int4 rx = tab.rx[q * nb + 32 * c + lane];
+                            w = 0.0f;
+                            for (int e = rx.z; e < rx.w; ++e)
+                                w = __fmaf_rn((float)stoich_delta(tab.st[e]), lam[stoich_species(tab.st[e])], w);
+                        }
+                        rl[32 * q] = qv;
+                        cl[32 * q] = w;
+                        Zp += qv;
+                        const float qw = qv * w;
+                        Wp += qv > 0.0f ? qw : 0.0f;
                     }
-                    if (live) {
-                        lj[pos] = qv;
-                        ct[pos] = w;  // kept for pass 3, which overwrites the slot afterwards
-                    }
-                    Zp += qv;  // + 0 where qv = 0: the same bits
-                    Wp += qv > 0.0f ? qv * w : 0.0f;
                 }
-            }
+            };
+            if (tab.many) weights(std::true_type{});
+            else weights(std::false_type{});
+            // the recorded reaction won the race if its key is the only one at the top; near ties are raced again
+            if (__reduce_add_sync(0xffffffffu, near) == 1) mism += !k_tops;
+            else mism += warp_race_exact(n_rounds, ad, k, noise) != jk;
             const float Z = warp_sum(Zp), Wq = warp_sum(Wp);
-            const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ;
-            // pass 3: per-reaction adjoints and reactant-slot contributions to the state adjoint
-            for (int pos = lane, q = q_first, b = b_first; pos < 4 * v.nb; pos += 32, next_slot(q, b)) {
-                {
-                    const int j = 4 * b + q - 1;
-                    const bool live = j >= 0 && j < M;  // predicated: the other slots write zero contributions
-                    const int4 rx = s_rx[pos];
-                    const float qv = live ? lj[pos] : 0.0f, a = live ? aj[pos] : 0.0f;
-                    float psi = 0.0f;
-                    if (qv > 0.0f) psi = qv * invZ * (ct[pos] - Wbar) * invT;  // w_j from pass 2
-                    if (live) dA[pos] += psi + dLda0 * a;
-                    // d log a_j / dX and d a_j / dX of each reactant slot, formed with selects (the lanes hold
-                    // reactions of different orders): first order is the hetero form with x2 = 1
-                    const bool has1 = rx.x >= 0, has2 = rx.y >= 0, homo = has2 && rx.y == rx.x;
-                    const float c_tau = dLda0 * s_k[pos];
-                    const float x1 = int2f(X[has1 ? rx.x : 0]);
-                    const float xr2 = int2f(X[has2 ? rx.y : 0]);
-                    const float x2 = (has2 && !homo) ? xr2 : 1.0f;
-                    const float dh = x1 - 0.5f;
-                    const float num = homo ? psi * dh : psi;
-                    const float den = homo ? mass_action_h_sel(rx, X) : x1;
-                    const float t1 = a > 0.0f ? __fdividef(num, den) : 0.0f;
-                    const float c1 = has1 ? t1 + c_tau * (homo ? dh : x2) : 0.0f;
-                    const float c2 = (has2 && !homo) ? (a > 0.0f ? __fdividef(psi, xr2) : 0.0f) + c_tau * x1 : 0.0f;
-                    // the soft weight and w_j of this reaction are spent: its slots take the contributions
-                    lj[pos] = c1;  // reactant slot 0
-                    ct[pos] = c2;  // reactant slot 1
+            const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ, scale = invZ * invT;
+            // pass 3: g_j = psi_j + dL/da0 a_j
+            for (int c = 0; c < n_rounds; ++c) {
+                const int at0 = 128 * c + lane;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float qv = rj[at0 + 32 * q];
+                    float psi = qv * scale * (ct[at0 + 32 * q] - Wbar);
+                    psi = qv > 0.0f ? psi : 0.0f;
+                    const float g = __fmaf_rn(dLda0, fmaxf(ad[at0 + 32 * q], 0.0f), psi);
+                    dA[at0 + 32 * q] += g;
+                    rj[at0 + 32 * q] = g;
                 }
             }
             __syncwarp();
-            // lambda_s += sum of the reactant-slot contributions of species s. With N <= 32 each species
-            // gets g = 32 / 2^ceil(log2 N) lanes that stride over its incidence list with four
-            // accumulators and combine by a butterfly inside the group; with more species each lane takes
-            // whole species. The order is fixed, so the result is the same on every run.
-            int pow2 = 1;
-            while (pow2 < N && pow2 < 32) pow2 <<= 1;
-            const int gsz = N <= 32 ? 32 / pow2 : 1;
-            for (int base = 0; base < N; base += 32 / gsz) {
-                const int sp = base + lane / gsz, r = lane % gsz;
-                float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, c3 = 0.0f;
+            // the state adjoint, in a fixed order
+            for (int sp0 = 0; sp0 < N; sp0 += g_step) {
+                const int sp = sp0 + g_first;
+                float acc = 0.0f;
                 if (sp < N) {
-                    const int e1 = s_inc_ptr[sp + 1];
-                    int e = s_inc_ptr[sp] + r;
-                    auto slot_val = [&](int ee) {
-                        const int slot = s_inc[ee];  // 2 j + reactant slot
-                        return ((slot & 1) ? ct : lj)[jpos(slot >> 1, v.nb)];
-                    };
-                    for (; e + 3 * gsz < e1; e += 4 * gsz) {
-                        c0 += slot_val(e);
-                        c1 += slot_val(e + gsz);
-                        c2 += slot_val(e + 2 * gsz);
-                        c3 += slot_val(e + 3 * gsz);
+                    const int4 c = tab.inc[sp];
+                    const int x = X[sp];
+                    const float xf = int2f(x);
+                    // plain reactants: g_j / X, or D_j dL/da0 where the species is absent (a_j = 0 on its whole list)
+                    const float *src = x > 0 ? rj : ad;
+                    float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, c3 = 0.0f;
+                    int e = c.x + g_lane;
+                    for (; e + 3 * gsz < c.y; e += 4 * gsz) {
+                        c0 += src[tab.list[e] & 0xffff];
+                        c1 += src[tab.list[e + gsz] & 0xffff];
+                        c2 += src[tab.list[e + 2 * gsz] & 0xffff];
+                        c3 += src[tab.list[e + 3 * gsz] & 0xffff];
                     }
-                    for (; e < e1; e += gsz) c0 += slot_val(e);
+                    for (; e < c.y; e += gsz) c0 += src[tab.list[e] & 0xffff];
+                    acc = (c0 + c1) + (c2 + c3);
+                    acc = x > 0 ? __fdividef(acc, xf) : -dLda0 * acc;
+                    if (c.y < c.z) {  // homodimers: d log h/dX = (2 X - 1)/(X (X - 1)), dh/dX = X - 1/2 below X = 2
+                        float ch = 0.0f;
+                        for (int eh = c.y + g_lane; eh < c.z; eh += gsz) {
+                            const int le = tab.list[eh];
+                            ch += x >= 2 ? rj[le & 0xffff] : tab.k[le >> 16];
+                        }
+                        acc += x >= 2 ? __fdividef(ch * (xf - 0.5f), __fmul_rn(xf, xf - 1.0f) * 0.5f)
+                                      : dLda0 * (xf - 0.5f) * ch;
+                    }
                 }
-                float acc = (c0 + c1) + (c2 + c3);
                 for (int off = gsz >> 1; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-                if (r == 0 && sp < N) lam[sp] += acc;
+                if (g_lane == 0 && sp < N) lam[sp] += acc;
             }
             mu += dt_dir;
         }
@@ -939,11 +1115,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const int4 *s_
         }
         --ck_off;
         __syncwarp();
-        if (k > 0) {
-            const int4 rp = s_rx[jpos(event_at(k - 1), v.nb)];
-            for (int e = rp.z + lane; e < rp.w; e += 32) X[stoich_species(s_st[e])] -= stoich_delta(s_st[e]);
-        }
-        __syncwarp();
+        if (k > 0) warp_apply<true>(tab, event_at(k - 1), -1, X, ad);
     }
     if (lane == 0 && mism) atomicAdd(p.mismatch, mism);
 }
