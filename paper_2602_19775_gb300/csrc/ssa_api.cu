@@ -303,13 +303,13 @@ extern "C" ssa_status ssa_create_network(int32_t n_species, int32_t n_reactions,
     }
     for (int sp = n_species + 1; sp < upd_ptr_pad; ++sp) upd[sp] = upd[n_species];
     upd.resize((upd.size() + 3) / 4 * 4, 0);
-    // the warp kernels' second table region (WarpTab): the entries of v_j by wide position, and per species the
+    // the warp kernels' second table region (WarpTab): the entries of v_j, and per species the
     // reactions it reacts in, homodimers last. Networks past these sizes are refused by those kernels (shared
     // memory).
     const bool has_wtab = n_species <= kEntMaxSpecies && n_reactions <= kEntMaxReactions;
     const int wtab_ent = 4 * wide_len(n_reactions);
     std::vector<int> wtab(has_wtab ? wtab_ent + 4 * (n_species + 1) : 0, 0);
-    auto list_entry = [&](int j) { return jpos(j, nb_warp) << 16 | wpos(j); };
+    auto list_entry = [&](int j) { return jpos(j, nb_warp) << 16 | (j + 1); };
     if (has_wtab) {
         std::fill(wtab.begin(), wtab.begin() + wtab_ent, (int)((uint32_t)n_species << 18));
         for (int j = 0; j < n_reactions; ++j) {

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
             }
             float *slot = p.partial + b.slot_off + (int64_t)u.slot * p.M;
             const int nb = (p.M + 4) >> 2;
-            for (int j = lane; j < p.M; j += 32) slot[j] = dA[SOFT ? jpos(j, nb) : wpos(j)];
+            for (int j = lane; j < p.M; j += 32) slot[j] = dA[SOFT ? jpos(j, nb) : j + 1];
         }
         __syncwarp();
     }

@@ -22,16 +22,16 @@ struct NetTables {
     uint32_t tab_bytes;  // 16 * M + 4 * nnz_pad, a multiple of 16
 };
 
-// What a warp-per-trajectory kernel reads of the network, in shared or global memory. Its per-reaction values live
-// at wide positions (wpos): round c, word q and lane l of reaction j's word at 128 c + 32 q + l, so that a lane's
-// addresses differ by constants and the lanes of an access lie side by side.
+// What a warp-per-trajectory kernel reads of the network, in shared or global memory. Its per-reaction values lie by
+// the word that drives them (index j + 1; index 0 is the waiting time's): a lane's block of four is one 16-byte
+// access, and the lanes' blocks lie side by side.
 //   rx, k     reactants and rates, lane-major (jpos)
-//   ent[w]    by wide position, up to four entries (species, change) of v_j, each (4 species << 16) | bf16 bits of
-//             the change; an absent entry is species N with change 0, whose list in inc is empty and whose lambda
+//   ent[w]    at w = wpos(j), up to four entries (species, change) of v_j, each (4 species << 16) | bf16 bits of the
+//             change; an absent entry is species N with change 0, whose list in inc is empty and whose lambda
 //             slot holds 0; a reaction with more entries is marked by ent[w].x = kEntMany and read from
 //             st[rx.z .. rx.w)
 //   inc[s]    {begin, first homodimer, end} of species s in list: the reactions it reacts in, each
-//             (jpos << 16) | wpos; inc[N].w: whether any reaction is marked
+//             (jpos << 16) | (j + 1); inc[N].w: whether any reaction is marked
 struct WarpTab {
     const int4 *rx;
     const int *st;
@@ -59,12 +59,14 @@ struct WarpNoise {
 // side, so those shared-memory accesses are free of bank conflicts.
 __host__ __device__ __forceinline__ int jpos(int j, int nb) { return ((j + 1) & 3) * nb + ((j + 1) >> 2); }
 
+// Round c, word q and lane l of reaction j's word, at 128 c + 32 q + l: 16-byte entries read by the lanes of one word
+// are free of bank conflicts.
 __host__ __device__ __forceinline__ int wpos(int j)
 {
     const int b = (j + 1) >> 2;
     return ((b >> 5) << 7) + (((j + 1) & 3) << 5) + (b & 31);
 }
-// length of an array by wide position
+// length of an array by word or by wpos, whole rounds of 32 blocks
 __host__ __device__ __forceinline__ int wide_len(int M) { return ((((M + 4) >> 2) + 31) >> 5) << 7; }
 
 // Warp reductions shared by the warp-per-trajectory kernels (butterfly: every lane gets the same

@@ -12,15 +12,14 @@
 //     exact race (a butterfly argmax of (a_j, E_j, j) with a_i E_b > a_b E_i and ties to the lowest j);
 //   - the clock, the sample writes and the state update are warp-uniform (lanes share the stoichiometry
 //     and observable loops).
-// Per-reaction values lie at wide positions (wpos in ssa_internal.cuh): the lanes' accesses are free of
-// shared-memory bank conflicts and a lane's addresses differ by constants.
+// Per-reaction values lie by the word that drives them: a lane reads and writes its block of four at once.
 // The adjoint keeps per-reaction values in per-warp shared memory and accumulates the state adjoint
 // through a species -> reactions table in a fixed order (no atomics, deterministic).
 // Bound: instruction issue (ncu, 11 species and 301 reactions, 2,500 trajectories: ~63% issue active at four to five
 // warps per scheduler, the rest fixed-latency dependences of a step). Instructions per step: forward 1,340 -> 725
 // (the logarithms of the race and the propensities of untouched reactions are gone), adjoint 4,430 -> 1,756 (the same,
 // one division per species instead of two per reaction, keys without logarithms of E). One gradient step of those
-// trajectories to t = 2: 30.1 -> 14.5 ms.
+// trajectories to t = 2: 30.1 -> 13.8 ms.
 #include <cstdint>
 
 #include "ssa_warp_body.cuh"
@@ -171,7 +170,7 @@ __global__ void __launch_bounds__(128, kWarpAdjBlocks) adj_warp_kernel(const Adj
     // fixed-order reduction over the block's warps
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
         float acc = 0.0f;
-        for (int w = 0; w < W; ++w) acc += base0[w * per_warp + 2 * Npad + 3 * Mw + wpos(j)];
+        for (int w = 0; w < W; ++w) acc += base0[w * per_warp + 2 * Npad + 3 * Mw + j + 1];
         p.partial[(int64_t)blockIdx.x * M + j] = acc;
     }
 }

@@ -57,7 +57,7 @@ __device__ __forceinline__ void warp_propensities_all(const WarpTab &t, const in
     for (int c = 0; c < t.rounds; ++c)
         for (int q = 0; q < 4; ++q) {
             const int b = 32 * c + lane;
-            a[128 * c + 32 * q + lane] = b < t.nb ? warp_propensity<SIGNED>(t, q * t.nb + b, X) : 0.0f;
+            a[4 * b + q] = b < t.nb ? warp_propensity<SIGNED>(t, q * t.nb + b, X) : 0.0f;
         }
     __syncwarp();
 }
@@ -154,7 +154,7 @@ static __device__ __noinline__ int warp_race_exact(int rounds, const float *a, i
         const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            race(fmaxf(a[128 * c + 32 * q + lane], 0.0f), neg_log_unit(u01(word_of(r, q))), 4 * b + q - 1, ab, Eb, jb);
+            race(fmaxf(a[4 * b + q], 0.0f), neg_log_unit(u01(word_of(r, q))), 4 * b + q - 1, ab, Eb, jb);
     }
     warp_race_combine(ab, Eb, jb);
     return jb;
@@ -180,13 +180,13 @@ __device__ __forceinline__ void warp_step_eval(int n_rounds, int k, const WarpNo
         if (t0 == 0) x0 = r[0].x;
 #pragma unroll
         for (int t = 0; t < C; ++t) {
+            // the waiting-time word's slot (j = -1) and the padded ones have rate 0: they add 0 to a0 and never win
+            const float4 av = reinterpret_cast<const float4 *>(a)[lane + 32 * (t0 + t)];
+            const float aq[4] = {av.x, av.y, av.z, av.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                // the waiting-time word's slot (j = -1) and the padded ones have rate 0: they add 0 to a0 and
-                // never win
-                const float aq = a[128 * (t0 + t) + 32 * q + lane];
-                a0p = __fadd_rn(a0p, aq);
-                warp_top_add(top, aq, word_of(r[t], q), 4 * (t0 + t) + q);
+                a0p = __fadd_rn(a0p, aq[q]);
+                warp_top_add(top, aq[q], word_of(r[t], q), 4 * (t0 + t) + q);
             }
         }
     };
@@ -200,7 +200,7 @@ __device__ __forceinline__ void warp_step_eval(int n_rounds, int k, const WarpNo
     a0 = warp_sum(a0p);
     E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
     int src, slot;
-    const bool sure = warp_top_decide(top, a0, [&](int s) { return a[min(s, 4 * n_rounds - 1) * 32 + lane]; }, src, slot);
+    const bool sure = warp_top_decide(top, a0, [&](int s) { return a[4 * (lane + 32 * min(s >> 2, n_rounds - 1)) + (s & 3)]; }, src, slot);
     if (sure && n_rounds <= 16) jb = 4 * (src + 32 * (slot >> 2)) + (slot & 3) - 1;
     else jb = warp_race_exact(n_rounds, a, k, z);
 }
@@ -840,7 +840,7 @@ static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *a
         const uint4 r = philox4x32_10(make_uint4((uint32_t)(32 * c + lane), (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int w = 128 * c + 32 * q + lane;
+            const int w = 4 * (32 * c + lane) + q;
             const float key = (fmaxf(ad[w], 0.0f) * sc) * inv_exp_of_word(word_of(r, q));
             rmax = fmaxf(rmax, key);
             rj[w] = key;
@@ -942,20 +942,23 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             // slot and the padded ones have rate 0: they add 0 and have key 0
             float a0p = 0.0f, rmax = 0.0f;
             uint32_t x0 = 0;
+            float4 *ad4 = reinterpret_cast<float4 *>(ad), *rj4 = reinterpret_cast<float4 *>(rj),
+                   *ct4 = reinterpret_cast<float4 *>(ct), *dA4 = reinterpret_cast<float4 *>(dA);
             for (int c = 0; c < n_rounds; ++c) {
                 const uint4 r = philox4x32_10(make_uint4((uint32_t)(lane + 32 * c), (uint32_t)k, noise.c2, noise.c3),
                                               noise.key0, noise.key1);
                 if (c == 0) x0 = r.x;
-                const float *al = ad + 128 * c + lane;
-                float *rl = rj + 128 * c + lane;
+                const float4 av = ad4[32 * c + lane];
+                const float aq[4] = {av.x, av.y, av.z, av.w};
+                float key[4];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    const float a = fmaxf(al[32 * q], 0.0f);
+                    const float a = fmaxf(aq[q], 0.0f);
                     a0p = __fadd_rn(a0p, a);
-                    const float key = a * inv_exp_of_word(word_of(r, q));
-                    rmax = fmaxf(rmax, key);
-                    rl[32 * q] = key;
+                    key[q] = a * inv_exp_of_word(word_of(r, q));
+                    rmax = fmaxf(rmax, key[q]);
                 }
+                rj4[32 * c + lane] = make_float4(key[0], key[1], key[2], key[3]);
             }
             const float a0 = warp_sum(a0p);
             const float E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
@@ -963,7 +966,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, rj);
             __syncwarp();
             const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
-            const bool k_tops = rj[wpos(jk)] * inv_rmax >= 1.0f - kTieMargin;
+            const bool k_tops = rj[jk + 1] * inv_rmax >= 1.0f - kTieMargin;
             const float tau = waiting_time(E0, a0);
             tau_k = tau;
             const int4 rk = tab.rx[jpos(jk, nb)];
@@ -1003,13 +1006,14 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             auto at = [&](int e) { return *reinterpret_cast<const float *>(reinterpret_cast<const char *>(lam) + ent_offset(e)); };
             auto weights = [&](auto many) {
                 for (int c = 0; c < n_rounds; ++c) {
-                    float *rl = rj + 128 * c + lane, *cl = ct + 128 * c + lane;
+                    const float4 rv = rj4[32 * c + lane];
+                    float qv[4] = {rv.x, rv.y, rv.z, rv.w}, wv[4];
                     const int4 *el = tab.ent + 128 * c + lane;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const float rel = rl[32 * q] * inv_rmax;
+                        const float rel = qv[q] * inv_rmax;
                         near += rel >= 1.0f - kTieMargin;
-                        const float qv = ex2_approx(lg2_approx(rel) * invT);
+                        qv[q] = ex2_approx(lg2_approx(rel) * invT);
                         const int4 en = el[32 * q];
                         float w = ent_change(en.x) * at(en.x);
                         w = __fmaf_rn(ent_change(en.y), at(en.y), w);
@@ -1021,12 +1025,13 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
                             for (int e = rx.z; e < rx.w; ++e)
                                 w = __fmaf_rn((float)stoich_delta(tab.st[e]), lam[stoich_species(tab.st[e])], w);
                         }
-                        rl[32 * q] = qv;
-                        cl[32 * q] = w;
-                        Zp += qv;
-                        const float qw = qv * w;
-                        Wp += qv > 0.0f ? qw : 0.0f;
+                        wv[q] = w;
+                        Zp += qv[q];
+                        const float qw = qv[q] * w;
+                        Wp += qv[q] > 0.0f ? qw : 0.0f;
                     }
+                    rj4[32 * c + lane] = make_float4(qv[0], qv[1], qv[2], qv[3]);
+                    ct4[32 * c + lane] = make_float4(wv[0], wv[1], wv[2], wv[3]);
                 }
             };
             if (tab.many) weights(std::true_type{});
@@ -1038,16 +1043,20 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ, scale = invZ * invT;
             // pass 3: g_j = psi_j + dL/da0 a_j
             for (int c = 0; c < n_rounds; ++c) {
-                const int at0 = 128 * c + lane;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const float qv = rj[at0 + 32 * q];
-                    float psi = qv * scale * (ct[at0 + 32 * q] - Wbar);
+                const int b = 32 * c + lane;
+                const float4 qf = rj4[b], wf = ct4[b], af = ad4[b];
+                float4 df = dA4[b];
+                auto adjoint = [&](float qv, float w, float a, float &sum) {
+                    float psi = qv * scale * (w - Wbar);
                     psi = qv > 0.0f ? psi : 0.0f;
-                    const float g = __fmaf_rn(dLda0, fmaxf(ad[at0 + 32 * q], 0.0f), psi);
-                    dA[at0 + 32 * q] += g;
-                    rj[at0 + 32 * q] = g;
-                }
+                    const float g = __fmaf_rn(dLda0, fmaxf(a, 0.0f), psi);
+                    sum += g;
+                    return g;
+                };
+                const float4 gf = make_float4(adjoint(qf.x, wf.x, af.x, df.x), adjoint(qf.y, wf.y, af.y, df.y),
+                                              adjoint(qf.z, wf.z, af.z, df.z), adjoint(qf.w, wf.w, af.w, df.w));
+                dA4[b] = df;
+                rj4[b] = gf;
             }
             __syncwarp();
             // the state adjoint, in a fixed order
