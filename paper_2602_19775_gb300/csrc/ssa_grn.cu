@@ -29,6 +29,7 @@
 
 #include "ssa_host.h"
 #include "ssa_tc.cuh"
+#include "ssa_warp_body.cuh"
 
 namespace ssa {
 
@@ -41,8 +42,8 @@ cudaError_t launch_column_sums(const float *x, int64_t n_rows, int64_t row_len, 
 
 constexpr int kGrnLimbs = 8;       // 6-bit limbs of W1 on one grid: 48 bits of dynamic range
 constexpr int kGrnLimbBits = 6;
-constexpr int kGrnOutBatch = 12;   // output counts up to this take the adjoint's batched W2 column loads
-constexpr int kGrnWarps = 4;
+constexpr int kGrnWarps = 4;       // warps per block, fewer for networks whose arrays leave no room (grn_warps)
+constexpr int kGrnRegSpecies = 288;  // dynamic species up to this: the adjoint's per-species sums stay in registers
 
 struct GrnParams {
     int n_in, n_hid, n_out, n_dyn, M, Mp, nb;
@@ -52,6 +53,7 @@ struct GrnParams {
     const float *E1;      // [n_img][n_hid]
     const int *W2fix;     // [n_out][n_hid]: W2 = W2fix * 2^g2
     const float *W2f;     // [n_out][n_hid]
+    const float4 *W2t;    // [n_dyn][ceil(n_out / 4)]: the columns of W2, padded with zeros; rows of zeros for the outputs
     const float *b2;      // [n_out]
     const float *dvec;    // [n_dyn]: d = exp(log_d)
     const int *grid;      // [0] = g2
@@ -98,16 +100,6 @@ __device__ __forceinline__ float e2_value(long long acc, float scale, float b2)
     return __fadd_rn(b2, __fmul_rn(__ll2float_rn(acc), scale));
 }
 
-// propensity of reaction j (one lane's view); padded j >= M give 0
-__device__ __forceinline__ float grn_prop(const GrnParams &p, int j, const float *aH, const float *aO, const int *X,
-                                          const float *s_d)
-{
-    if (j < p.n_hid) return aH[j];
-    if (j < p.n_dyn) return aO[j - p.n_hid];
-    if (j < p.M) return __fmul_rn(s_d[j - p.n_dyn], int2f(X[j - p.n_dyn]));
-    return 0.0f;
-}
-
 }  // namespace
 
 // ---------------------------------------------------------------------------------------------
@@ -138,7 +130,7 @@ __device__ __forceinline__ uint16_t float_to_bf16_rn(float f)
 
 __global__ void grn_prepare_kernel(const uint16_t *W1, const uint16_t *W2, const int32_t *x_img, const float *log_d,
                                    int n_in, int n_hid, int n_out, int64_t n_img, int n_in_pad, uint16_t *W1L,
-                                   int *W2fix, float *W2f, uint16_t *xb, float *dvec, int *grid)
+                                   int *W2fix, float *W2f, float *W2t, uint16_t *xb, float *dvec, int *grid)
 {
     // W1 on the grid 2^g1, g1 = (max exponent + 1) - 48: |W1| = n 2^g1, n < 2^48, limbs of 6 bits
     const int g1 = (grid[0] - 127 + 1) - kGrnLimbBits * kGrnLimbs;
@@ -170,6 +162,7 @@ __global__ void grn_prepare_kernel(const uint16_t *W1, const uint16_t *W2, const
         if (q < (int64_t)n_out * n_hid) {
             const float w = bf16_to_float(W2[q]);
             W2f[q] = w;
+            W2t[(q % n_hid) * ((n_out + 3) & ~3) + q / n_hid] = w;  // the padding was cleared before
             const double nd = (double)w * exp2(-(double)g2);
             if (fabs(nd) >= 1073741824.0 || (double)(long long)nd != nd) atomicOr(&grid[2], 2);
             W2fix[q] = (int)fmax(-1073741823.0, fmin(1073741823.0, nd));
@@ -196,7 +189,10 @@ __global__ void grn_prepare_kernel(const uint16_t *W1, const uint16_t *W2, const
 // ---------------------------------------------------------------------------------------------
 // forward: one warp per trajectory
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) grn_fwd_kernel(const GrnParams p, int record)
+// The warp-per-trajectory forward's step (ssa_warp_body.cuh) over propensities kept by word: those of the hidden
+// productions are constant, an event changes one degradation and, for a hidden gene, the output productions. Bound
+// by instruction issue: 1,620 -> 796 warp instructions per step at 784-256-10.
+__global__ void __launch_bounds__(128, 6) grn_fwd_kernel(const GrnParams p, int record)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
@@ -204,16 +200,15 @@ __global__ void __launch_bounds__(128) grn_fwd_kernel(const GrnParams p, int rec
     int *s_W2fix = reinterpret_cast<int *>(smem);
     float *s_d = reinterpret_cast<float *>(s_W2fix + no * nh);
     float *s_b2 = s_d + nd;
-    const int ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3;
+    const int ndp = (nd + 3) & ~3, wide = wide_len(p.M), rounds = wide >> 7;
     const int nop = (no + 3) & ~3;
-    const size_t per_warp = (size_t)ndp + nhp + 3 * (size_t)nop;  // X, aH, E2acc (2 words each), aO
+    const size_t per_warp = (size_t)ndp + wide + 2 * (size_t)nop;  // X, a, E2acc (2 words each)
     // offsets from the shared array itself (not through an integer round trip), so that every access below
     // compiles to a shared-memory load or store with 32-bit addressing
     unsigned char *wb = smem + ((4 * ((size_t)no * nh + nd + ((no + 3) & ~3)) + 15) & ~(size_t)15);
     int *X = reinterpret_cast<int *>(wb) + wib * per_warp;
-    float *aH = reinterpret_cast<float *>(X + ndp);
-    long long *E2acc = reinterpret_cast<long long *>(aH + nhp);
-    float *aO = reinterpret_cast<float *>(E2acc + no);
+    float *a = reinterpret_cast<float *>(X + ndp);
+    long long *E2acc = reinterpret_cast<long long *>(a + wide);
 
     for (int q = threadIdx.x; q < no * nh; q += blockDim.x) s_W2fix[q] = p.W2fix[q];
     for (int q = threadIdx.x; q < nd; q += blockDim.x) s_d[q] = p.dvec[q];
@@ -226,15 +221,17 @@ __global__ void __launch_bounds__(128) grn_fwd_kernel(const GrnParams p, int rec
     const float scale = exp2f((float)p.grid[0]);
     const float *E1 = p.E1 + (i / p.tpi) * nh;
     for (int s = lane; s < nd; s += 32) X[s] = 0;
-    for (int h = lane; h < nh; h += 32) aH[h] = p.k_max * sigmoid_f(E1[h]);
+    for (int q = lane; q < wide; q += 32) a[q] = 0.0f;  // every gene starts at zero: no degradation
+    __syncwarp();
+    for (int h = lane; h < nh; h += 32) a[h + 1] = p.k_max * sigmoid_f(E1[h]);
     for (int o = lane; o < no; o += 32) {
         E2acc[o] = 0;
-        aO[o] = p.k_max * sigmoid_f(s_b2[o]);
+        a[nh + o + 1] = p.k_max * sigmoid_f(s_b2[o]);
     }
     __syncwarp();
     const bool bad_input = (*p.flag & kErrBadSamples) != 0;
     const uint64_t gid = p.traj_offset + (uint64_t)i;
-    const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32), key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
+    const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
 
     double t = 0.0;
     int s = 0;
@@ -244,25 +241,9 @@ __global__ void __launch_bounds__(128) grn_fwd_kernel(const GrnParams p, int rec
     uint32_t e0 = 0, e1 = 0, e2 = 0, e3 = 0;
     while (!bad_input) {
         if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
-        float a0p = 0.0f, ab = 0.0f, Eb = 1.0f, E0 = 0.0f;
-        int jb = -1;
-        for (int b = lane; b < p.nb; b += 32) {
-            const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, c2, c3), key0, key1);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                // predicated: every word's variate is formed (the warp forms it whenever one lane needs it), word
-                // 0 of lane 0's first block is E0, and j = -1 takes part with rate 0 (adds 0, never wins)
-                const int j = 4 * b + q - 1;
-                const float E = neg_log_unit(u01(word_of(r, q)));
-                if (q == 0 && j < 0) E0 = E;
-                const float a = j < 0 ? 0.0f : grn_prop(p, max(j, 0), aH, aO, X, s_d);
-                a0p = __fadd_rn(a0p, a);
-                race(a, E, j, ab, Eb, jb);
-            }
-        }
-        const float a0 = warp_sum(a0p);
-        warp_race_combine(ab, Eb, jb);
-        E0 = __shfl_sync(0xffffffffu, E0, 0);
+        float a0, E0;
+        int jb;
+        warp_step_eval(rounds, k, noise, a, a0, E0, jb);
         if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
         if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
         if (jb < 0) { status = SSA_TRAJ_BAD_RATE; break; }
@@ -293,11 +274,15 @@ __global__ void __launch_bounds__(128) grn_fwd_kernel(const GrnParams p, int rec
             if (cross) break;
         }
         __syncwarp();
-        if (lane == 0) X[sp] += delta;
+        if (lane == 0) {
+            const int x = X[sp] + delta;
+            X[sp] = x;
+            a[nd + sp + 1] = __fmul_rn(s_d[sp], int2f(x));
+        }
         if (sp < nh) {
             for (int o = lane; o < no; o += 32) {
                 E2acc[o] += (long long)delta * s_W2fix[o * nh + sp];
-                aO[o] = p.k_max * sigmoid_f(e2_value(E2acc[o], scale, s_b2[o]));
+                a[nh + o + 1] = p.k_max * sigmoid_f(e2_value(E2acc[o], scale, s_b2[o]));
             }
         }
         __syncwarp();
@@ -679,42 +664,56 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
 // ---------------------------------------------------------------------------------------------
 // backward: one warp per trajectory, reverse walk
 // ---------------------------------------------------------------------------------------------
-#ifndef SSA_GRN_ADJ_BLOCKS
-#define SSA_GRN_ADJ_BLOCKS 6  // resident blocks per SM the adjoint is compiled for (36 KB of shared memory each)
-#endif
-__global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const GrnParams p)
+// words of one warp's arrays in the adjoint (grn_adj_kernel)
+__host__ __device__ inline size_t grn_adj_words(int nh, int no, bool shared_sums)
+{
+    const int nd = nh + no, ndp = (nd + 3) & ~3, nop = (no + 3) & ~3;
+    return 2 * (size_t)wide_len(2 * nd) + 2 * ndp + 6 * (size_t)nop + (shared_sums ? 3 * (size_t)ndp : 0);
+}
+
+// Per step: pass 1, by Philox block, forms the race's keys a_j / E_j from the kept propensities; pass 2, by species
+// (a lane's species s = lane, lane + 32, ... with their productions and degradations), the soft weights and their
+// moment with lambda; pass 3, by species again, psi of both reactions and the state adjoint. With NS rounds of
+// species (n_dyn <= 32 NS) lambda, dL/dE1 and dL/dlog d live in registers; NS = 0 keeps them in shared memory.
+// Bound by instruction issue; 784-256-10: 4,280 -> 1,610 warp instructions per step, a training step of 48 x 64
+// trajectories 127 -> 63 ms with the forward. Four resident blocks (128 registers): 63 ms; five 75, six 70 (spills),
+// six with the sums in shared memory 77.
+constexpr int kGrnAdjBlocks = 4;
+// NF: the first rounds of species that are full (n_dyn >= 32 NF).
+template <int NS, int NF>
+__global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
-    const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn, Mp = p.Mp;
+    const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn;
     float *s_d = reinterpret_cast<float *>(smem);
     float *s_b2 = s_d + nd;
-    const int ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3, nop = (no + 3) & ~3;
-    // per warp (words): X, lam, ctd [ndp each], aH, G1 [nhp each], E2acc [2 nop], aO, G2, R, db2 [nop each],
-    // lj [Mp], dlogd [ndp]. dL/dW2 goes to the trajectory's own row of p.dW2t (global, L2-resident while the
-    // warp works on it), which keeps the per-warp shared memory independent of n_out x n_hid.
-    const size_t per_warp = 4 * (size_t)ndp + 2 * (size_t)nhp + 6 * (size_t)nop + (size_t)Mp;
+    const int ndp = (nd + 3) & ~3, nop = (no + 3) & ~3, wide = wide_len(p.M), rounds = wide >> 7;
+    const int ns = NS > 0 ? NS : (nd + 31) >> 5;  // rounds of species
+    // per warp (words): a, key [wide each], X [ndp], 1 - sigma(E1), 0 for the outputs
+    // [ndp], E2acc [2 nop], 1 - sigma(E2), G2, R, db2
+    // [nop each]; NS = 0 also lam, G1, dlogd [ndp]. dL/dW2 goes to the trajectory's own row of p.dW2t
+    // (global, L2-resident while the warp works on it).
+    const size_t per_warp = grn_adj_words(nh, no, NS == 0);
     unsigned char *wb = smem + ((4 * ((size_t)nd + nop) + 15) & ~(size_t)15);  // shared-space offsets (see the forward)
     float *wbase = reinterpret_cast<float *>(wb) + wib * per_warp;
-    int *X = reinterpret_cast<int *>(wbase);
-    float *lam = wbase + ndp;
-    float *ctd = lam + ndp;
-    float *aH = ctd + ndp;
-    float *G1 = aH + nhp;
-    long long *E2acc = reinterpret_cast<long long *>(G1 + nhp);
-    float *aO = reinterpret_cast<float *>(E2acc + nop);
-    float *G2 = aO + nop;
+    float *a = wbase;
+    float *key = a + wide;
+    int *X = reinterpret_cast<int *>(key + wide);
+    float *cH = reinterpret_cast<float *>(X + ndp);
+    long long *E2acc = reinterpret_cast<long long *>(cH + ndp);
+    float *cO = reinterpret_cast<float *>(E2acc + nop);
+    float *G2 = cO + nop;
     float *R = G2 + nop;
     float *db2 = R + nop;
-    float *lj = db2 + nop;
-    float *dlogd = lj + Mp;
+    float *lam_s = db2 + nop, *G1_s = lam_s + ndp, *dlogd_s = G1_s + ndp;
     const int *__restrict__ W2fix = p.W2fix;
-    const float *__restrict__ W2f = p.W2f;
+    const float4 *__restrict__ W2t = p.W2t;
 
     for (int q = threadIdx.x; q < nd; q += blockDim.x) s_d[q] = p.dvec[q];
     for (int q = threadIdx.x; q < no; q += blockDim.x) s_b2[q] = p.b2[q];
-    for (int q = lane; q < nd; q += 32) dlogd[q] = 0.0f;
-    for (int q = lane; q < no; q += 32) db2[q] = 0.0f;
+    for (int q = lane; q < wide; q += 32) key[q] = 0.0f;
+    for (int q = lane; q < nop; q += 32) db2[q] = G2[q] = 0.0f;
     __syncthreads();
 
     const int64_t n = p.n_traj;
@@ -725,40 +724,68 @@ __global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const 
     float *dW2 = p.dW2t + (i < n ? i : 0) * (int64_t)no * nh;
     if (i < n)
         for (int q = lane; q < no * nh; q += 32) dW2[q] = 0.0f;
+    float lam_r[NS > 0 ? NS : 1], G1_r[NS > 0 ? NS : 1], dlogd_r[NS > 0 ? NS : 1];
+    auto lam = [&](int c) -> float & { return NS > 0 ? lam_r[NS > 0 ? c : 0] : lam_s[32 * c + lane]; };
+    auto G1 = [&](int c) -> float & { return NS > 0 ? G1_r[NS > 0 ? c : 0] : G1_s[32 * c + lane]; };
+    auto dlogd = [&](int c) -> float & { return NS > 0 ? dlogd_r[NS > 0 ? c : 0] : dlogd_s[32 * c + lane]; };
+    auto each_species = [&](auto body) {  // body(c, s) for this lane's species s = 32 c + lane below n_dyn
+#pragma unroll (NS > 0 ? NS : 1)
+        for (int c = 0; c < ns; ++c) {
+            const int s = 32 * c + lane;
+            if (c < NF) body(c, s);
+            else if (s < nd) body(c, s);
+        }
+    };
     if (active) {
         const float scale = exp2f((float)p.grid[0]);
         const float inv_kmax = 1.0f / p.k_max;
         const float *E1 = p.E1 + (i / p.tpi) * nh;
         const int d = p.draws[i];
         const int L = (st == SSA_TRAJ_OK) ? d - 1 : d;
-        for (int s = lane; s < nd; s += 32) {
-            X[s] = p.xfinal[(int64_t)s * n + i];
-            lam[s] = 0.0f;
-        }
-        for (int h = lane; h < nh; h += 32) {
-            aH[h] = p.k_max * sigmoid_f(E1[h]);
-            G1[h] = 0.0f;
-        }
+        for (int q = lane; q < wide; q += 32) a[q] = 0.0f;
+        __syncwarp();
+        each_species([&](int c, int s) {
+            const int x = p.xfinal[(int64_t)s * n + i];
+            X[s] = x;
+            a[nd + s + 1] = __fmul_rn(s_d[s], int2f(x));
+            lam(c) = 0.0f;
+            dlogd(c) = 0.0f;
+            G1(c) = 0.0f;
+            cH[s] = 0.0f;  // the outputs take no part in dL/dE1
+            if (s < nh) {
+                const float ah = p.k_max * sigmoid_f(E1[s]);
+                a[s + 1] = ah;
+                cH[s] = 1.0f - ah * inv_kmax;  // d log(k_max sigma(E)) / dE = 1 - sigma(E)
+            }
+        });
         __syncwarp();
         // E2 at the final state, exactly (integer fixed point)
+        auto set_output = [&](int o) {
+            const float ao = p.k_max * sigmoid_f(e2_value(E2acc[o], scale, s_b2[o]));
+            a[nh + o + 1] = ao;
+            cO[o] = 1.0f - ao * inv_kmax;
+        };
         for (int o = lane; o < no; o += 32) {
             long long acc = 0;
             for (int h = 0; h < nh; ++h) acc += (long long)__ldg(W2fix + o * nh + h) * X[h];
             E2acc[o] = acc;
-            aO[o] = p.k_max * sigmoid_f(e2_value(acc, scale, s_b2[o]));
+            set_output(o);
             R[o] = 0.0f;
         }
         __syncwarp();
         const uint64_t gid = p.traj_offset + (uint64_t)i;
-        const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32), key0 = (uint32_t)p.seed,
-                       key1 = (uint32_t)(p.seed >> 32);
+        const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
         const float invT = p.invT;
         const float *gl = p.dl_dobs + i * p.dl_stride;
         int row_cached = -1;
-        uint4 row = make_uint4(0, 0, 0, 0);
+        uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
         auto event_at = [&](int kk) -> int {
             const int r = kk >> 3;
-            if (r != row_cached) { row = p.ev[(int64_t)r * n + i]; row_cached = r; }
+            if (r != row_cached) {
+                row = (r == row_cached - 1) ? row_below : p.ev[(int64_t)r * n + i];
+                row_cached = r;
+                if (r > 0) row_below = p.ev[(int64_t)(r - 1) * n + i];
+            }
             const int slot = kk & 7;
             const uint32_t w = word_of(row, slot >> 1);
             return (slot & 1) ? (int)(w >> 16) : (int)(w & 0xffff);
@@ -767,6 +794,10 @@ __global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const 
         int brk_next = s_hi >= 0 ? p.brk_k[(int64_t)s_hi * n + i] : -1;
         int mism = 0;
         int ck_row = L / p.K, ck_off = L - ck_row * p.K;
+        const float4 *a4 = reinterpret_cast<const float4 *>(a);
+        float4 *key4 = reinterpret_cast<float4 *>(key);
+        const float4 *G24 = reinterpret_cast<const float4 *>(G2);
+        const int nq = nop >> 2;
         for (int k = L; k >= 0; --k) {
             const bool draw = (k < L) || (st == SSA_TRAJ_OK);
             const int s_top = s_hi;
@@ -776,95 +807,85 @@ __global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const 
             }
             if (draw) {
                 const int jk = event_at(k);
-                // pass 1: the forward's propensities and race, log2 keys
-                float ab = 0.0f, Eb = 1.0f, lmaxp = -CUDART_INF_F;
-                int jb = -1;
-                for (int b = lane; b < p.nb; b += 32) {
-                    const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, c2, c3), key0, key1);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        // predicated as in the forward (j = -1 and a = 0 add nothing and have key -inf)
-                        const int j = 4 * b + q - 1;
-                        const float E = neg_log_unit(u01(word_of(r, q)));
-                        const float a = j < 0 ? 0.0f : grn_prop(p, max(j, 0), aH, aO, X, s_d);
-                        race(a, E, j, ab, Eb, jb);
-                        const float l = a > 0.0f ? __log2f(a) - __log2f(E) : -CUDART_INF_F;
-                        lmaxp = fmaxf(lmaxp, l);
-                        if (j >= 0 && j < p.M) lj[j] = l;
-                    }
+                // pass 1: the keys; the waiting-time word and the padded ones have rate 0 and key 0
+                float rmax = 0.0f;
+                for (int c = 0; c < rounds; ++c) {
+                    const int b = 32 * c + lane;
+                    const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, noise.c2, noise.c3), noise.key0,
+                                                  noise.key1);
+                    const float4 av = a4[b];
+                    const float4 kv = make_float4(av.x * inv_exp_of_word(r.x), av.y * inv_exp_of_word(r.y),
+                                                  av.z * inv_exp_of_word(r.z), av.w * inv_exp_of_word(r.w));
+                    rmax = fmaxf(rmax, fmaxf(fmaxf(kv.x, kv.y), fmaxf(kv.z, kv.w)));
+                    key4[b] = kv;
                 }
-                warp_race_combine(ab, Eb, jb);
-                const float lmax = warp_max(lmaxp);
-                mism += (jb != jk);
+                rmax = warp_max_nonneg(rmax);
+                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f)) rmax = warp_keys_scaled(rounds, a, k, noise, rmax, key);
                 __syncwarp();
-                // pass 2: soft-sample weights q_j = exp2((l_j - l_max)/T), Z = sum q, W = sum q w with
-                // w_j = +lam_s (production of s) or -lam_s (degradation of s); one loop per reaction range, so
-                // neither pass branches on the kind of reaction
+                const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
+                const bool k_tops = key[jk + 1] * inv_rmax >= 1.0f - kTieMargin;
+                // pass 2: soft-sample weights q_j = (key_j / largest)^(1/T), Z = sum q, W = sum q w with
+                // w_j = +lam_s (production of s) or -lam_s (degradation of s)
                 float Zp = 0.0f, Wp = 0.0f;
-                for (int j = lane; j < nd; j += 32) {
-                    const float l = lj[j];
-                    const float qv = l > -CUDART_INF_F ? exp2f((l - lmax) * invT) : 0.0f;
-                    lj[j] = qv;
-                    Zp += qv;
-                    Wp = fmaf(qv, lam[j], Wp);
-                }
-                for (int s2 = lane; s2 < nd; s2 += 32) {
-                    const float l = lj[nd + s2];
-                    const float qv = l > -CUDART_INF_F ? exp2f((l - lmax) * invT) : 0.0f;
-                    lj[nd + s2] = qv;
-                    Zp += qv;
-                    Wp = fmaf(-qv, lam[s2], Wp);
-                }
+                int near = 0;  // keys within the tie margin of the largest
+                float qp[NS > 0 ? NS : 1], qd[NS > 0 ? NS : 1];
+                each_species([&](int c, int s) {
+                    const float rp = key[s + 1] * inv_rmax, rd = key[nd + s + 1] * inv_rmax;
+                    near += (rp >= 1.0f - kTieMargin) + (rd >= 1.0f - kTieMargin);
+                    const float q1 = ex2_approx(lg2_approx(rp) * invT), q2 = ex2_approx(lg2_approx(rd) * invT);
+                    Zp += q1 + q2;
+                    Wp = fmaf(q1 - q2, lam(c), Wp);
+                    if (NS > 0) {
+                        qp[NS > 0 ? c : 0] = q1;
+                        qd[NS > 0 ? c : 0] = q2;
+                    } else {
+                        key[s + 1] = q1;
+                        key[nd + s + 1] = q2;
+                    }
+                });
+                // the recorded reaction won the race if its key is the only one at the top; near ties are raced again
+                if (__reduce_add_sync(0xffffffffu, near) == 1) mism += !k_tops;
+                else mism += warp_race_exact(rounds, a, k, noise) != jk;
                 const float Z = warp_sum(Zp), Wq = warp_sum(Wp);
-                const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ;
-                const float cz = invZ * invT;
-                // pass 3: choice-path adjoints psi_j = q_j / Z (w_j - W/Z) / T per reaction (HOLD readout: no
-                // waiting-time path); d log(k_max sigma(E)) / dE = 1 - sigma(E)
-                for (int h = lane; h < nh; h += 32) {
-                    const float psi = lj[h] * cz * (lam[h] - Wbar);
-                    G1[h] = fmaf(psi, 1.0f - aH[h] * inv_kmax, G1[h]);
-                }
-                for (int o = lane; o < no; o += 32) {
-                    const float psi = lj[nh + o] * cz * (lam[nh + o] - Wbar);
-                    G2[o] = psi * (1.0f - aO[o] * inv_kmax);
-                }
-                for (int s2 = lane; s2 < nd; s2 += 32) {
-                    const float psi = lj[nd + s2] * cz * (-lam[s2] - Wbar);
-                    dlogd[s2] += psi;
-                    ctd[s2] = X[s2] > 0 ? __fdividef(psi, int2f(X[s2])) : 0.0f;  // a = d X > 0 where X > 0
-                }
+                const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ, cz = invZ * invT;
+                // pass 3: psi_j = q_j / Z (w_j - W/Z) / T (HOLD readout: no waiting-time path); the outputs first,
+                // since lambda_h receives (W2^T G2)_h
+                auto weight_p = [&](int c, int s) { return NS > 0 ? qp[NS > 0 ? c : 0] : key[s + 1]; };
+                auto weight_d = [&](int c, int s) { return NS > 0 ? qd[NS > 0 ? c : 0] : key[nd + s + 1]; };
+                each_species([&](int c, int s) {
+                    if (32 * c + 31 >= nh && s >= nh) {
+                        const int o = s - nh;
+                        const float g = weight_p(c, s) * cz * (lam(c) - Wbar) * cO[o];
+                        G2[o] = g;
+                        db2[o] += g;
+                        R[o] += g;
+                    }
+                });
                 __syncwarp();
-                for (int o = lane; o < no; o += 32) {
-                    db2[o] += G2[o];
-                    R[o] += G2[o];
-                }
-                // lam_h += (W2^T G2)_h for the hidden genes; every species adds its degradation term
-                if (no <= kGrnOutBatch) {
-                    // up to kGrnOutBatch outputs: the column's loads are issued together (one L1 latency per
-                    // hidden gene instead of one per output), then summed in output order
-                    for (int h = lane; h < nh; h += 32) {
-                        float w[kGrnOutBatch];
+                each_species([&](int c, int s) {
+                    const float l = lam(c), psi = weight_d(c, s) * cz * (-l - Wbar);
+                    const int x = X[s];
+                    dlogd(c) += psi;
+                    float acc = __fdividef(psi, __int2float_rn(x));
+                    acc = x > 0 ? acc : 0.0f;  // a = d X > 0 where X > 0
+                    G1(c) = fmaf(weight_p(c, s) * cz * (l - Wbar), cH[s], G1(c));
+                    const float4 *w = W2t + (int64_t)s * nq;
+                    auto column = [&](int q) {  // in output order; the padding and the outputs' rows add 0
+                        const float4 wv = __ldg(w + q), g = G24[q];
+                        acc = fmaf(wv.w, g.w, fmaf(wv.z, g.z, fmaf(wv.y, g.y, fmaf(wv.x, g.x, acc))));
+                    };
 #pragma unroll
-                        for (int o = 0; o < kGrnOutBatch; ++o) w[o] = o < no ? __ldg(W2f + o * nh + h) : 0.0f;
-                        float acc = ctd[h];
-#pragma unroll
-                        for (int o = 0; o < kGrnOutBatch; ++o)
-                            if (o < no) acc = fmaf(w[o], G2[o], acc);
-                        lam[h] += acc;
-                    }
-                } else {
-                    for (int h = lane; h < nh; h += 32) {
-                        float acc = ctd[h];
-                        for (int o = 0; o < no; ++o) acc = fmaf(__ldg(W2f + o * nh + h), G2[o], acc);
-                        lam[h] += acc;
-                    }
-                }
-                for (int s2 = nh + lane; s2 < nd; s2 += 32) lam[s2] += ctd[s2];
+                    for (int q = 0; q < 3; ++q)
+                        if (q < nq) column(q);
+                    for (int q = 3; q < nq; ++q) column(q);
+                    lam(c) = l + acc;
+                });
             }
-            __syncwarp();
             // HOLD samples of the outputs at state k
-            for (int s = s_hi + 1; s <= s_top; ++s)
-                for (int o = lane; o < no; o += 32) lam[nh + o] += gl[(int64_t)s * no + o];
+            for (int s2 = s_hi + 1; s2 <= s_top; ++s2)
+                each_species([&](int c, int s) {
+                    if (32 * c + 31 >= nh && s >= nh) lam(c) += gl[(int64_t)s2 * no + s - nh];
+                });
             if (ck_off == 0) {
                 const int *ck = p.ckpt + (int64_t)ck_row * nd * n + i;
                 int bad = 0;
@@ -876,22 +897,30 @@ __global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const 
             --ck_off;
             __syncwarp();
             if (k > 0) {
-                // undo event k-1 (state k -> k-1); a hidden change adds delta R to dW2[:, i]
+                // undo event k-1 (state k -> k-1); a hidden change adds delta R to dW2[:, i] (a reduction without a
+                // returned value: the warp does not wait for memory, and one lane's adds to a place keep their order)
                 const int jp = event_at(k - 1);
                 const int sp = jp < nd ? jp : jp - nd;
                 const int delta = jp < nd ? 1 : -1;
-                if (lane == 0) X[sp] -= delta;
+                if (lane == 0) {
+                    const int x = X[sp] - delta;
+                    X[sp] = x;
+                    a[nd + sp + 1] = __fmul_rn(s_d[sp], int2f(x));
+                }
                 if (sp < nh) {
                     for (int o = lane; o < no; o += 32) {
-                        dW2[o * nh + sp] += (float)delta * R[o];
+                        atomicAdd(dW2 + o * nh + sp, (float)delta * R[o]);
                         E2acc[o] -= (long long)delta * __ldg(W2fix + o * nh + sp);
-                        aO[o] = p.k_max * sigmoid_f(e2_value(E2acc[o], scale, s_b2[o]));
+                        set_output(o);
                     }
                 }
             }
             __syncwarp();
         }
-        for (int h = lane; h < nh; h += 32) p.G1[i * nh + h] = G1[h];
+        each_species([&](int c, int s) {
+            if (s < nh) p.G1[i * nh + s] = G1(c);
+            key[s] = dlogd(c);  // for the block's sum
+        });
         if (lane == 0 && mism) atomicAdd(p.mismatch, mism);
     } else if (i < n) {
         for (int h = lane; h < nh; h += 32) p.G1[i * nh + h] = 0.0f;
@@ -899,12 +928,13 @@ __global__ void __launch_bounds__(128, SSA_GRN_ADJ_BLOCKS) grn_adj_kernel(const 
     __syncthreads();
     // fixed-order sum over the block's warps: [db2 | dlogd]
     const int red = no + nd;
-    float *base0 = reinterpret_cast<float *>(wb);
+    const float *base0 = reinterpret_cast<const float *>(wb);
+    const size_t at_db2 = (db2 - wbase), at_dlogd = wide;
     for (int q = threadIdx.x; q < red; q += blockDim.x) {
         float acc = 0.0f;
         for (int w = 0; w < W; ++w) {
             const float *wp = base0 + w * per_warp;
-            acc += q < no ? wp[3 * ndp + 2 * nhp + 5 * nop + q] : wp[3 * ndp + 2 * nhp + 6 * nop + Mp + (q - no)];
+            acc += q < no ? wp[at_db2 + q] : wp[at_dlogd + (q - no)];
         }
         p.partial[(int64_t)blockIdx.x * red + q] = acc;
     }
@@ -968,6 +998,33 @@ namespace {
 // N-tile of the tensor-core dW1 = G^T x (n_in columns)
 int grn_dw1_nt(const ssa_grn *g) { return (g->n_in % 112 == 0) ? 112 : 64; }
 
+// shared memory one CTA may hold on sm_103a
+constexpr size_t kGrnMaxSmem = 227 * 1024;
+
+size_t grn_fwd_smem(const ssa_grn *g, int warps)
+{
+    const int ndp = (g->n_dyn + 3) & ~3, nop = (g->n_out + 3) & ~3;
+    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop) + 16 +
+           4 * (size_t)warps * (ndp + wide_len(g->M) + 2 * (size_t)nop);
+}
+
+bool grn_sums_in_registers(const ssa_grn *g) { return g->n_dyn <= kGrnRegSpecies; }  // 288 = 9 rounds
+
+size_t grn_adj_smem(const ssa_grn *g, int warps)
+{
+    const int nop = (g->n_out + 3) & ~3;
+    return 4 * ((size_t)g->n_dyn + nop) + 16 +
+           4 * (size_t)warps * grn_adj_words(g->n_hid, g->n_out, !grn_sums_in_registers(g));
+}
+
+// warps per block of the exact forward and its adjoint
+int grn_warps(const ssa_grn *g)
+{
+    int w = kGrnWarps;
+    while (w > 1 && std::max(grn_fwd_smem(g, w), grn_adj_smem(g, w)) > kGrnMaxSmem) --w;
+    return w;
+}
+
 WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, const ssa_fwd_opts *o)
 {
     WsLayout L{};
@@ -995,6 +1052,7 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
     L.xb = take((size_t)(n_img > 0 ? n_img : 1) * L.n_in_pad * 2);
     L.W2fix = take((size_t)g->n_out * g->n_hid * 4);
     L.W2f = take((size_t)g->n_out * g->n_hid * 4);
+    L.W2t = take((size_t)((g->n_out + 3) & ~3) * g->n_dyn * 4);
     L.dvec = take((size_t)g->n_dyn * 4);
     L.grid = take(16 * sizeof(int));
     // split-K partial sums of E1 (forward) and of dW1 (backward), when the product fills too few SMs
@@ -1007,7 +1065,8 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
         const int K = o->selector == SSA_SELECT_SOFT ? kGrnSoftK : o->ckpt_interval > 0 ? o->ckpt_interval : 64;
         L.ev_rows = (o->max_steps + 7) / 8;
         L.n_ckpt = o->max_steps / K + 1;
-        L.max_blocks = (n + kGrnWarps - 1) / kGrnWarps;
+        const int wpb = o->selector == SSA_SELECT_SOFT ? kGrnWarps : grn_warps(g);
+        L.max_blocks = (n + wpb - 1) / wpb;
         L.xfinal = take((size_t)g->n_dyn * n * 4);
         L.ev = take((size_t)L.ev_rows * n * sizeof(uint4));
         L.ckpt = take((size_t)L.n_ckpt * g->n_dyn * n * 4);
@@ -1030,11 +1089,6 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
     return L;
 }
 
-size_t grn_fwd_smem(const ssa_grn *g)
-{
-    const int ndp = (g->n_dyn + 3) & ~3, nhp = (g->n_hid + 3) & ~3, nop = (g->n_out + 3) & ~3;
-    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop) + 16 + 4 * (size_t)kGrnWarps * (ndp + nhp + 3 * (size_t)nop);
-}
 
 size_t grn_soft_fwd_smem(const ssa_grn *g)
 {
@@ -1049,15 +1103,6 @@ size_t grn_soft_adj_smem(const ssa_grn *g)
     return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop + (size_t)kGrnWarps * per_warp);
 }
 
-// shared memory one CTA may hold on sm_103a
-constexpr size_t kGrnMaxSmem = 227 * 1024;
-
-size_t grn_adj_smem(const ssa_grn *g)
-{
-    const int ndp = (g->n_dyn + 3) & ~3, nhp = (g->n_hid + 3) & ~3, nop = (g->n_out + 3) & ~3;
-    const size_t per_warp = 4 * (size_t)ndp + 2 * (size_t)nhp + 6 * (size_t)nop + (size_t)g->Mp;
-    return 4 * ((size_t)g->n_dyn + nop) + 16 + 4 * (size_t)kGrnWarps * per_warp;
-}
 
 #define GRN_CUDA_TRY(expr)                                                                              \
     do {                                                                                                \
@@ -1141,10 +1186,12 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
     if (S > 0) GRN_CUDA_TRY(cudaMemcpyAsync(ws + L.ts, sample_times, (size_t)S * 8, cudaMemcpyDeviceToDevice, st));
     GRN_CUDA_TRY(launch_validate_inputs(reinterpret_cast<const double *>(ws + L.ts), S, t_end, nullptr, 0, g->n_dyn,
                                         0, flag, st));
+    GRN_CUDA_TRY(cudaMemsetAsync(ws + L.W2t, 0, (size_t)((g->n_out + 3) & ~3) * g->n_dyn * 4, st));
     grn_exponents_kernel<<<64, 256, 0, st>>>(W1, (int64_t)g->n_hid * g->n_in, W2, (int64_t)g->n_out * g->n_hid, grid);
     grn_prepare_kernel<<<256, 256, 0, st>>>(W1, W2, x_img, log_d, g->n_in, g->n_hid, g->n_out, n_img, L.n_in_pad,
                                             reinterpret_cast<uint16_t *>(ws + L.W1L), reinterpret_cast<int *>(ws + L.W2fix),
-                                            reinterpret_cast<float *>(ws + L.W2f), reinterpret_cast<uint16_t *>(ws + L.xb),
+                                            reinterpret_cast<float *>(ws + L.W2f), reinterpret_cast<float *>(ws + L.W2t),
+                                            reinterpret_cast<uint16_t *>(ws + L.xb),
                                             reinterpret_cast<float *>(ws + L.dvec), grid);
     GRN_CUDA_TRY(cudaGetLastError());
     // E1 = W1 x + b1 on the tensor cores: one accumulator per limb, summed in binary64
@@ -1180,6 +1227,7 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
     p.E1 = reinterpret_cast<const float *>(ws + L.E1);
     p.W2fix = reinterpret_cast<const int *>(ws + L.W2fix);
     p.W2f = reinterpret_cast<const float *>(ws + L.W2f);
+    p.W2t = reinterpret_cast<const float4 *>(ws + L.W2t);
     p.b2 = b2;
     p.dvec = reinterpret_cast<const float *>(ws + L.dvec);
     p.grid = grid + 3;
@@ -1208,9 +1256,10 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
             p, reinterpret_cast<float *>(obs_out), opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
-        const size_t smem = grn_fwd_smem(g);
+        const int wpb = grn_warps(g);
+        const size_t smem = grn_fwd_smem(g, wpb);
         GRN_CUDA_TRY(cudaFuncSetAttribute(grn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_fwd_kernel<<<(unsigned)((n + kGrnWarps - 1) / kGrnWarps), 32 * kGrnWarps, smem, st>>>(p, opts->record);
+        grn_fwd_kernel<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(p, opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     }
     if (n > 0 && draws_out) GRN_CUDA_TRY(cudaMemcpyAsync(draws_out, p.draws, (size_t)n * 4, cudaMemcpyDeviceToDevice, st));
@@ -1275,6 +1324,7 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     p.E1 = reinterpret_cast<const float *>(ws + L.E1);
     p.W2fix = reinterpret_cast<const int *>(ws + L.W2fix);
     p.W2f = reinterpret_cast<const float *>(ws + L.W2f);
+    p.W2t = reinterpret_cast<const float4 *>(ws + L.W2t);
     p.b2 = run->b2;
     p.dvec = reinterpret_cast<const float *>(ws + L.dvec);
     p.grid = reinterpret_cast<const int *>(ws + L.grid) + 3;
@@ -1296,7 +1346,8 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     p.err = flag + 1;
     p.n_ckpt = L.n_ckpt;
     p.seg = soft ? reinterpret_cast<float *>(ws + L.soft_seg) : nullptr;
-    const int64_t nblk = (n + kGrnWarps - 1) / kGrnWarps;
+    const int wpb = soft ? kGrnWarps : grn_warps(g);
+    const int64_t nblk = (n + wpb - 1) / wpb;
     float *red = reinterpret_cast<float *>(ws + L.red);
     if (n > 0 && soft) {
         const size_t smem = grn_soft_adj_smem(g);
@@ -1304,9 +1355,12 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
         grn_soft_adj_kernel<<<(unsigned)nblk, 32 * kGrnWarps, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
-        const size_t smem = grn_adj_smem(g);
-        GRN_CUDA_TRY(cudaFuncSetAttribute(grn_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_adj_kernel<<<(unsigned)nblk, 32 * kGrnWarps, smem, st>>>(p);
+        const size_t smem = grn_adj_smem(g, wpb);
+        const int nd = g->n_dyn;
+        auto kern = !grn_sums_in_registers(g) ? grn_adj_kernel<0, 0>
+                    : nd > 192 ? grn_adj_kernel<9, 6> : nd > 96 ? grn_adj_kernel<6, 3> : grn_adj_kernel<3, 0>;
+        GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());
     }
     GRN_CUDA_TRY(launch_reduce_partials(p.partial, nblk, L.red_len, nullptr, 0, red, nullptr, st));
