@@ -62,6 +62,11 @@ __device__ __forceinline__ void jit_lam_add2(float (&lam)[JN], float (&lo)[JN], 
         if (s == sp) acc2(lam[s], lo[s], v);
 }
 
+// The bin readout's held runs in shared memory, one column per thread (kJitFwdBlock threads at most).
+#define SSA_JIT_BIN_RUNS(R)                                                                               \
+    __shared__ int s_runs[(R) == SSA_READOUT_BIN ? (kBinRuns + 1) * kRunWords * kJitFwdBlock : 1];        \
+    BinRunsShared bruns{0, 0, s_runs + threadIdx.x, kJitFwdBlock}
+
 // BIN readout state of a forward: cleared integrals, observed species (0 where the list is invalid)
 __device__ __forceinline__ void jit_bin_init(const FwdParams &p, bool bad_obs, float (&bacc)[kBinMaxObs],
                                              int (&osp)[kBinMaxObs])
@@ -199,8 +204,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     float E[NQ], En[NQ];
     step_noise<NQ>(E, 0u, c2, c3, key0, key1);
     float bacc[kBinMaxObs];
-    BinRuns bruns;
-    bin_runs_init(bruns);
+    SSA_JIT_BIN_RUNS(READOUT);
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
@@ -363,8 +367,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
     uint4 r = philox4x32_10(make_uint4(0u, 0u, c2, c3), key0, key1);
     float E0 = neg_log_unit(u01(r.x)), U1 = u01(r.y);
     float bacc[kBinMaxObs];
-    BinRuns bruns;
-    bin_runs_init(bruns);
+    SSA_JIT_BIN_RUNS(READOUT);
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
@@ -445,6 +448,69 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
     p.status[i] = status;
 }
 
+// Bin readout with a gradient per trajectory (one observable): the sums over aligned chunks of 16 bins and more of
+// every trajectory's row, formed before the walk by the warp's lanes side by side along the row; the walk then sums
+// the whole bins of an interval from chunks and the loose bins at its ends. Summed bin by bin in the walk, a row per
+// lane, the loads set the time. A row that starts and ends on 16 bytes is read in 16-byte pieces, others (of up to
+// 32 bins a chunk) by the float. s_chunk [kChunkRows][kJitAdjBlock]; from kChunkMinBins bins on (below, a row is a line
+// or two and the intervals hold no long runs).
+// Ion channel, 262,144 trajectories x 800 bins, the adjoint: 2,050 us bin by bin; 800 with the sum of every interval
+// formed by the warp beforehand (a reduction per interval and row); 395 so.
+constexpr int kJitAdjBlock = 128;
+constexpr int kChunkRows = 56, kChunkMinBins = 32;
+
+// bits of the chunk size for S bins, 0: no chunks
+__device__ __forceinline__ int jit_chunk_shift(const AdjParams &p)
+{
+    if (p.bin_prefix || p.n_obs != 1 || p.S < kChunkMinBins || (int)blockDim.x != kJitAdjBlock) return 0;
+    int shift = 4;
+    while (((p.S - 1) >> shift) >= kChunkRows) ++shift;
+    const bool pieces = (p.S & 3) == 0 && (p.dl_stride & 3) == 0 && (reinterpret_cast<uintptr_t>(p.dl_dobs) & 15) == 0;
+    return shift <= (pieces ? 7 : 5) ? shift : 0;
+}
+
+__device__ __forceinline__ void jit_bin_chunk_sums(const AdjParams &p, int64_t i, bool active, int shift, float *s_chunk)
+{
+    const int lane = threadIdx.x & 31, S = p.S;
+    const bool pieces = (p.S & 3) == 0 && (p.dl_stride & 3) == 0 && (reinterpret_cast<uintptr_t>(p.dl_dobs) & 15) == 0;
+    const int per = pieces ? 4 : 1;                  // bins of a lane's load
+    const int group = (1 << shift) / per;            // lanes of a chunk: 4 to 32
+    float *col = s_chunk + (threadIdx.x & ~31);
+    unsigned rows = __ballot_sync(0xffffffffu, active);
+    while (rows) {
+        const int j = __ffs(rows) - 1;
+        rows &= rows - 1;
+        const float *row = p.dl_dobs + __shfl_sync(0xffffffffu, (long long)i, j) * p.dl_stride;
+        for (int e0 = per * lane; e0 - per * lane < S; e0 += 8 * 32 * per) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int e = e0 + 32 * per * u;
+                v[u] = 0.0f;
+                if (e < S) {
+                    if (pieces) {
+                        const float4 w = *reinterpret_cast<const float4 *>(row + e);
+                        v[u] = (w.x + w.y) + (w.z + w.w);
+                    } else {
+                        v[u] = row[e];
+                    }
+                }
+            }
+            for (int off = 1; off < group; off <<= 1)
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] += __shfl_xor_sync(0xffffffffu, v[u], off);
+            if ((lane & (group - 1)) == 0) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    const int e = e0 + 32 * per * u;
+                    if (e < S) col[(e >> shift) * kJitAdjBlock + j] = v[u];
+                }
+            }
+        }
+    }
+    __syncwarp();
+}
+
 // Per-trajectory adjoint; returns the trajectory's per-reaction adjoints in dAr.
 //
 // NT temperatures at once (NT > 1): the walk, the regenerated noise, the propensities, the race check and
@@ -461,7 +527,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
 // 2^-sc. The trajectory's result is dAr 2^sc. With sc = 0 the arithmetic is the plain walk's bit for bit.
 template <int READOUT, bool WIDE = false, int NT = 1>
 __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&kr)[JM], const int64_t i, const int st,
-                                             float (&dAr)[NT][JM], int &sc)
+                                             float (&dAr)[NT][JM], int &sc, const BinChunks chunks)
 {
     static_assert(!WIDE || NT == 1, "the wide-range walk takes one temperature");
     sc = 0;
@@ -654,7 +720,8 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
             }
         }
         if (kBin) {
-            bin_state_terms(addx, d_first, d_last, gl, p.bin_prefix, p.n_obs, s_hi + 1, s_top, draw, tau_k, gq, gk);
+            bin_state_terms(addx, d_first, d_last, gl, p.bin_prefix, p.n_obs, s_hi + 1, s_top, draw, tau_k, gq, gk,
+                            chunks);
 #pragma unroll
             for (int c = 0; c < kBinMaxObs; ++c) {
                 gq[c] = gk[c];
@@ -800,8 +867,7 @@ __device__ __forceinline__ void jit_fwd_soft(const FwdParams &p)
     float E[NQ], En[NQ];
     step_noise<NQ>(E, 0u, c2, c3, key0, key1);
     float bacc[kBinMaxObs];
-    BinRuns bruns;
-    bin_runs_init(bruns);
+    SSA_JIT_BIN_RUNS(READOUT);
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     auto xobs = [&](int c) { return jit_fsel(X, osp[c]); };
@@ -883,7 +949,7 @@ __device__ __forceinline__ void jit_fwd_soft(const FwdParams &p)
 // Exact gradient of the soft forward, one trajectory; per-reaction adjoints into dAr.
 template <int READOUT>
 __device__ __forceinline__ void jit_adj_soft_traj(const AdjParams &p, const float (&kr)[JM], const int64_t i,
-                                                  const int st, float (&dAr)[JM])
+                                                  const int st, float (&dAr)[JM], const BinChunks chunks)
 {
     const int64_t n = p.n_traj;
     const int d = p.draws[i];
@@ -1009,7 +1075,8 @@ __device__ __forceinline__ void jit_adj_soft_traj(const AdjParams &p, const floa
                 mu += dt_dir;
             }
             if (kBin) {
-                bin_state_terms(addx, d_first, d_last, gl, p.bin_prefix, p.n_obs, s_hi + 1, s_top, draw, tau_k, gq, gk);
+                bin_state_terms(addx, d_first, d_last, gl, p.bin_prefix, p.n_obs, s_hi + 1, s_top, draw, tau_k, gq, gk,
+                                chunks);
 #pragma unroll
                 for (int q = 0; q < kBinMaxObs; ++q) gq[q] = gk[q];
             } else {
@@ -1060,9 +1127,18 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
     if (i < n) st = p.status[i];
     const bool active = st == SSA_TRAJ_OK || st == SSA_TRAJ_ABSORBED || st == SSA_TRAJ_STEP_CAP;
     int sc = 0;
+    BinChunks chunks{nullptr, 0, kJitAdjBlock};
+    if constexpr (READOUT == SSA_READOUT_BIN) {
+        __shared__ float s_chunk[kChunkRows * kJitAdjBlock];
+        chunks.shift = jit_chunk_shift(p);
+        if (chunks.shift) {
+            jit_bin_chunk_sums(p, i, active, chunks.shift, s_chunk);
+            chunks.sum = s_chunk + tid;
+        }
+    }
     if (active) {
-        if constexpr (SOFT) jit_adj_soft_traj<READOUT>(p, kr, i, st, dAr[0]);
-        else jit_adj_traj<READOUT, WIDE, NT>(p, kr, i, st, dAr, sc);
+        if constexpr (SOFT) jit_adj_soft_traj<READOUT>(p, kr, i, st, dAr[0], chunks);
+        else jit_adj_traj<READOUT, WIDE, NT>(p, kr, i, st, dAr, sc, chunks);
     }
     const int warp = tid >> 5, lane = tid & 31, nwarps = B >> 5;
     if constexpr (WIDE) {
