@@ -79,7 +79,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
     constexpr int NQ = MC > 0 ? MC + 1 : 1;
     float E[NQ], En[NQ];
     const bool draw_last = st == SSA_TRAJ_OK;
-    if (MC > 0) step_noise<NQ>(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
+    if (MC > 0) step_noise_inv<NQ>(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
 
     // BIN readout: gq = g of the bin that contains t_{k+1} (none past the last edge), xo = X_{k+1}
     // at the observables
@@ -118,39 +118,60 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
         float tau_k = 0.0f;
         if (draw) {
             const int jk = event_at(k);
-            float a0 = 0.0f, ab = 0.0f, Eb = 1.0f, E0, lmax = -CUDART_INF_F;
+            float a0 = 0.0f, E0, m1 = 0.0f, m2 = 0.0f;
             int jb = -1;
             float ar[MC > 0 ? MC : 1], lr[MC > 0 ? MC : 1];
-            // pass 1: the forward's propensities, a0 and race, bit for bit; log2 keys
+            // pass 1: the forward's propensities and a0; the race's keys a_j / E_j with the two largest
+            auto enter = [&](float key, int j) {
+                jb = key > m1 ? j : jb;
+                m2 = fmaxf(m2, fminf(m1, key));
+                m1 = fmaxf(m1, key);
+            };
             if constexpr (MC > 0) {
-                if (k > 0) step_noise<NQ>(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
+                if (k > 0) step_noise_inv<NQ>(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
                 E0 = E[0];
 #pragma unroll
                 for (int j = 0; j < MC; ++j) {
-                    const float a = __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B));
-                    a0 = __fadd_rn(a0, a);
-                    race(a, E[j + 1], j, ab, Eb, jb);
-                    ar[j] = a;
-                    lr[j] = a > 0.0f ? __log2f(a) - __log2f(E[j + 1]) : -CUDART_INF_F;
-                    lmax = fmaxf(lmax, lr[j]);
+                    ar[j] = __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B));
+                    a0 = __fadd_rn(a0, ar[j]);
+                }
+                const float sc_key = key_scale(a0);
+#pragma unroll
+                for (int j = 0; j < MC; ++j) {
+                    lr[j] = (ar[j] * sc_key) * E[j + 1];
+                    enter(lr[j], j);
                 }
             } else {
                 uint4 cache;
                 int cb = -1;
                 E0 = exp_variate((uint32_t)k, 0, c2, c3, key0, key1, cache, cb);
+                for (int j = 0; j < M; ++j) a0 = __fadd_rn(a0, __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B)));
+                const float sc_key = key_scale(a0);
                 for (int j = 0; j < M; ++j) {
-                    const float a = __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B));
-                    a0 = __fadd_rn(a0, a);
-                    float l = -CUDART_INF_F;
-                    if (a > 0.0f) {
-                        const float Ej = exp_variate((uint32_t)k, j + 1, c2, c3, key0, key1, cache, cb);
-                        race(a, Ej, j, ab, Eb, jb);
-                        l = __log2f(a) - __log2f(Ej);
-                        lmax = fmaxf(lmax, l);
+                    const int q = j + 1;
+                    if ((q >> 2) != cb) {
+                        cb = q >> 2;
+                        cache = philox4x32_10(make_uint4((uint32_t)cb, (uint32_t)k, c2, c3), key0, key1);
                     }
-                    qbuf[j * B] = l;
+                    const float a = __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B));
+                    const float key = (a * sc_key) * inv_exp_of_word(word_of(cache, q & 3));
+                    enter(key, j);
+                    qbuf[j * B] = key;
                 }
             }
+            // the recorded reaction won the race if its key is the largest by more than the keys' error; near ties are
+            // raced again as the forward races
+            if (m2 >= m1 * (1.0f - kTieMargin)) {
+                float ab = 0.0f, Eb = 1.0f;
+                uint4 cache;
+                int cb = -1;
+                jb = -1;
+                for (int j = 0; j < M; ++j) {
+                    const float a = __fmul_rn(s_k[j], mass_action_h(s_rx[j], X, B));
+                    race(a, exp_variate((uint32_t)k, j + 1, c2, c3, key0, key1, cache, cb), j, ab, Eb, jb);
+                }
+            }
+            const float inv_m1 = m1 > 0.0f ? __fdividef(1.0f, m1) : 0.0f;
             mism += (jb != jk);
             const float tau = waiting_time(E0, a0);
             tau_k = tau;
@@ -180,17 +201,17 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
             }
             const float dtau = mu + dtau_dir;
             const float dLda0 = -dtau * tau / a0;
-            // pass 2: soft-sample weights y~_j ~ exp2((l_j - l_max)/T) and W = sum y~ w
+            // pass 2: soft-sample weights y~_j ~ (key_j / largest)^(1/T) and W = sum y~ w
             float Z = 0.0f, Wq = 0.0f;
             if constexpr (MC > 0) {
                 float wr[MC];
 #pragma unroll
                 for (int j = 0; j < MC; ++j) {
-                    const float q = lr[j] == -CUDART_INF_F ? 0.0f : exp2f((lr[j] - lmax) * invT);
+                    const float q = ex2_approx(lg2_approx(lr[j] * inv_m1) * invT);
                     lr[j] = q;
                     wr[j] = stoich_dot(s_rx[j], s_st, lam, B);
                     Z += q;
-                    Wq += q * wr[j];
+                    Wq += q > 0.0f ? q * wr[j] : 0.0f;
                 }
                 const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ;
                 // pass 3: per-reaction adjoints and the state adjoint
@@ -204,8 +225,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 }
             } else {
                 for (int j = 0; j < M; ++j) {
-                    const float l = qbuf[j * B];
-                    const float q = (l == -CUDART_INF_F) ? 0.0f : exp2f((l - lmax) * invT);
+                    const float q = ex2_approx(lg2_approx(qbuf[j * B] * inv_m1) * invT);
                     qbuf[j * B] = q;
                     if (q > 0.0f) {
                         Z += q;

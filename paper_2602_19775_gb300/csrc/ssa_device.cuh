@@ -206,6 +206,31 @@ __device__ __forceinline__ void step_noise(float (&E)[NQ], uint32_t k, uint32_t 
     }
 }
 
+// The same for the adjoints: E_0 and 1/E_q of the race's words.
+template <int NQ>
+__device__ __forceinline__ void step_noise_inv(float (&v)[NQ], uint32_t k, uint32_t c2, uint32_t c3, uint32_t key0,
+                                               uint32_t key1)
+{
+#pragma unroll
+    for (int b = 0; b < (NQ + 3) / 4; ++b) {
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)b, k, c2, c3), key0, key1);
+        if (4 * b + 0 < NQ) v[4 * b + 0] = b == 0 ? neg_log_unit(u01(r.x)) : inv_exp_of_word(r.x);
+        if (4 * b + 1 < NQ) v[4 * b + 1] = inv_exp_of_word(r.y);
+        if (4 * b + 2 < NQ) v[4 * b + 2] = inv_exp_of_word(r.z);
+        if (4 * b + 3 < NQ) v[4 * b + 3] = inv_exp_of_word(r.w);
+    }
+}
+
+// The adjoints' race keys a_j / E_j enter as ratios only; where a0 could take them out of the binary32 range they are
+// scaled by this power of two.
+__device__ __forceinline__ float key_scale(float a0)
+{
+    return (a0 >= 0x1p-60f && a0 <= 0x1p100f) ? 1.0f : (a0 > 1.0f ? 0x1p-60f : 0x1p100f);
+}
+// Two keys within this of each other, relatively, count as a possible tie (a key is a few units in the last place
+// off, and so is the comparison of products that decides the race).
+constexpr float kTieMargin = 0x1p-15f;
+
 // -ln u_q of one word (runtime-indexed variant for networks without a compile-time size).
 __device__ __forceinline__ float exp_variate(uint32_t k, int q, uint32_t c2, uint32_t c3, uint32_t key0, uint32_t key1,
                                              uint4 &cache, int &cached_b)

@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                     key4[b] = kv;
                 }
                 rmax = warp_max_nonneg(rmax);
-                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f)) rmax = warp_keys_scaled(rounds, a, k, noise, rmax, key);
+                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f)) rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, key);
                 __syncwarp();
                 const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
                 const bool k_tops = key[jk + 1] * inv_rmax >= 1.0f - kTieMargin;

@@ -53,16 +53,6 @@ void emit(std::string &out, const char *fmt, ...)
     out += buf;
 }
 
-// The event hooks written as selects (bit 1: X -= v_jb, 2: a component of v_jb, 4: X += v_jb, 8: the range
-// check) for networks with up to kJitSelectNnz stoichiometric entries; the others switch on jb. Timed on one
-// box (C2 step: adjoint 0.745 ms with switches, 0.716 with the component as selects, 0.739 with X -= v_jb as
-// selects, 0.713 with both; the oscillator's forward + adjoint 4.75e9 steps/s with switches and with the
-// component as selects, 4.62e9 once X -= v_jb is selects): the component only.
-#ifndef SSA_JIT_SELECT
-#define SSA_JIT_SELECT 2
-#endif
-constexpr int kJitSelectNnz = 48;
-
 int st_species(int e) { return e >> 8; }
 int st_delta(int e) { return (int)(signed char)(e & 0xff); }
 
@@ -73,35 +63,62 @@ std::string jit_source(const ssa_network *net)
     std::string s;
     s += "#include \"ssa_device.cuh\"\n";
     emit(s, "#define JN %d\n#define JM %d\nnamespace ssa {\n", N, M);
-    // propensities, in reaction order
-    s += "__device__ __forceinline__ void jit_props(const int (&X)[JN], const float (&k)[JM], float (&a)[JM], "
-         "float (&h)[JM])\n{\n";
+    // propensities, in reaction order. Counts below 2^23 are exact in binary32 and need no further cases; one test over
+    // the reactant species sends a step with a larger one to the general expressions (returned: whether it did).
+    auto props = [&](bool general) {
+        for (int j = 0; j < M; ++j) {
+            const int4 r = net->h_rx[j];
+            const char *in = "        ";
+            if (r.x < 0) emit(s, "%sh[%d] = 1.0f;\n", in, j);
+            else if (r.y < 0) emit(s, general ? "%sh[%d] = h_first(X[%d]);\n" : "%sh[%d] = f[%d];\n", in, j, r.x);
+            else if (r.y == r.x && general) emit(s, "%sh[%d] = h_homodimer(X[%d]);\n", in, j, r.x);
+            else if (r.y == r.x) emit(s, "%sh[%d] = __fmul_rn(f[%d], fmaxf(f[%d] - 1.0f, 0.0f)) * 0.5f;\n", in, j, r.x, r.x);
+            else emit(s, general ? "%sh[%d] = h_hetero(X[%d], X[%d]);\n" : "%sh[%d] = __fmul_rn(f[%d], f[%d]);\n", in, j, r.x, r.y);
+        }
+    };
+    s += "__device__ __forceinline__ bool jit_props(const int (&X)[JN], const float (&k)[JM], float (&a)[JM], "
+         "float (&h)[JM])\n{\n    unsigned m = 0;\n";
+    std::vector<bool> reacts(N, false);
     for (int j = 0; j < M; ++j) {
-        const int4 r = net->h_rx[j];
-        if (r.x < 0) emit(s, "    h[%d] = 1.0f;\n", j);
-        else if (r.y < 0) emit(s, "    h[%d] = h_first(X[%d]);\n", j, r.x);
-        else if (r.y == r.x) emit(s, "    h[%d] = h_homodimer(X[%d]);\n", j, r.x);
-        else emit(s, "    h[%d] = h_hetero(X[%d], X[%d]);\n", j, r.x, r.y);
-        emit(s, "    a[%d] = __fmul_rn(k[%d], h[%d]);\n", j, j, j);
+        if (net->h_rx[j].x >= 0) reacts[net->h_rx[j].x] = true;
+        if (net->h_rx[j].y >= 0) reacts[net->h_rx[j].y] = true;
     }
-    s += "}\n";
-    // The event-dependent hooks (range check, X += v_jb, X -= v_jb, a component of v_jb) switch on jb, whose
-    // cases the lanes of a warp run one after another when their events differ; up to kJitSelectNnz
-    // stoichiometric entries, the hooks named in SSA_JIT_SELECT are written instead as selects over every entry
-    // (the same results, no divergence; a tuning choice, set by timing both forms).
-    const bool small = net->nnz <= kJitSelectNnz;
-    const bool sel_check = small && (SSA_JIT_SELECT & 8), sel_apply = small && (SSA_JIT_SELECT & 4);
-    const bool sel_unapply = small && (SSA_JIT_SELECT & 1), sel_dv = small && (SSA_JIT_SELECT & 2);
+    for (int sp = 0; sp < N; ++sp) emit(s, "    m |= (unsigned)X[%d];\n", sp);
+    s += "    const bool big = m >= (1u << 23);\n    if (!big) {\n        float f[JN];\n";
+    for (int sp = 0; sp < N; ++sp)
+        if (reacts[sp]) emit(s, "        f[%d] = __int2float_rn(X[%d]);\n", sp, sp);
+    props(false);
+    s += "    } else {\n";
+    props(true);
+    s += "    }\n#pragma unroll\n    for (int j = 0; j < JM; ++j) a[j] = __fmul_rn(k[j], h[j]);\n    return big;\n}\n";
+    // The changes of every reaction, int8 by species, four to a word: the kernels keep the table in shared memory and
+    // apply an event with one 4-way byte dot product per species, whatever events the other lanes drew. (As a switch
+    // on the event, the cases of a warp's lanes ran one after another.)
+    const int W = (N + 3) / 4;
+    emit(s, "#define JW %d\n__device__ const int jit_changes[JM * JW] = {", W);
+    for (int j = 0; j < M; ++j)
+        for (int w = 0; w < W; ++w) {
+            uint32_t v = 0;
+            for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e)
+                if (st_species(net->h_st[e]) / 4 == w)
+                    v |= (uint32_t)(uint8_t)st_delta(net->h_st[e]) << (8 * (st_species(net->h_st[e]) % 4));
+            emit(s, "(int)0x%08xu, ", v);
+        }
+    s += "};\n";
+    // A reaction that only consumes its own reactants cannot take a count below zero (its propensity was positive), and
+    // no count below 2^23 can overflow: such networks check a step only where a count is large.
+    bool safe = true;
+    for (int j = 0; j < M; ++j)
+        for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e) {
+            const int4 r = net->h_rx[j];
+            const int sp = st_species(net->h_st[e]), d = st_delta(net->h_st[e]);
+            const int held = (r.x == sp) + (r.y == sp);  // a > 0: at least this many of the species
+            safe &= d >= -held;
+        }
+    emit(s, "constexpr bool kJitSafe = %s;\n", safe ? "true" : "false");
     // range check of X + v_jb (entries in table order; the last failing entry decides)
     s += "__device__ __forceinline__ int jit_check(const int (&X)[JN], int jb)\n{\n    int st = SSA_TRAJ_OK;\n";
-    if (sel_check) {
-        for (int j = 0; j < M; ++j)
-            for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e) {
-                const int sp = st_species(net->h_st[e]), d = st_delta(net->h_st[e]);
-                if (d < 0) emit(s, "    st = (jb == %d && X[%d] + (%d) < 0) ? SSA_TRAJ_NEG_COUNT : st;\n", j, sp, d);
-                else if (d > 0) emit(s, "    st = (jb == %d && X[%d] > 2147483647 - %d) ? SSA_TRAJ_OVERFLOW : st;\n", j, sp, d);
-            }
-    } else {
+    {
         s += "    switch (jb) {\n";
         for (int j = 0; j < M; ++j) {
             emit(s, "    case %d:\n", j);
@@ -115,53 +132,6 @@ std::string jit_source(const ssa_network *net)
         s += "    default: break;\n    }\n";
     }
     s += "    return st;\n}\n";
-    // X += v_jb and X -= v_jb
-    for (int dir = 0; dir < 2; ++dir) {
-        emit(s, "__device__ __forceinline__ void %s(int (&X)[JN], int jb)\n{\n", dir == 0 ? "jit_apply" : "jit_unapply");
-        if (dir == 0 ? sel_apply : sel_unapply) {
-            // per species, the change of the reaction that fired (a chain of selects over its entries)
-            for (int sp = 0; sp < N; ++sp) {
-                std::string expr = "0";
-                for (int j = M - 1; j >= 0; --j)
-                    for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e)
-                        if (st_species(net->h_st[e]) == sp) {
-                            char buf[64];
-                            snprintf(buf, sizeof(buf), "(jb == %d ? %d : ", j, st_delta(net->h_st[e]));
-                            expr = buf + expr + ")";
-                        }
-                // appended directly: the expression may exceed emit's buffer
-                if (expr != "0") s += "    X[" + std::to_string(sp) + "] " + (dir == 0 ? "+=" : "-=") + " " + expr + ";\n";
-            }
-        } else {
-            s += "    switch (jb) {\n";
-            for (int j = 0; j < M; ++j) {
-                emit(s, "    case %d:\n", j);
-                for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e)
-                    emit(s, "        X[%d] %s %d;\n", st_species(net->h_st[e]), dir == 0 ? "+=" : "-=",
-                         st_delta(net->h_st[e]));
-                s += "        break;\n";
-            }
-            s += "    default: break;\n    }\n";
-        }
-        s += "}\n";
-    }
-    // component sp of v_jb
-    s += "__device__ __forceinline__ int jit_dv(int jb, int sp)\n{\n    int v = 0;\n";
-    if (sel_dv) {
-        for (int j = 0; j < M; ++j)
-            for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e)
-                emit(s, "    v += (jb == %d && sp == %d) ? %d : 0;\n", j, st_species(net->h_st[e]), st_delta(net->h_st[e]));
-    } else {
-        s += "    switch (jb) {\n";
-        for (int j = 0; j < M; ++j) {
-            emit(s, "    case %d:\n", j);
-            for (int e = net->h_rx[j].z; e < net->h_rx[j].w; ++e)
-                emit(s, "        if (sp == %d) v += %d;\n", st_species(net->h_st[e]), st_delta(net->h_st[e]));
-            s += "        break;\n";
-        }
-        s += "    default: break;\n    }\n";
-    }
-    s += "    return v;\n}\n";
     // w_j = v_j . lambda, summed over the entries in table order from zero
     s += "__device__ __forceinline__ void jit_w(const float (&lam)[JN], float (&w)[JM])\n{\n";
     for (int j = 0; j < M; ++j) {
@@ -171,22 +141,53 @@ std::string jit_source(const ssa_network *net)
         emit(s, "        w[%d] = v;\n    }\n", j);
     }
     s += "}\n";
-    // state adjoint of every reaction, in order
-    s += "__device__ __forceinline__ void jit_state_adj(const int (&X)[JN], const float (&a)[JM], const float (&h)[JM], "
-         "const float (&psi)[JM], const float (&ctau)[JM], float (&lam)[JN])\n{\n";
+    // State adjoint from the per-reaction adjoints g_j = psi_j + dL/da0 a_j: a_j is proportional to the count of each
+    // plain reactant, so its species receive g_j / X; a homodimer's receives g_j (X - 1/2) / h; where a reactant is
+    // absent (a_j = 0) only the waiting-time path remains, dL/da0 k_j dh_j/dX. The coefficients of a state serve every
+    // temperature: rx[s] = 1/X_s or 0, dz[s] = the sum of k_j dh_j/dX over the reactions of an absent species,
+    // ch[j], cz[j] = the same two for homodimers.
+    s += "struct JitCoef {\n    float rx[JN], dz[JN], ch[JM], cz[JM];\n};\n"
+         "__device__ __forceinline__ void jit_coef(const int (&X)[JN], const float (&k)[JM], const float (&a)[JM], "
+         "const float (&h)[JM], JitCoef &c)\n{\n";
+    for (int sp = 0; sp < N; ++sp) {
+        std::string absent;
+        for (int j = 0; j < M; ++j) {
+            const int4 r = net->h_rx[j];
+            if (r.x == r.y || (r.x != sp && r.y != sp)) continue;
+            const int other = r.x == sp ? r.y : r.x;
+            absent += absent.empty() ? "" : " + ";
+            absent += "k[" + std::to_string(j) + "]";
+            if (other >= 0) absent += " * __int2float_rn(X[" + std::to_string(other) + "])";
+        }
+        if (absent.empty()) continue;
+        emit(s, "    c.rx[%d] = X[%d] > 0 ? __fdividef(1.0f, __int2float_rn(X[%d])) : 0.0f;\n", sp, sp, sp);
+        s += "    c.dz[" + std::to_string(sp) + "] = X[" + std::to_string(sp) + "] > 0 ? 0.0f : " + absent + ";\n";
+    }
     for (int j = 0; j < M; ++j) {
         const int4 r = net->h_rx[j];
-        if (r.x < 0) continue;
-        if (r.y < 0) {
-            emit(s, "    lam[%d] += sadj_first(int2f(X[%d]), a[%d], psi[%d], ctau[%d]);\n", r.x, r.x, j, j, j);
-        } else if (r.y == r.x) {
-            emit(s, "    lam[%d] += sadj_homodimer(int2f(X[%d]), a[%d], h[%d], psi[%d], ctau[%d]);\n", r.x, r.x, j, j,
-                 j, j);
-        } else {
-            emit(s, "    {\n        const float x1 = int2f(X[%d]), x2 = int2f(X[%d]);\n", r.x, r.y);
-            emit(s, "        lam[%d] += sadj_hetero(x1, x2, a[%d], psi[%d], ctau[%d]);\n", r.x, j, j, j);
-            emit(s, "        lam[%d] += sadj_hetero(x2, x1, a[%d], psi[%d], ctau[%d]);\n    }\n", r.y, j, j, j);
+        if (r.x < 0 || r.x != r.y) continue;
+        emit(s, "    {\n        const float d = __int2float_rn(X[%d]) - 0.5f;\n", r.x);
+        emit(s, "        c.ch[%d] = a[%d] > 0.0f ? __fdividef(d, h[%d]) : 0.0f;\n", j, j, j);
+        emit(s, "        c.cz[%d] = a[%d] > 0.0f ? 0.0f : k[%d] * d;\n    }\n", j, j, j);
+    }
+    s += "}\n__device__ __forceinline__ void jit_state_adj(const JitCoef &c, const float (&g)[JM], float dLda0, "
+         "float (&lam)[JN])\n{\n";
+    for (int sp = 0; sp < N; ++sp) {
+        std::string sum;
+        for (int j = 0; j < M; ++j) {
+            const int4 r = net->h_rx[j];
+            if (r.x == r.y || (r.x != sp && r.y != sp)) continue;
+            sum += (sum.empty() ? "g[" : " + g[") + std::to_string(j) + "]";
         }
+        if (!sum.empty()) {
+            const std::string at = std::to_string(sp);
+            s += "    lam[" + at + "] += fmaf(c.rx[" + at + "], " + sum + ", dLda0 * c.dz[" + at + "]);\n";
+        }
+    }
+    for (int j = 0; j < M; ++j) {
+        const int4 r = net->h_rx[j];
+        if (r.x < 0 || r.x != r.y) continue;
+        emit(s, "    lam[%d] += fmaf(c.ch[%d], g[%d], dLda0 * c.cz[%d]);\n", r.x, j, j, j);
     }
     s += "}\n";
     // soft forward (Eq. 4): propensities of the real-valued state (negative factors clipped to 0), the

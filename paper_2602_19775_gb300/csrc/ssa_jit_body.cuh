@@ -3,12 +3,13 @@
 //
 // This file is compiled by NVRTC, not by nvcc: the library prepends a generated prologue that
 // defines JN (species), JM (reactions) and the network hooks
-//     jit_props(X, k, a, h)       h_j(X) and a_j = k_j h_j for every reaction, in reaction order
-//     jit_check(X, jb)            status of applying v_jb to X (negative count / overflow)
-//     jit_apply(X, jb), jit_unapply(X, jb)
-//     jit_dv(jb, sp)              component sp of v_jb
+//     jit_props(X, k, a, h)       h_j(X) and a_j = k_j h_j for every reaction, in reaction order; returns whether a
+//                                 count is 2^23 or more
+//     jit_check(X, jb)            status of applying v_jb to X (negative count / overflow); kJitSafe: needed only
+//                                 where a count is that large
+//     jit_changes                 v_j as int8 by species, JW words a reaction
 //     jit_w(lam, w)               w_j = v_j . lambda for every reaction
-//     jit_state_adj(X, a, h, psi, ctau, lam)   the state adjoint of every reaction, in order
+//     jit_coef(X, k, a, h, c), jit_state_adj(c, g, dLda0, lam)   the state adjoint from the per-reaction adjoints
 // with the reactant indices and stoichiometry written into the code as constants. Counts and the
 // state adjoint then live in registers and every table lookup disappears. The arithmetic is the
 // generic thread kernels' (same helpers from ssa_device.cuh, same order), so a specialised run
@@ -24,6 +25,99 @@ __device__ __forceinline__ int jit_xsel(const int (&X)[JN], int sp)
 #pragma unroll
     for (int s = 0; s < JN; ++s) v = (s == sp) ? X[s] : v;
     return v;
+}
+
+// v_jb from the table in shared memory (s_chg, one row of kJitRow words a reaction): X += sign v_jb, and a component
+constexpr int kJitRow = JW <= 1 ? 1 : JW <= 2 ? 2 : (JW + 3) / 4 * 4;
+#define SSA_JIT_CHANGES()                                                                                 \
+    __shared__ __align__(16) int s_chg[JM * kJitRow];                                                     \
+    for (int q = threadIdx.x; q < JM * JW; q += blockDim.x) s_chg[q / JW * kJitRow + q % JW] = jit_changes[q]; \
+    __syncthreads()
+template <int SIGN>
+__device__ __forceinline__ void jit_move(int (&X)[JN], const int *s_chg, int jb)
+{
+    int w[kJitRow];
+    if constexpr (kJitRow == 1) {
+        w[0] = s_chg[jb];
+    } else if constexpr (kJitRow == 2) {
+        const int2 v = reinterpret_cast<const int2 *>(s_chg)[jb];
+        w[0] = v.x;
+        w[1] = v.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < kJitRow / 4; ++q) {
+            const int4 v = reinterpret_cast<const int4 *>(s_chg)[jb * (kJitRow / 4) + q];
+            w[4 * q] = v.x;
+            w[4 * q + 1] = v.y;
+            w[4 * q + 2] = v.z;
+            w[4 * q + 3] = v.w;
+        }
+    }
+#pragma unroll
+    for (int s = 0; s < JN; ++s) X[s] = __dp4a(w[s >> 2], (SIGN > 0 ? 0x01 : 0xff) << (8 * (s & 3)), X[s]);
+}
+__device__ __forceinline__ int jit_dv(const int *s_chg, int jb, int sp)
+{
+    return reinterpret_cast<const signed char *>(s_chg)[jb * (4 * kJitRow) + sp];
+}
+
+// ---------------------------------------------------------------------------------------------
+// The Gumbel-max choice without its logarithms. With L_j = -log2 u_j the race argmax a_j / L_j has the bounds
+// U_j = a_j / (L_j (1 - 2^-21) - 2^-21) from the hardware log2 (absolute error 2^-22 on (1/2, 1), relative 2^-22 below)
+// and one approximate reciprocal. Where the second largest bound stays below the leader's own lower bound, with a
+// margin above every rounding here and in the exact comparison, the leader wins the race as the binary32 comparisons
+// of E decide it; else (about one step in 10^4) the race is run on the variates themselves. Per reaction 14 issue slots
+// instead of 34.
+// ---------------------------------------------------------------------------------------------
+// E_0 and the factors 1 / (L_j (1 - 2^-21) - 2^-21) of one step
+__device__ __forceinline__ void jit_noise(float &E0, float (&c)[JM], uint32_t k, uint32_t c2, uint32_t c3, uint32_t key0,
+                                          uint32_t key1)
+{
+#pragma unroll
+    for (int b = 0; b < (JM + 4) / 4; ++b) {
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)b, k, c2, c3), key0, key1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int j = 4 * b + q - 1;
+            if (j >= JM) continue;
+            const float u = u01(word_of(r, q));
+            if (j < 0) E0 = neg_log_unit(u);
+            else c[j < 0 ? 0 : j] = rcp_approx(fmaxf(fmaf(lg2_approx(u), -0x1.fffff0p-1f, -0x1p-21f), 0x1p-26f));
+        }
+    }
+}
+
+struct JitRates {
+    float a[JM];
+};
+// the race itself, with the accurate variates; -1: no positive key
+__device__ __noinline__ int jit_race_exact(JitRates r, uint32_t k, uint32_t c2, uint32_t c3, uint32_t key0, uint32_t key1)
+{
+    float E[JM + 1];
+    step_noise<JM + 1>(E, k, c2, c3, key0, key1);
+    float ab = 0.0f, Eb = 1.0f;
+    int jb = -1;
+#pragma unroll
+    for (int j = 0; j < JM; ++j) race(r.a[j], E[j + 1], j, ab, Eb, jb);
+    return jb;
+}
+
+// the leader of the bounds; returns whether it is certain (a0: the step's total rate)
+__device__ __forceinline__ bool jit_leader(const float (&a)[JM], const float (&c)[JM], float a0, int &jb)
+{
+    float m1 = 0.0f, m2 = 0.0f, a1 = 1.0f;
+    jb = 0;
+#pragma unroll
+    for (int j = 0; j < JM; ++j) {
+        const float U = a[j] * c[j];
+        const bool lead = U > m1;
+        m2 = fmaxf(m2, fminf(m1, U));
+        jb = lead ? j : jb;
+        a1 = lead ? a[j] : a1;
+        m1 = fmaxf(m1, U);
+    }
+    // 1/lower bound = (L (1 + 2^-21) + 2^-21)/a <= (1 + 2^-18)/m1 + 2^-20/a1
+    return m2 * fmaf(m1 * rcp_approx(a1), 0x1p-20f, 1.0f + 0x1p-16f) < m1 && a0 > 0x1p-90f && a0 < 0x1p90f;
 }
 
 __device__ __forceinline__ void jit_lam_add(float (&lam)[JN], int sp, float v)
@@ -173,6 +267,7 @@ template <int READOUT, bool RECORD>
 __device__ __forceinline__ void jit_fwd(const FwdParams &p)
 {
     __shared__ __align__(16) uint32_t s_stage[kJitFwdBlock * kStageWords];
+    SSA_JIT_CHANGES();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.n_traj) return;
     const int64_t n = p.n_traj;
@@ -200,13 +295,15 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     int k = 0, draws = 0;
     int ck_left = p.K, ck_row = 0;
     uint32_t e0 = 0, e1 = 0, e2 = 0, e3 = 0;
-    constexpr int NQ = JM + 1;
-    float E[NQ], En[NQ];
-    step_noise<NQ>(E, 0u, c2, c3, key0, key1);
+    const int max_steps = (int)p.max_steps;  // at most 2^31 - 1
+    float E0, E0n, c[JM], cn[JM];
+    jit_noise(E0, c, 0u, c2, c3, key0, key1);
     float bacc[kBinMaxObs];
     SSA_JIT_BIN_RUNS(READOUT);
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
+    const bool few = p.n_obs <= kBinMaxObs;  // their species in registers
+    auto species = [&](int q) { return few ? (q == 0 ? osp[0] : q == 1 ? osp[1] : q == 2 ? osp[2] : osp[3]) : p.obs_sp[q]; };
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
     const bool staged = READOUT != SSA_READOUT_BIN && p.n_obs >= 1 && p.n_obs <= 4 && blockDim.x <= kJitFwdBlock;
     SampleStage stg{s_stage + threadIdx.x * kStageWords, static_cast<uint32_t *>(p.obs_out), i * p.S * p.n_obs,
@@ -214,26 +311,28 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
 
     while (!bad_input) {
         if (staged) stage_warp_flush(stg, s_stage);
-        if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
-        step_noise<NQ>(En, (uint32_t)(k + 1), c2, c3, key0, key1);  // next step, state-independent
+        if (k >= max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
+        jit_noise(E0n, cn, (uint32_t)(k + 1), c2, c3, key0, key1);  // next step, state-independent
         float a[JM], h[JM];
-        jit_props(X, kr, a, h);
-        float a0 = 0.0f, ab = 0.0f, Eb = 1.0f;
-        int jb = -1;
-        const float E0 = E[0];
+        const bool big = jit_props(X, kr, a, h);
+        float a0 = 0.0f;
 #pragma unroll
-        for (int j = 0; j < JM; ++j) {
-            a0 = __fadd_rn(a0, a[j]);
-            race(a[j], E[j + 1], j, ab, Eb, jb);
+        for (int j = 0; j < JM; ++j) a0 = __fadd_rn(a0, a[j]);
+        int jb;
+        if (!jit_leader(a, c, a0, jb)) {
+            if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
+            if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
+            JitRates r;
+#pragma unroll
+            for (int j = 0; j < JM; ++j) r.a[j] = a[j];
+            jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
+            if (jb < 0) { status = SSA_TRAJ_BAD_RATE; break; }
         }
-        if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
-        if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
-        if (jb < 0) { status = SSA_TRAJ_BAD_RATE; break; }
         const float tau = waiting_time(E0, a0);
         const double t_next = t + f2d_pos(tau);
         const bool slow = gt_nonneg(t_next, thr);
         const bool cross = slow && gt_nonneg(t_next, p.t_end);
-        if (!cross) status = jit_check(X, jb);
+        if ((big || !kJitSafe) && !cross) status = jit_check(X, jb);
         if (RECORD) {
             e0 = __funnelshift_r(e0, e1, 16);
             e1 = __funnelshift_r(e1, e2, 16);
@@ -248,19 +347,19 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
             if constexpr (READOUT == SSA_READOUT_BIN) {
                 s = bin_edges<RECORD>(p, i, s, t, t_next, k, bacc, xobs, bruns);
             } else {
-                while (s < p.S && gt_nonneg(t_next, p.ts[s])) {
+                while (s < p.S && gt_nonneg(t_next, thr)) {
                     if (READOUT == SSA_READOUT_HOLD) {
                         if (staged) {
-                            stage_put(stg, s, [&](int c) { return (uint32_t)jit_xsel(X, p.obs_sp[c]); });
+                            stage_put(stg, s, [&](int c) { return (uint32_t)jit_xsel(X, species(c)); });
                         } else {
                             int *o = static_cast<int *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                             for (int c = 0; c < p.n_obs; ++c) o[c] = jit_xsel(X, p.obs_sp[c]);
                         }
                     } else {
-                        const float alpha = __fdiv_rn(d2f_nonneg(p.ts[s] - t), tau);
+                        const float alpha = __fdiv_rn(d2f_nonneg(thr - t), tau);
                         auto lin = [&](int c) {
-                            const int sp = p.obs_sp[c];
-                            return __fmaf_rn(alpha, (float)jit_dv(jb, sp), (float)jit_xsel(X, sp));
+                            const int sp = species(c);
+                            return __fmaf_rn(alpha, (float)jit_dv(s_chg, jb, sp), (float)jit_xsel(X, sp));
                         };
                         if (staged) {
                             stage_put(stg, s, [&](int c) { return __float_as_uint(lin(c)); });
@@ -272,16 +371,17 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
                     }
                     if (RECORD) p.brk_k[(int64_t)s * n + i] = k;
                     ++s;
+                    thr = s < p.S ? p.ts[s] : p.t_end;  // the next sample time
                 }
             }
             if (READOUT == SSA_READOUT_BIN && !cross && s > s_first)
                 bin_accumulate(bacc, xobs, p.n_obs, d2f_nonneg(t_next - p.ts[s - 1]));
-            thr = s < p.S ? p.ts[s] : p.t_end;
+            if (READOUT == SSA_READOUT_BIN) thr = s < p.S ? p.ts[s] : p.t_end;
             if (cross) break;  // the crossing draw is made but not applied
         } else if (READOUT == SSA_READOUT_BIN) {
             bin_accumulate(bacc, xobs, p.n_obs, tau);
         }
-        jit_apply(X, jb);
+        jit_move<1>(X, s_chg, jb);
         t = t_next;
         ++k;
         if (RECORD && --ck_left == 0) {
@@ -291,8 +391,9 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
 #pragma unroll
             for (int sp = 0; sp < JN; ++sp) ck[(int64_t)sp * n] = X[sp];
         }
+        E0 = E0n;
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) E[q] = En[q];
+        for (int j = 0; j < JM; ++j) c[j] = cn[j];
     }
     if constexpr (READOUT == SSA_READOUT_BIN) bin_tail<RECORD>(p, i, s, t, k, bacc, xobs, bad_obs, bruns);
     for (; READOUT != SSA_READOUT_BIN && s < p.S; ++s) {
@@ -342,6 +443,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
 template <int READOUT>
 __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
 {
+    SSA_JIT_CHANGES();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= p.n_traj) return;
     float kr[JM];
@@ -375,7 +477,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
         if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
         r = philox4x32_10(make_uint4(0u, (uint32_t)(k + 1), c2, c3), key0, key1);  // next step
         float a[JM], h[JM];
-        jit_props(X, kr, a, h);
+        const bool big = jit_props(X, kr, a, h);
         float a0 = 0.0f;
 #pragma unroll
         for (int j = 0; j < JM; ++j) a0 = __fadd_rn(a0, a[j]);
@@ -398,7 +500,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
         const double t_next = t + f2d_pos(tau);
         const bool slow = gt_nonneg(t_next, thr);
         const bool cross = slow && gt_nonneg(t_next, p.t_end);
-        if (!cross) status = jit_check(X, jb);
+        if ((big || !kJitSafe) && !cross) status = jit_check(X, jb);
         draws = k + 1;
         if (status != SSA_TRAJ_OK) break;
         if (slow) {
@@ -415,7 +517,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
                         float *o = static_cast<float *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                         for (int c = 0; c < p.n_obs; ++c) {
                             const int sp = p.obs_sp[c];
-                            o[c] = __fmaf_rn(alpha, (float)jit_dv(jb, sp), (float)jit_xsel(X, sp));
+                            o[c] = __fmaf_rn(alpha, (float)jit_dv(s_chg, jb, sp), (float)jit_xsel(X, sp));
                         }
                     }
                     ++s;
@@ -428,7 +530,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
         } else if (READOUT == SSA_READOUT_BIN) {
             bin_accumulate(bacc, xobs, p.n_obs, tau);
         }
-        jit_apply(X, jb);
+        jit_move<1>(X, s_chg, jb);
         t = t_next;
         ++k;
         E0 = neg_log_unit(u01(r.x));
@@ -527,7 +629,7 @@ __device__ __forceinline__ void jit_bin_chunk_sums(const AdjParams &p, int64_t i
 // 2^-sc. The trajectory's result is dAr 2^sc. With sc = 0 the arithmetic is the plain walk's bit for bit.
 template <int READOUT, bool WIDE = false, int NT = 1>
 __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&kr)[JM], const int64_t i, const int st,
-                                             float (&dAr)[NT][JM], int &sc, const BinChunks chunks)
+                                             float (&dAr)[NT][JM], int &sc, const BinChunks chunks, const int *s_chg)
 {
     static_assert(!WIDE || NT == 1, "the wide-range walk takes one temperature");
     sc = 0;
@@ -588,10 +690,12 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
 #pragma unroll
     for (int s = 0; s < JN; ++s) ckv[s] = p.ckpt[((int64_t)ck_row * JN + s) * n + i];
 
+    // E_0 and 1/E_{1+j} of a step
     constexpr int NQ = JM + 1;
     float E[NQ], En[NQ];
     const bool draw_last = st == SSA_TRAJ_OK;
-    step_noise<NQ>(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
+    step_noise_inv<NQ>(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
+    const bool few = p.n_obs <= kBinMaxObs;  // their species in registers
 
     // BIN readout (NT = 1): gq = g of the bin that contains t_{k+1}, xo = X_{k+1} at the observables
     constexpr bool kBin = READOUT == SSA_READOUT_BIN;
@@ -599,7 +703,8 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
     float gq[kBinMaxObs], gk[kBinMaxObs];
     int osp[kBinMaxObs], xo[kBinMaxObs];
 #pragma unroll
-    for (int c = 0; c < kBinMaxObs; ++c) osp[c] = (kBin && c < p.n_obs) ? p.obs_sp[c] : 0;
+    for (int c = 0; c < kBinMaxObs; ++c) osp[c] = c < p.n_obs ? p.obs_sp[c] : 0;
+    auto species = [&](int q) { return few ? (q == 0 ? osp[0] : q == 1 ? osp[1] : q == 2 ? osp[2] : osp[3]) : p.obs_sp[q]; };
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
     auto addx = [&](int c, float v) { jit_lam_add(lam[0], osp[c], v); };
     if (kBin) {
@@ -633,21 +738,38 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
         float tau_k = 0.0f;
         if (draw) {
             const int jk = event_at(k);
-            if (k > 0) step_noise<NQ>(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
-            float a[JM], h[JM], lr[JM];
+            if (k > 0) step_noise_inv<NQ>(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
+            float a[JM], h[JM], key[JM];
             jit_props(X, kr, a, h);
-            float a0 = 0.0f, ab = 0.0f, Eb = 1.0f, lmax = -CUDART_INF_F;
+            // pass 1: a0 and the race's keys a_j / E_j, with the two largest
+            float a0 = 0.0f, m1 = 0.0f, m2 = 0.0f;
             int jb = -1;
             const float E0 = E[0];
-            // pass 1: the forward's a0 and race, bit for bit; log2 keys
+#pragma unroll
+            for (int j = 0; j < JM; ++j) a0 = __fadd_rn(a0, a[j]);
+            const float sc_key = key_scale(a0);
 #pragma unroll
             for (int j = 0; j < JM; ++j) {
-                a0 = __fadd_rn(a0, a[j]);
-                race(a[j], E[j + 1], j, ab, Eb, jb);
-                lr[j] = a[j] > 0.0f ? __log2f(a[j]) - __log2f(E[j + 1]) : -CUDART_INF_F;
-                lmax = fmaxf(lmax, lr[j]);
+                key[j] = (a[j] * sc_key) * E[j + 1];
+                jb = key[j] > m1 ? j : jb;
+                m2 = fmaxf(m2, fminf(m1, key[j]));
+                m1 = fmaxf(m1, key[j]);
+            }
+            // the recorded reaction won the race if its key is the largest by more than the keys' error; near ties are
+            // raced again
+            if (m2 >= m1 * (1.0f - kTieMargin)) {
+                JitRates r;
+#pragma unroll
+                for (int j = 0; j < JM; ++j) r.a[j] = a[j];
+                jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
             }
             mism += (jb != jk);
+            const float inv_m1 = m1 > 0.0f ? __fdividef(1.0f, m1) : 0.0f;
+            float lg2_key[JM];
+#pragma unroll
+            for (int j = 0; j < JM; ++j) lg2_key[j] = lg2_approx(key[j] * inv_m1);
+            JitCoef coef;
+            jit_coef(X, kr, a, h, coef);
             // The walk's divisions by a0 (tau = E0/a0 and d tau/d a0 = -tau/a0) take one approximate
             // reciprocal per step, accurate to 2 ulp where a0 s lies in [2^-126, 2^126]: the power of two s
             // puts it there. They only enter the gradient (the clock is the forward's), and without the IEEE
@@ -667,13 +789,13 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
                     float c = 0.0f;
                     for (int o = 0; o < p.n_obs; ++o) {
                         const float g = WIDE ? gl[(int64_t)s * p.n_obs + o] * inj : gl[(int64_t)s * p.n_obs + o];
-                        const int sp = p.obs_sp[o];
+                        const int sp = species(o);
                         if (WIDE) jit_lam_add2(lam[0], lam_lo, sp, alpha * g);
                         else {
 #pragma unroll
                             for (int t = 0; t < NT; ++t) jit_lam_add(lam[t], sp, alpha * g);
                         }
-                        c += g * (float)jit_dv(jk, sp);
+                        c += g * (float)jit_dv(s_chg, jk, sp);
                     }
                     const float c_tau = __fdividef(c, tau);
                     dt_dir -= c_tau;
@@ -684,37 +806,38 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
             for (int t = 0; t < NT; ++t) {
                 const float dtau = WIDE ? (mu[t] + dtau_dir) + mu_lo : mu[t] + dtau_dir;
                 const float dLda0 = ((-dtau * tau) * sc_a0) * ra0;
-                // pass 2: soft-sample weights y~_j ~ exp2((l_j - l_max)/T) and W = sum y~ w
+                // pass 2: soft-sample weights y~_j ~ (key_j / largest)^(1/T) and W = sum y~ w
                 float wr[JM], qr[JM];
                 jit_w(lam[t], wr);
                 float Z = 0.0f, Wq = 0.0f;
 #pragma unroll
                 for (int j = 0; j < JM; ++j) {
-                    const float q = lr[j] == -CUDART_INF_F ? 0.0f : exp2f((lr[j] - lmax) * invT[t]);
+                    const float q = ex2_approx(lg2_key[j] * invT[t]);
                     qr[j] = q;
                     Z += q;
-                    Wq += q * wr[j];
+                    Wq += q > 0.0f ? q * wr[j] : 0.0f;
                 }
-                const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ;
-                // pass 3: per-reaction adjoints, then the state adjoint of every reaction in order
-                float psi[JM], ctau[JM];
+                const float invZ = __fdividef(1.0f, Z), Wbar = Wq * invZ, scale = invZ * invT[t];
+                // pass 3: per-reaction adjoints g_j = psi_j + dL/da0 a_j, then the state adjoint
+                float g[JM];
 #pragma unroll
                 for (int j = 0; j < JM; ++j) {
-                    psi[j] = qr[j] > 0.0f ? qr[j] * invZ * (wr[j] - Wbar) * invT[t] : 0.0f;
-                    dAr[t][j] += psi[j] + dLda0 * a[j];
-                    ctau[j] = dLda0 * kr[j];
+                    float psi = qr[j] * scale * (wr[j] - Wbar);
+                    psi = qr[j] > 0.0f ? psi : 0.0f;
+                    g[j] = __fmaf_rn(dLda0, a[j], psi);
+                    dAr[t][j] += g[j];
                 }
                 if (WIDE) {
                     // this step's state-adjoint increment in binary32, then added to the compensated sum
                     float dl[JN];
 #pragma unroll
                     for (int s = 0; s < JN; ++s) dl[s] = 0.0f;
-                    jit_state_adj(X, a, h, psi, ctau, dl);
+                    jit_state_adj(coef, g, dLda0, dl);
 #pragma unroll
                     for (int s = 0; s < JN; ++s) acc2(lam[0][s], lam_lo[s], dl[s]);
                     acc2(mu[0], mu_lo, dt_dir);  // t_{k+1} = t_k + tau_k
                 } else {
-                    jit_state_adj(X, a, h, psi, ctau, lam[t]);
+                    jit_state_adj(coef, g, dLda0, lam[t]);
                     mu[t] += dt_dir;  // t_{k+1} = t_k + tau_k
                 }
             }
@@ -736,10 +859,10 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
                 }
                 for (int o = 0; o < p.n_obs; ++o) {
                     const float g = WIDE ? gl[(int64_t)s * p.n_obs + o] * inj : gl[(int64_t)s * p.n_obs + o];
-                    if (WIDE) jit_lam_add2(lam[0], lam_lo, p.obs_sp[o], coef * g);
+                    if (WIDE) jit_lam_add2(lam[0], lam_lo, species(o), coef * g);
                     else {
 #pragma unroll
-                        for (int t = 0; t < NT; ++t) jit_lam_add(lam[t], p.obs_sp[o], coef * g);
+                        for (int t = 0; t < NT; ++t) jit_lam_add(lam[t], species(o), coef * g);
                     }
                 }
             }
@@ -782,7 +905,7 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
             }
         }
         --ck_off;
-        if (k > 0) jit_unapply(X, event_at(k - 1));
+        if (k > 0) jit_move<-1>(X, s_chg, event_at(k - 1));
         if (draw) {
 #pragma unroll
             for (int q = 0; q < NQ; ++q) E[q] = En[q];
@@ -1100,6 +1223,7 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
 {
     extern __shared__ float s_dA[];  // [NT][JM][blockDim.x] (WIDE: binary64)
     __shared__ int s_len[256], s_perm[256];
+    SSA_JIT_CHANGES();
     const int B = blockDim.x, tid = threadIdx.x;
     const int64_t n = p.n_traj;
     // the threads of the block take its trajectories longest first, so that each warp walks trajectories
@@ -1138,7 +1262,7 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
     }
     if (active) {
         if constexpr (SOFT) jit_adj_soft_traj<READOUT>(p, kr, i, st, dAr[0], chunks);
-        else jit_adj_traj<READOUT, WIDE, NT>(p, kr, i, st, dAr, sc, chunks);
+        else jit_adj_traj<READOUT, WIDE, NT>(p, kr, i, st, dAr, sc, chunks, s_chg);
     }
     const int warp = tid >> 5, lane = tid & 31, nwarps = B >> 5;
     if constexpr (WIDE) {

@@ -825,15 +825,11 @@ __device__ __forceinline__ void warp_soft_adj_body(const AdjParams &p, const int
     if (lane == 0 && mism) atomicAdd(p.mismatch, mism);
 }
 
-// Two keys within this of each other, relatively, count as a possible tie (a key is a few units in the last place
-// off, and so is the comparison of products that decides the race).
-constexpr float kTieMargin = 0x1p-15f;
-
 // The keys of a step whose a0 lies where a_j / E_j could leave the binary32 range, scaled by a power of two (all
 // that follows uses ratios of keys); returns the largest.
 static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *ad, int k, WarpNoise z, float a0, float *rj)
 {
-    const float sc = a0 > 1.0f ? 0x1p-60f : 0x1p100f;
+    const float sc = key_scale(a0);
     const int lane = threadIdx.x & 31;
     float rmax = 0.0f;
     for (int c = 0; c < rounds; ++c) {
