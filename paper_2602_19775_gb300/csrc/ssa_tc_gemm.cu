@@ -313,12 +313,11 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(const void *p)
 }
 
 
-// split K: with Dpart given, the CTAs of blockIdx.z = s take the 64-wide K blocks [s per, (s + 1) per) and
-// write their sums in binary64 to Dpart [gridDim.z][M][N] (no bias); tc_splitk_reduce_kernel adds them
+// split K: the CTAs of blockIdx.z = s take the 64-wide K blocks [s per, (s + 1) per) and write their sums in binary64
+// to Dpart [gridDim.z][M][N] (no bias); tc_splitk_reduce_kernel adds them
 __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_constant__ CUtensorMap mapA,
                                                                 const __grid_constant__ CUtensorMap mapB, int M,
-                                                                int N, int K, const float *bias, float *D, int ldd,
-                                                                double *Dpart, int chunks_per, int *err)
+                                                                int N, int K, double *Dpart, int chunks_per, int *err)
 {
     extern __shared__ __align__(1024) unsigned char sw_raw[];
     // the swizzled tiles need 1,024-byte alignment
@@ -331,8 +330,8 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
     int *s_ok = reinterpret_cast<int *>(s_tmem + 1);
     const int m0 = blockIdx.x * 128, n0 = blockIdx.y * kSwBN;
     const int total_kb = (K + 63) / 64;
-    const int kb0 = Dpart ? (int)blockIdx.z * chunks_per : 0;
-    const int nkb = Dpart ? max(0, min(chunks_per, total_kb - kb0)) : total_kb;
+    const int kb0 = (int)blockIdx.z * chunks_per;
+    const int nkb = max(0, min(chunks_per, total_kb - kb0));
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(s_tmem)),
@@ -402,33 +401,14 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
             float v[16];
             tmem_ld16(lane_base + (uint32_t)(16 * c16), v);
             const int col0 = n0 + 16 * c16;
-            if (Dpart) {
-                if (row < M) {
-                    double *dp = Dpart + ((int64_t)blockIdx.z * M + row) * N + col0;
-                    if (col0 + 16 <= N && (N % 2) == 0) {
+            if (row < M) {
+                double *dp = Dpart + ((int64_t)blockIdx.z * M + row) * N + col0;
+                if (col0 + 16 <= N && (N % 2) == 0) {
 #pragma unroll
-                        for (int i = 0; i < 16; i += 2)
-                            *reinterpret_cast<double2 *>(dp + i) = make_double2((double)v[i], (double)v[i + 1]);
-                    } else {
-                        for (int i = 0; i < 16 && col0 + i < N; ++i) dp[i] = (double)v[i];
-                    }
-                }
-            } else if (row < M) {
-                float *dst = D + (int64_t)row * ldd + col0;
-                if (col0 + 16 <= N && (ldd % 4) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0) {
-#pragma unroll
-                    for (int i = 0; i < 16; i += 4) {
-                        float4 o = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                        if (bias) {
-                            o.x += bias[col0 + i];
-                            o.y += bias[col0 + i + 1];
-                            o.z += bias[col0 + i + 2];
-                            o.w += bias[col0 + i + 3];
-                        }
-                        *reinterpret_cast<float4 *>(dst + i) = o;
-                    }
+                    for (int i = 0; i < 16; i += 2)
+                        *reinterpret_cast<double2 *>(dp + i) = make_double2((double)v[i], (double)v[i + 1]);
                 } else {
-                    for (int i = 0; i < 16 && col0 + i < N; ++i) dst[i] = v[i] + (bias ? bias[col0 + i] : 0.0f);
+                    for (int i = 0; i < 16 && col0 + i < N; ++i) dp[i] = (double)v[i];
                 }
             }
         }
@@ -438,6 +418,162 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSwBN) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The same product without a split of K: one persistent CTA per SM walks the output tiles (128 x BN, m fastest) with
+// its ring of four stages never drained between tiles, and two TMEM accumulators of 256 columns, so that four
+// epilogue warps write a tile while the next one is multiplied. Warp 0 loads (TMA), warp 1 issues tcgen05.mma, warps
+// 2 to 5 read TMEM lanes 32 (warp % 4) ... and store. BN (a multiple of 16 up to 256) is the launch's: the width that
+// takes the fewest rounds of the SMs times columns (sw_tile_columns).
+// 4096 x 4096 x 4096: 126 -> 116 us (one tile per CTA, 128 x 256, the epilogue after the tile), bound by the operand
+// reads from L2 (44 KB per SM and K block of 64).
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+constexpr int kPsThreads = 192;
+__global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap mapA,
+                                                                           const __grid_constant__ CUtensorMap mapB,
+                                                                           int M, int N, int K, int BN, int tiles_m,
+                                                                           int tiles, const float *bias, float *D,
+                                                                           int ldd, int *err)
+{
+    extern __shared__ __align__(1024) unsigned char sw_raw[];
+    unsigned char *sw = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(sw_raw) + 1023) & ~(uintptr_t)1023);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    uint64_t *full = reinterpret_cast<uint64_t *>(sw + kSwStages * kSwStage);
+    uint64_t *empty = full + kSwStages;
+    uint64_t *acc_full = empty + kSwStages;  // [2]
+    uint64_t *acc_empty = acc_full + 2;      // [2], one arrival per epilogue warp
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(acc_empty + 2);
+    volatile int *s_ok = reinterpret_cast<int *>(s_tmem + 1);
+    const int nkb = (K + 63) / 64;
+
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(s_tmem)), "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    if (tid == 0) {
+        for (int b = 0; b < kSwStages; ++b) {
+            mbar_init(&full[b], 1);
+            mbar_init(&empty[b], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], 4);
+        }
+        *s_ok = 1;
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *s_tmem;
+    auto give_up = [&]() {
+        atomicOr(err, kErrTcTimeout);
+        *s_ok = 0;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int c = 0;  // K blocks loaded so far, over all tiles
+            bool ok = true;
+            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+                const int m0 = t % tiles_m * 128, n0 = t / tiles_m * BN;
+                for (int kb = 0; kb < nkb; ++kb, ++c) {
+                    const int st = c % kSwStages, round = c / kSwStages;
+                    ok = (round == 0 || mbar_wait_bounded(&empty[st], (round - 1) & 1, kWaitLimit)) && *s_ok;
+                    if (!ok) break;
+                    unsigned char *stage = sw + st * kSwStage;
+                    mbar_arrive_expect_tx(&full[st], (uint32_t)(kSwTileA + BN * 128));
+                    tma_load_2d(stage, &mapA, kb * 64, m0, &full[st]);
+                    tma_load_2d(stage + kSwTileA, &mapB, kb * 64, n0, &full[st]);
+                }
+            }
+            if (!ok) {
+                give_up();
+                // the copies in flight land before the CTA exits (each wait bounded)
+                for (int q = max(0, c - kSwStages); q < c; ++q)
+                    mbar_wait_bounded(&full[q % kSwStages], (q / kSwStages) & 1, kWaitLimit);
+            }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            int c = 0, it = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
+                const int buf = it & 1;
+                ok = (it < 2 || mbar_wait_bounded(&acc_empty[buf], ((it >> 1) - 1) & 1, kWaitLimit)) && *s_ok;
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t acc = tmem + (uint32_t)(256 * buf);
+                for (int kb = 0; kb < nkb; ++kb, ++c) {
+                    const int st = c % kSwStages;
+                    ok = mbar_wait_bounded(&full[st], (c / kSwStages) & 1, kWaitLimit) && *s_ok;
+                    if (!ok) break;
+                    tc_fence_after();
+                    const unsigned char *stage = sw + st * kSwStage;
+                    const uint64_t ad = smem_desc_sw128(stage), bd = smem_desc_sw128(stage + kSwTileA);
+#pragma unroll
+                    for (int kk = 0; kk < 4; ++kk)
+                        tc_mma(acc, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
+                    tc_commit(&empty[st]);  // the stage is free once these MMAs have read it
+                }
+                if (ok) tc_commit(&acc_full[buf]);
+            }
+            if (!ok) give_up();
+        }
+    } else {
+        int it = 0;
+        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
+            const int buf = it & 1, quad = warp & 3;
+            bool ok = mbar_wait_bounded(&acc_full[buf], (it >> 1) & 1, kWaitLimit);
+            if (!ok && lane == 0) give_up();
+            ok = __all_sync(0xffffffffu, ok && *s_ok);
+            if (!ok) break;
+            tc_fence_after();
+            const int row = t % tiles_m * 128 + 32 * quad + lane, n0 = t / tiles_m * BN;
+            const uint32_t base = tmem + (uint32_t)(256 * buf) + ((uint32_t)(32 * quad) << 16);
+            const bool wide = (ldd % 4) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
+            for (int c16 = 0; c16 < BN / 16; ++c16) {
+                float v[16];
+                tmem_ld16(base + (uint32_t)(16 * c16), v);
+                const int col0 = n0 + 16 * c16;
+                if (row < M && col0 < N) {
+                    float *dst = D + (int64_t)row * ldd + col0;
+                    if (col0 + 16 <= N && wide) {
+#pragma unroll
+                        for (int i = 0; i < 16; i += 4) {
+                            float4 o = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+                            if (bias) {
+                                o.x += bias[col0 + i];
+                                o.y += bias[col0 + i + 1];
+                                o.z += bias[col0 + i + 2];
+                                o.w += bias[col0 + i + 3];
+                            }
+                            *reinterpret_cast<float4 *>(dst + i) = o;
+                        }
+                    } else {
+                        for (int i = 0; i < 16 && col0 + i < N; ++i) dst[i] = v[i] + (bias ? bias[col0 + i] : 0.0f);
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
 
@@ -554,11 +690,32 @@ static int sw_split(int M, int N, int K, int *per)
     return (total + *per - 1) / *per;  // every split non-empty
 }
 
-static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K,
-                                        const float *bias, float *D, int ldd, double *work, int *err, cudaStream_t st)
+constexpr int kGemmSms = 152;
+
+// Columns of a tile of the persistent kernel: the multiple of 16 that takes the fewest rounds of one tile per SM times
+// the columns of a tile (16 more stand for a tile's fixed cost); ties take the wider tile. Below 128 columns the
+// instruction's time no longer falls with its width. 4096 x 4096: 224 columns, 608 tiles, exactly four rounds.
+static int sw_tile_columns(int M, int N)
+{
+    const int64_t tm = (M + 127) / 128;
+    int best = 256;
+    int64_t best_cost = INT64_MAX;
+    for (int bn = 256; bn >= 128; bn -= 16) {
+        const int64_t tiles = tm * ((N + bn - 1) / bn), cost = (tiles + kGemmSms - 1) / kGemmSms * (bn + 16);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = bn;
+        }
+    }
+    return best;
+}
+
+static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, int bn,
+                                        const float *bias, float *D, int ldd, double *work, int k_split, int per,
+                                        int *err, cudaStream_t st)
 {
     const size_t smem = (size_t)kSwStages * kSwStage + 128 + 1024;  // ring, barriers, alignment slack
-    // the attribute is set once per device and kept by the context, so calls inside a graph capture make no
+    // the attributes are set once per device and kept by the context, so calls inside a graph capture make no
     // further runtime calls (after cudaDeviceReset the launch fails with an error instead)
     static std::atomic<uint64_t> attr_set{0};
     int dev = 0;
@@ -566,17 +723,22 @@ static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap
     if (e != cudaSuccess) return e;
     if (dev >= 64 || !(attr_set.load() & (1ull << dev))) {
         e = cudaFuncSetAttribute(tc_gemm_sw128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(tc_gemm_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_set.fetch_or(1ull << dev);
     }
-    int per = (K + 63) / 64;
-    const int k_split = work ? sw_split(M, N, K, &per) : 1;
-    dim3 grid((unsigned)((M + 127) / 128), (unsigned)((N + kSwBN - 1) / kSwBN), (unsigned)k_split);
-    tc_gemm_sw128_kernel<<<grid, 128, smem, st>>>(ma, mb, M, N, K, bias, D, ldd, k_split > 1 ? work : nullptr, per,
-                                                  err);
+    const int tiles_m = (M + 127) / 128, tiles_n = (N + bn - 1) / bn;
     if (k_split > 1) {
+        dim3 grid((unsigned)tiles_m, (unsigned)tiles_n, (unsigned)k_split);
+        tc_gemm_sw128_kernel<<<grid, 128, smem, st>>>(ma, mb, M, N, K, work, per, err);
         const int64_t n = (int64_t)M * N;
         tc_splitk_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(work, k_split, M, N, bias, D, ldd);
+    } else {
+        const int64_t tiles = (int64_t)tiles_m * tiles_n;
+        if (tiles > INT32_MAX - kGemmSms) return cudaErrorInvalidValue;
+        tc_gemm_persistent_kernel<<<(unsigned)std::min<int64_t>(tiles, kGemmSms), kPsThreads, smem, st>>>(
+            ma, mb, M, N, K, bn, tiles_m, (int)tiles, bias, D, ldd, err);
     }
     return cudaGetLastError();
 }
@@ -663,9 +825,13 @@ extern "C" ssa_status ssa_bf16_gemm(const uint16_t *A, const uint16_t *B, int32_
         cudaError_t e = cudaGetLastError();
         return e == cudaSuccess ? SSA_OK : set_error(SSA_ERR_CUDA, cudaGetErrorString(e));
     }
+    // with the caller's work buffer K is split where the output tiles fill few SMs
+    int per = (K + 63) / 64;
+    const int k_split = work && work_words > 0 ? sw_split(M, N, K, &per) : 1;
+    const int bn = k_split > 1 ? kSwBN : sw_tile_columns(M, N);
     CUtensorMap ma, mb;
-    if (!tc_make_map_sw128(&ma, A, M, K, lda, 128) || !tc_make_map_sw128(&mb, B, N, K, ldb, kSwBN))
+    if (!tc_make_map_sw128(&ma, A, M, K, lda, 128) || !tc_make_map_sw128(&mb, B, N, K, ldb, bn))
         return set_error(SSA_ERR_INVALID_ARG, "tensor map encoding failed (alignment or driver entry point)");
-    cudaError_t e = tc_gemm_sw128_launch(ma, mb, M, N, K, bias, D, ldd, work_words > 0 ? work : nullptr, err_flag, st);
+    cudaError_t e = tc_gemm_sw128_launch(ma, mb, M, N, K, bn, bias, D, ldd, work, k_split, per, err_flag, st);
     return e == cudaSuccess ? SSA_OK : set_error(SSA_ERR_CUDA, cudaGetErrorString(e));
 }
