@@ -333,62 +333,78 @@ namespace {
 
 constexpr int kGrnSoftK = 8;  // float checkpoints of the soft forward every 8 steps
 
-// output propensities k_max sigma(W2 h + b2) of the relaxed state X (the warp's lanes cooperate)
+// Propensities and keys lie by word (index j + 1), as in the exact path. Per step at 784-256-10: ~1,200 warp
+// instructions; with an accurate logarithm of every variate and two accurate log2 of every key, and the outputs'
+// sigmoids evaluated one lane at a time, ~3,300.
+
+// output propensities k_max sigma(W2 h + b2) of the relaxed state X (the warp's lanes cooperate); aO: a + nh + 1
 __device__ __forceinline__ void grn_soft_outputs(const GrnParams &p, const float *s_W2, const float *s_b2,
                                                  const float *X, float *aO, int lane)
 {
     const int nh = p.n_hid, no = p.n_out;
-    for (int o = 0; o < no; ++o) {
-        float part = 0.0f;
-        for (int h = lane; h < nh; h += 32) part = __fmaf_rn(s_W2[(size_t)o * nh + h], X[h], part);
-        const float e2 = __fadd_rn(warp_sum(part), s_b2[o]);
-        if (lane == (o & 31)) aO[o] = p.k_max * sigmoid_f(e2);
+    for (int o0 = 0; o0 < no; o0 += 32) {  // up to 32 outputs, then one sigmoid per lane
+        float mine = 0.0f;
+        for (int o = o0; o < min(no, o0 + 32); ++o) {
+            float part = 0.0f;
+#pragma unroll 8
+            for (int h = lane; h < nh; h += 32) part = __fmaf_rn(s_W2[(size_t)o * nh + h], X[h], part);
+            const float sum = warp_sum(part);
+            if (lane == o - o0) mine = sum;
+        }
+        if (o0 + lane < no) aO[o0 + lane] = p.k_max * sigmoid_f(__fadd_rn(mine, s_b2[o0 + lane]));
     }
     __syncwarp();
 }
 
-// one soft step from state X at step k: propensities, keys, then the unnormalised
-// weights q_j = exp2((l_j - l_max)/T); returns a0 and sets E0 and invZ = 1/sum q
-__device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const float *s_d, const float *X, const float *aH,
-                                                  const float *aO, float *q, int k, uint32_t c2,
-                                                  uint32_t c3, uint32_t key0, uint32_t key1, int lane, float &E0,
-                                                  float &invZ)
+// one soft step at step k from the propensities a: the race's keys a_j / E_j, then the unnormalised weights
+// q_j = (key_j / largest)^(1/T) in their place; returns a0 and sets E0 and invZ = 1/sum q
+__device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const float *a, float *key, int k,
+                                                  const WarpNoise &z, int lane, float &E0, float &invZ)
 {
-    const int nh = p.n_hid, nd = p.n_dyn, M = p.M;
-    float a0p = 0.0f, lmaxp = -CUDART_INF_F, e0 = 0.0f;
-    for (int b = lane; b < p.nb; b += 32) {
-        const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, c2, c3), key0, key1);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            const int j = 4 * b + w - 1;
-            if (j < 0) { e0 = neg_log_unit(u01(r.x)); continue; }
-            if (j >= M) continue;
-            const float a = j < nh ? aH[j] : j < nd ? aO[j - nh] : __fmul_rn(s_d[j - nd], fmaxf(X[j - nd], 0.0f));
-            a0p = __fadd_rn(a0p, a);
-            const float l = a > 0.0f ? log2f(a) - log2f(neg_log_unit(u01(word_of(r, w)))) : -CUDART_INF_F;
-            q[j] = l;
-            lmaxp = fmaxf(lmaxp, l);
-        }
+    const int rounds = wide_len(p.M) >> 7;
+    const float4 *a4 = reinterpret_cast<const float4 *>(a);
+    float4 *key4 = reinterpret_cast<float4 *>(key);
+    float a0p = 0.0f, rmax = 0.0f;
+    uint32_t x0 = 0;
+    for (int c = 0; c < rounds; ++c) {
+        const int b = 32 * c + lane;
+        const uint4 r = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
+        if (c == 0) x0 = r.x;
+        const float4 av = a4[b];  // the waiting-time word's and the padded ones are 0
+        a0p = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(a0p, av.x), av.y), av.z), av.w);
+        const float4 kv = make_float4(av.x * inv_exp_of_word(r.x), av.y * inv_exp_of_word(r.y),
+                                      av.z * inv_exp_of_word(r.z), av.w * inv_exp_of_word(r.w));
+        rmax = fmaxf(rmax, fmaxf(fmaxf(kv.x, kv.y), fmaxf(kv.z, kv.w)));
+        key4[b] = kv;
     }
-    const float a0 = warp_sum(a0p), lmax = warp_max(lmaxp);
-    E0 = __shfl_sync(0xffffffffu, e0, 0);
-    __syncwarp();
+    const float a0 = warp_sum(a0p);
+    rmax = warp_max_nonneg(rmax);
+    E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
+    if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(rounds, a, k, z, a0, key);
+    const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
     float Zp = 0.0f;
-    for (int j = lane; j < M; j += 32) {
-        const float wgt = q[j] == -CUDART_INF_F ? 0.0f : exp2f((q[j] - lmax) * p.invT);
-        q[j] = wgt;
-        Zp += wgt;
+    for (int c = 0; c < rounds; ++c) {
+        const float4 kv = key4[32 * c + lane];
+        auto weight = [&](float v) { return ex2_approx(lg2_approx(v * inv_rmax) * p.invT); };
+        const float4 q = make_float4(weight(kv.x), weight(kv.y), weight(kv.z), weight(kv.w));
+        key4[32 * c + lane] = q;
+        Zp += (q.x + q.y) + (q.z + q.w);
     }
     invZ = __fdividef(1.0f, warp_sum(Zp));
     __syncwarp();
     return a0;
 }
 
-// the relaxed update X += (y~_prod - y~_deg) for every dynamic species
-__device__ __forceinline__ void grn_soft_update(const GrnParams &p, float *X, const float *q, float invZ, int lane)
+// the relaxed update X += y~_prod - y~_deg for every dynamic species, and its degradation's propensity
+__device__ __forceinline__ void grn_soft_update(const GrnParams &p, const float *s_d, float *X, float *a, const float *q,
+                                                float invZ, int lane)
 {
     const int nd = p.n_dyn;
-    for (int u = lane; u < nd; u += 32) X[u] = __fadd_rn(X[u], (q[u] - q[nd + u]) * invZ);
+    for (int u = lane; u < nd; u += 32) {
+        const float x = __fadd_rn(X[u], (q[u + 1] - q[nd + u + 1]) * invZ);
+        X[u] = x;
+        a[nd + u + 1] = __fmul_rn(s_d[u], fmaxf(x, 0.0f));
+    }
     __syncwarp();
 }
 
@@ -398,15 +414,16 @@ __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, fl
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
-    const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn, M = p.M;
-    const int ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3, nop = (no + 3) & ~3, Mq = (M + 3) & ~3;
+    const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn;
+    const int ndp = (nd + 3) & ~3, nop = (no + 3) & ~3, wide = wide_len(p.M);
     float *s_W2 = reinterpret_cast<float *>(smem);  // [no][nh]
     float *s_d = s_W2 + (size_t)no * nh;            // [nd]
     float *s_b2 = s_d + nd;                         // [no]
-    float *X = s_b2 + nop + (size_t)wib * (ndp + nhp + nop + Mq);
-    float *aH = X + ndp;   // production of the hidden genes: constant per image
-    float *aO = aH + nhp;  // production of the outputs
-    float *q = aO + nop;   // per reaction: key, then unnormalised soft weight
+    float *X = reinterpret_cast<float *>(smem + ((4 * ((size_t)no * nh + nd + nop) + 15) & ~(size_t)15)) +
+               (size_t)wib * (ndp + 2 * wide);
+    float *a = X + ndp;    // propensities by word
+    float *q = a + wide;   // keys, then unnormalised soft weights
+    float *aO = a + nh + 1;
     for (int u = threadIdx.x; u < no * nh; u += blockDim.x) s_W2[u] = p.W2f[u];
     for (int u = threadIdx.x; u < nd; u += blockDim.x) s_d[u] = p.dvec[u];
     for (int u = threadIdx.x; u < no; u += blockDim.x) s_b2[u] = p.b2[u];
@@ -418,12 +435,14 @@ __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, fl
     float *ckf = reinterpret_cast<float *>(p.ckpt);
     const float *E1 = p.E1 + (i / p.tpi) * nh;
     for (int u = lane; u < nd; u += 32) X[u] = 0.0f;
-    for (int h = lane; h < nh; h += 32) aH[h] = p.k_max * sigmoid_f(E1[h]);
+    for (int u = lane; u < wide; u += 32) a[u] = 0.0f;
+    __syncwarp();
+    for (int h = lane; h < nh; h += 32) a[h + 1] = p.k_max * sigmoid_f(E1[h]);  // constant per image
     __syncwarp();
     grn_soft_outputs(p, s_W2, s_b2, X, aO, lane);
     const bool bad_input = (*p.flag & kErrBadSamples) != 0;
     const uint64_t gid = p.traj_offset + (uint64_t)i;
-    const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32), key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
+    const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
 
     double t = 0.0;
     int s = 0;
@@ -433,7 +452,7 @@ __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, fl
     while (!bad_input) {
         if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
         float E0, invZ;
-        const float a0 = grn_soft_weights(p, s_d, X, aH, aO, q, k, c2, c3, key0, key1, lane, E0, invZ);
+        const float a0 = grn_soft_weights(p, a, q, k, noise, lane, E0, invZ);
         if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
         if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
         const float tau = waiting_time(E0, a0);
@@ -451,7 +470,7 @@ __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, fl
             thr = s < p.S ? p.ts[s] : p.t_end;
             if (cross) break;
         }
-        grn_soft_update(p, X, q, invZ, lane);
+        grn_soft_update(p, s_d, X, a, q, invZ, lane);
         grn_soft_outputs(p, s_W2, s_b2, X, aO, lane);
         t = t_next;
         ++k;
@@ -492,6 +511,13 @@ __host__ __device__ inline int grn_soft_row(int nd, int no, int M)
     return ((nd + 3) & ~3) + ((no + 3) & ~3) + ((M + 3) & ~3) + 4;
 }
 
+// words of one warp's arrays in the soft adjoint: X, a, key, lam, dlogd, 1 - sigma(E1), G1, db2, G2 of a segment
+__host__ __device__ inline size_t grn_soft_adj_words(int nh, int no)
+{
+    const int nd = nh + no, ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3, nop = (no + 3) & ~3;
+    return 3 * (size_t)ndp + 2 * (size_t)wide_len(2 * nd) + 2 * (size_t)nhp + (1 + kGrnSoftK) * (size_t)nop;
+}
+
 }  // namespace
 
 __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
@@ -499,21 +525,23 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
     const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn, M = p.M;
-    const int ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3, nop = (no + 3) & ~3, Mq = (M + 3) & ~3;
+    const int ndp = (nd + 3) & ~3, nhp = (nh + 3) & ~3, nop = (no + 3) & ~3, Mq = (M + 3) & ~3, wide = wide_len(M);
     const int RS = grn_soft_row(nd, no, M);
     float *s_W2 = reinterpret_cast<float *>(smem);
     float *s_d = s_W2 + (size_t)no * nh;
     float *s_b2 = s_d + nd;
-    const size_t per_warp = 3 * (size_t)ndp + 2 * (size_t)nhp + (2 + kGrnSoftK) * (size_t)nop + (size_t)Mq;
-    float *X = s_b2 + nop + (size_t)wib * per_warp;  // the state being stepped or differentiated
-    float *lam = X + ndp;                             // dL/dX of the state after the step
+    const size_t per_warp = grn_soft_adj_words(nh, no);
+    float *base0 = reinterpret_cast<float *>(smem + ((4 * ((size_t)no * nh + nd + nop) + 15) & ~(size_t)15));
+    float *X = base0 + (size_t)wib * per_warp;       // the state being stepped or differentiated
+    float *a = X + ndp;                               // propensities by word
+    float *q = a + wide;                              // keys, then unnormalised weights, by word
+    float *lam = q + wide;                            // dL/dX of the state after the step
     float *dlogd = lam + ndp;
-    float *aH = dlogd + ndp;
-    float *G1 = aH + nhp;
-    float *aO = G1 + nhp;
-    float *db2 = aO + nop;
+    float *cH = dlogd + ndp;                          // 1 - sigma(E1)
+    float *G1 = cH + nhp;
+    float *db2 = G1 + nhp;
     float *G2h = db2 + nop;                           // [kGrnSoftK][nop]: dL/dE2 of the segment's steps
-    float *q = G2h + kGrnSoftK * nop;
+    float *aO = a + nh + 1;
     for (int u = threadIdx.x; u < no * nh; u += blockDim.x) s_W2[u] = p.W2f[u];
     for (int u = threadIdx.x; u < nd; u += blockDim.x) s_d[u] = p.dvec[u];
     for (int u = threadIdx.x; u < no; u += blockDim.x) s_b2[u] = p.b2[u];
@@ -542,14 +570,18 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
         // a finished run's last draw is the crossing one, which moves no observed state
         const int L = (st == SSA_TRAJ_OK) ? d - 1 : d;
         for (int u = lane; u < nd; u += 32) lam[u] = 0.0f;
+        for (int u = lane; u < wide; u += 32) a[u] = 0.0f;
+        for (int u = lane; u < kGrnSoftK * nop; u += 32) G2h[u] = 0.0f;
+        __syncwarp();
+        const float inv_kmax = 1.0f / p.k_max;
         for (int h = lane; h < nh; h += 32) {
-            aH[h] = p.k_max * sigmoid_f(E1[h]);
+            a[h + 1] = p.k_max * sigmoid_f(E1[h]);
+            cH[h] = 1.0f - a[h + 1] * inv_kmax;
             G1[h] = 0.0f;
         }
         __syncwarp();
         const uint64_t gid = p.traj_offset + (uint64_t)i;
-        const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32), key0 = (uint32_t)p.seed,
-                       key1 = (uint32_t)(p.seed >> 32);
+        const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
         const float invT = p.invT;
         const float *gl = p.dl_dobs + i * p.dl_stride;
         int s_hi = p.S - 1;
@@ -557,7 +589,11 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
         int mism = 0;
         for (int c = L / kGrnSoftK; c >= 0; --c) {
             const int k0 = c * kGrnSoftK, k1 = min(k0 + kGrnSoftK - 1, L);
-            for (int u = lane; u < nd; u += 32) X[u] = ckf[(int64_t)c * nd + u];
+            for (int u = lane; u < nd; u += 32) {
+                const float x = ckf[(int64_t)c * nd + u];
+                X[u] = x;
+                a[nd + u + 1] = __fmul_rn(s_d[u], fmaxf(x, 0.0f));
+            }
             __syncwarp();
             for (int kk = k0; kk <= k1; ++kk) {  // re-run the segment with the forward's routines
                 float *row = seg + (kk - k0) * RS;
@@ -565,11 +601,11 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
                 if (kk < L) {
                     grn_soft_outputs(p, s_W2, s_b2, X, aO, lane);
                     float E0, invZ;
-                    grn_soft_weights(p, s_d, X, aH, aO, q, kk, c2, c3, key0, key1, lane, E0, invZ);
+                    grn_soft_weights(p, a, q, kk, noise, lane, E0, invZ);
                     for (int o = lane; o < no; o += 32) row[ndp + o] = aO[o];
-                    for (int j = lane; j < M; j += 32) row[ndp + nop + j] = q[j];
+                    for (int j = lane; j < M; j += 32) row[ndp + nop + j] = q[j + 1];
                     if (lane == 0) row[ndp + nop + Mq] = invZ;
-                    grn_soft_update(p, X, q, invZ, lane);
+                    grn_soft_update(p, s_d, X, a, q, invZ, lane);
                 }
             }
             if (k1 < L) {
@@ -588,36 +624,39 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
                     brk_next = s_hi >= 0 ? p.brk_k[(int64_t)s_hi * n + i] : -1;
                 }
                 if (k < L) {
-                    for (int u = lane; u < nd; u += 32) X[u] = row[u];
-                    for (int o = lane; o < no; o += 32) aO[o] = row[ndp + o];
                     const float invZ = row[ndp + nop + Mq];
-                    // W = sum_j q_j w_j / Z with w_j = +lam_s (production) or -lam_s (degradation)
+                    const float *qrow = row + ndp + nop;
+                    // W = sum_j q_j w_j / Z with w_j = +lam_s (production) or -lam_s (degradation); a lane takes both
+                    // reactions of its species
                     float Wp = 0.0f;
-                    for (int j = lane; j < M; j += 32) {
-                        const float qj = row[ndp + nop + j];
-                        q[j] = qj;
-                        Wp += qj * (j < nd ? lam[j] : -lam[j - nd]);
-                    }
-                    const float Wbar = warp_sum(Wp) * invZ;
-                    __syncwarp();
-                    // choice-path adjoints psi_j = dL/dlog a_j of the productions (HOLD readout: no waiting-time path)
-                    for (int j = lane; j < nd; j += 32) {
-                        const float psi = q[j] > 0.0f ? q[j] * invZ * (lam[j] - Wbar) * invT : 0.0f;
-                        if (j < nh)
-                            G1[j] += psi * (1.0f - __fdividef(aH[j], p.k_max));
-                        else
-                            G2[j - nh] = psi * (1.0f - __fdividef(aO[j - nh], p.k_max));
+#pragma unroll 4
+                    for (int u = lane; u < nd; u += 32) Wp = fmaf(qrow[u] - qrow[nd + u], lam[u], Wp);
+                    const float Wbar = warp_sum(Wp) * invZ, scale = invZ * invT;
+                    // choice-path adjoints psi_j = dL/dlog a_j (HOLD readout: no waiting-time path), the outputs first
+                    for (int o = lane; o < no; o += 32) {
+                        const float qp = qrow[nh + o], psi = qp * scale * (lam[nh + o] - Wbar);
+                        G2[o] = (qp > 0.0f ? psi : 0.0f) * (1.0f - row[ndp + o] * inv_kmax);
                     }
                     __syncwarp();
                     // the degradations: psi of d_u max(X_u, 0); a weight q > 0 implies a > 0, so X_u > 0 there
+#pragma unroll 2
                     for (int u = lane; u < nd; u += 32) {
-                        const float qd = q[nd + u];
-                        const float psi = qd > 0.0f ? qd * invZ * (-lam[u] - Wbar) * invT : 0.0f;
+                        const float l = lam[u], qd = qrow[nd + u];
+                        float psi = qd * scale * (-l - Wbar);
+                        psi = qd > 0.0f ? psi : 0.0f;
                         dlogd[u] += psi;
-                        float acc = qd > 0.0f ? __fdividef(psi, X[u]) : 0.0f;
-                        if (u < nh)
-                            for (int o = 0; o < no; ++o) acc += s_W2[(size_t)o * nh + u] * G2[o];
-                        lam[u] += acc;
+                        float acc = __fdividef(psi, row[u]);
+                        acc = qd > 0.0f ? acc : 0.0f;
+                        if (u < nh) {
+                            const float qp = qrow[u], psi_p = qp * scale * (l - Wbar);
+                            G1[u] += (qp > 0.0f ? psi_p : 0.0f) * cH[u];
+                            const float4 *w = p.W2t + (int64_t)u * (nop >> 2), *g = reinterpret_cast<const float4 *>(G2);
+                            for (int v = 0; v < nop >> 2; ++v) {  // in output order; the padding adds 0
+                                const float4 wv = __ldg(w + v), gv = g[v];
+                                acc = fmaf(wv.w, gv.w, fmaf(wv.z, gv.z, fmaf(wv.y, gv.y, fmaf(wv.x, gv.x, acc))));
+                            }
+                        }
+                        lam[u] = l + acc;
                     }
                 }
                 __syncwarp();
@@ -650,12 +689,11 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
     __syncthreads();
     // fixed-order sum over the block's warps: [db2 | dlogd]
     const int red = no + nd;
-    const float *base0 = s_b2 + nop;
     for (int u = threadIdx.x; u < red; u += blockDim.x) {
         float acc = 0.0f;
         for (int w = 0; w < W; ++w) {
             const float *wp = base0 + w * per_warp;
-            acc += u < no ? wp[3 * ndp + 2 * nhp + nop + u] : wp[2 * ndp + (u - no)];
+            acc += u < no ? wp[3 * ndp + 2 * wide + 2 * nhp + u] : wp[2 * ndp + 2 * wide + (u - no)];
         }
         p.partial[(int64_t)blockIdx.x * red + u] = acc;
     }
@@ -1025,6 +1063,37 @@ int grn_warps(const ssa_grn *g)
     return w;
 }
 
+// The relaxed path takes networks whose W2 leaves this much room (four warps with four arrays of the species and one of
+// the reactions each, and the segment's dL/dE2); a block has fewer warps where four of the kernels' own arrays do not
+// fit.
+bool grn_soft_fits(const ssa_grn *g, bool record)
+{
+    const size_t ndp = (g->n_dyn + 3) & ~3, nhp = (g->n_hid + 3) & ~3, nop = (g->n_out + 3) & ~3, Mq = (g->M + 3) & ~3;
+    const size_t shared = (size_t)g->n_out * g->n_hid + g->n_dyn + nop;
+    const size_t fwd = 4 * (shared + 4 * (ndp + nhp + nop + Mq));
+    const size_t adj = 4 * (shared + 4 * (3 * ndp + 2 * nhp + (2 + kGrnSoftK) * nop + Mq));
+    return fwd <= kGrnMaxSmem && (!record || adj <= kGrnMaxSmem);
+}
+
+size_t grn_soft_fwd_smem(const ssa_grn *g, int warps)
+{
+    const size_t ndp = (g->n_dyn + 3) & ~3, nop = (g->n_out + 3) & ~3;
+    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop + warps * (ndp + 2 * (size_t)wide_len(g->M))) + 16;
+}
+
+size_t grn_soft_adj_smem(const ssa_grn *g, int warps)
+{
+    const size_t nop = (g->n_out + 3) & ~3;
+    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop + warps * grn_soft_adj_words(g->n_hid, g->n_out)) + 16;
+}
+
+int grn_soft_warps(const ssa_grn *g)
+{
+    int w = kGrnWarps;
+    while (w > 1 && std::max(grn_soft_fwd_smem(g, w), grn_soft_adj_smem(g, w)) > kGrnMaxSmem) --w;
+    return w;
+}
+
 WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, const ssa_fwd_opts *o)
 {
     WsLayout L{};
@@ -1065,7 +1134,7 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
         const int K = o->selector == SSA_SELECT_SOFT ? kGrnSoftK : o->ckpt_interval > 0 ? o->ckpt_interval : 64;
         L.ev_rows = (o->max_steps + 7) / 8;
         L.n_ckpt = o->max_steps / K + 1;
-        const int wpb = o->selector == SSA_SELECT_SOFT ? kGrnWarps : grn_warps(g);
+        const int wpb = o->selector == SSA_SELECT_SOFT ? grn_soft_warps(g) : grn_warps(g);
         L.max_blocks = (n + wpb - 1) / wpb;
         L.xfinal = take((size_t)g->n_dyn * n * 4);
         L.ev = take((size_t)L.ev_rows * n * sizeof(uint4));
@@ -1087,20 +1156,6 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
     }
     L.total = off;
     return L;
-}
-
-
-size_t grn_soft_fwd_smem(const ssa_grn *g)
-{
-    const int ndp = (g->n_dyn + 3) & ~3, nhp = (g->n_hid + 3) & ~3, nop = (g->n_out + 3) & ~3, Mq = (g->M + 3) & ~3;
-    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop) + 4 * (size_t)kGrnWarps * (ndp + nhp + nop + Mq);
-}
-
-size_t grn_soft_adj_smem(const ssa_grn *g)
-{
-    const int ndp = (g->n_dyn + 3) & ~3, nhp = (g->n_hid + 3) & ~3, nop = (g->n_out + 3) & ~3, Mq = (g->M + 3) & ~3;
-    const size_t per_warp = 3 * (size_t)ndp + 2 * (size_t)nhp + (2 + kGrnSoftK) * (size_t)nop + (size_t)Mq;
-    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop + (size_t)kGrnWarps * per_warp);
 }
 
 
@@ -1160,7 +1215,7 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
         return set_error(SSA_ERR_UNSUPPORTED, "the GRN runs the Gumbel-max selector or the soft forward");
     if (soft && (!(opts->temperature > 0.0f) || !(opts->temperature < 3.0e38f)))
         return set_error(SSA_ERR_UNSUPPORTED, "the GRN's soft forward needs T > 0");
-    if (soft && (grn_soft_fwd_smem(g) > kGrnMaxSmem || (opts->record && grn_soft_adj_smem(g) > kGrnMaxSmem)))
+    if (soft && !grn_soft_fits(g, opts->record != 0))
         return set_error(SSA_ERR_UNSUPPORTED, "the GRN's soft path keeps W2 (and a recorded run dL/dW2) in shared memory: "
                                               "n_out * n_hid too large");
     if (opts->max_steps < 1 || opts->max_steps > 0x7fffffffLL || (opts->ckpt_interval % 8) || opts->ckpt_interval < 0)
@@ -1250,9 +1305,10 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
     }
     if (n > 0 && soft) {
         p.invT = 1.0f / opts->temperature;
-        const size_t smem = grn_soft_fwd_smem(g);
+        const int wpb = grn_soft_warps(g);
+        const size_t smem = grn_soft_fwd_smem(g, wpb);
         GRN_CUDA_TRY(cudaFuncSetAttribute(grn_soft_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_soft_fwd_kernel<<<(unsigned)((n + kGrnWarps - 1) / kGrnWarps), 32 * kGrnWarps, smem, st>>>(
+        grn_soft_fwd_kernel<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
             p, reinterpret_cast<float *>(obs_out), opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
@@ -1346,13 +1402,13 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     p.err = flag + 1;
     p.n_ckpt = L.n_ckpt;
     p.seg = soft ? reinterpret_cast<float *>(ws + L.soft_seg) : nullptr;
-    const int wpb = soft ? kGrnWarps : grn_warps(g);
+    const int wpb = soft ? grn_soft_warps(g) : grn_warps(g);
     const int64_t nblk = (n + wpb - 1) / wpb;
     float *red = reinterpret_cast<float *>(ws + L.red);
     if (n > 0 && soft) {
-        const size_t smem = grn_soft_adj_smem(g);
+        const size_t smem = grn_soft_adj_smem(g, wpb);
         GRN_CUDA_TRY(cudaFuncSetAttribute(grn_soft_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_soft_adj_kernel<<<(unsigned)nblk, 32 * kGrnWarps, smem, st>>>(p);
+        grn_soft_adj_kernel<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
         const size_t smem = grn_adj_smem(g, wpb);
