@@ -520,7 +520,10 @@ __host__ __device__ inline size_t grn_soft_adj_words(int nh, int no)
 
 }  // namespace
 
-__global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
+// NS rounds of species (n_dyn <= 32 NS) read a step's weights and state into registers together, one wait for memory a
+// step; NS = 0: any number, read where they are used.
+template <int NS>
+__global__ void __launch_bounds__(128, 4) grn_soft_adj_kernel(const GrnParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
@@ -629,8 +632,22 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
                     // W = sum_j q_j w_j / Z with w_j = +lam_s (production) or -lam_s (degradation); a lane takes both
                     // reactions of its species
                     float Wp = 0.0f;
-#pragma unroll 4
-                    for (int u = lane; u < nd; u += 32) Wp = fmaf(qrow[u] - qrow[nd + u], lam[u], Wp);
+                    constexpr int NR = NS > 0 ? NS : 1;
+                    float qpr[NR], qdr[NR], xr[NR];
+                    if constexpr (NS > 0) {
+#pragma unroll
+                        for (int c2 = 0; c2 < NS; ++c2) {
+                            const int u = min(32 * c2 + lane, nd - 1);
+                            qpr[c2] = qrow[u];
+                            qdr[c2] = qrow[nd + u];
+                            xr[c2] = row[u];
+                        }
+#pragma unroll
+                        for (int c2 = 0; c2 < NS; ++c2)
+                            if (32 * c2 + lane < nd) Wp = fmaf(qpr[c2] - qdr[c2], lam[32 * c2 + lane], Wp);
+                    } else {
+                        for (int u = lane; u < nd; u += 32) Wp = fmaf(qrow[u] - qrow[nd + u], lam[u], Wp);
+                    }
                     const float Wbar = warp_sum(Wp) * invZ, scale = invZ * invT;
                     // choice-path adjoints psi_j = dL/dlog a_j (HOLD readout: no waiting-time path), the outputs first
                     for (int o = lane; o < no; o += 32) {
@@ -639,16 +656,15 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
                     }
                     __syncwarp();
                     // the degradations: psi of d_u max(X_u, 0); a weight q > 0 implies a > 0, so X_u > 0 there
-#pragma unroll 2
-                    for (int u = lane; u < nd; u += 32) {
-                        const float l = lam[u], qd = qrow[nd + u];
+                    auto species = [&](int u, float qp, float qd, float x) {
+                        const float l = lam[u];
                         float psi = qd * scale * (-l - Wbar);
                         psi = qd > 0.0f ? psi : 0.0f;
                         dlogd[u] += psi;
-                        float acc = __fdividef(psi, row[u]);
+                        float acc = __fdividef(psi, x);
                         acc = qd > 0.0f ? acc : 0.0f;
                         if (u < nh) {
-                            const float qp = qrow[u], psi_p = qp * scale * (l - Wbar);
+                            const float psi_p = qp * scale * (l - Wbar);
                             G1[u] += (qp > 0.0f ? psi_p : 0.0f) * cH[u];
                             const float4 *w = p.W2t + (int64_t)u * (nop >> 2), *g = reinterpret_cast<const float4 *>(G2);
                             for (int v = 0; v < nop >> 2; ++v) {  // in output order; the padding adds 0
@@ -657,6 +673,13 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
                             }
                         }
                         lam[u] = l + acc;
+                    };
+                    if constexpr (NS > 0) {
+#pragma unroll
+                        for (int c2 = 0; c2 < NS; ++c2)
+                            if (32 * c2 + lane < nd) species(32 * c2 + lane, qpr[c2], qdr[c2], xr[c2]);
+                    } else {
+                        for (int u = lane; u < nd; u += 32) species(u, qrow[u], qrow[nd + u], row[u]);
                     }
                 }
                 __syncwarp();
@@ -672,11 +695,12 @@ __global__ void __launch_bounds__(128, 5) grn_soft_adj_kernel(const GrnParams p)
 #pragma unroll
                 for (int r = 0; r < kGrnSoftK; ++r) xs[r] = r < len ? seg[r * RS + h] : 0.0f;
                 for (int o = 0; o < no; ++o) {
-                    float acc = dW2[(size_t)o * nh + h];
+                    // rows past the segment's end carry 0; added without waiting for memory (one lane's adds to a place
+                    // keep their order)
+                    float acc = 0.0f;
 #pragma unroll
-                    for (int r = 0; r < kGrnSoftK; ++r)
-                        if (r < len) acc = __fmaf_rn(G2h[r * nop + o], xs[r], acc);
-                    dW2[(size_t)o * nh + h] = acc;
+                    for (int r = 0; r < kGrnSoftK; ++r) acc = __fmaf_rn(G2h[r * nop + o], xs[r], acc);
+                    atomicAdd(dW2 + (size_t)o * nh + h, acc);
                 }
             }
             for (int o = lane; o < no; o += 32)
@@ -1407,8 +1431,9 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     float *red = reinterpret_cast<float *>(ws + L.red);
     if (n > 0 && soft) {
         const size_t smem = grn_soft_adj_smem(g, wpb);
-        GRN_CUDA_TRY(cudaFuncSetAttribute(grn_soft_adj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_soft_adj_kernel<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
+        auto kern = grn_sums_in_registers(g) ? grn_soft_adj_kernel<9> : grn_soft_adj_kernel<0>;
+        GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
         const size_t smem = grn_adj_smem(g, wpb);
