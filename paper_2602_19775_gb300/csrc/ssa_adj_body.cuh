@@ -171,7 +171,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                     race(a, exp_variate((uint32_t)k, j + 1, c2, c3, key0, key1, cache, cb), j, ab, Eb, jb);
                 }
             }
-            const float inv_m1 = m1 > 0.0f ? __fdividef(1.0f, m1) : 0.0f;
+            const KeyTop top = key_top(m1);
             mism += (jb != jk);
             const float tau = waiting_time(E0, a0);
             tau_k = tau;
@@ -207,7 +207,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 float wr[MC];
 #pragma unroll
                 for (int j = 0; j < MC; ++j) {
-                    const float q = ex2_approx(lg2_approx(lr[j] * inv_m1) * invT);
+                    const float q = ex2_approx(top.lg2(lr[j]) * invT);
                     lr[j] = q;
                     wr[j] = stoich_dot(s_rx[j], s_st, lam, B);
                     Z += q;
@@ -225,7 +225,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 }
             } else {
                 for (int j = 0; j < M; ++j) {
-                    const float q = ex2_approx(lg2_approx(qbuf[j * B] * inv_m1) * invT);
+                    const float q = ex2_approx(top.lg2(qbuf[j * B]) * invT);
                     qbuf[j * B] = q;
                     if (q > 0.0f) {
                         Z += q;

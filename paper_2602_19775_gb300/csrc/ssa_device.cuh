@@ -227,6 +227,20 @@ __device__ __forceinline__ float key_scale(float a0)
 {
     return (a0 >= 0x1p-60f && a0 <= 0x1p100f) ? 1.0f : (a0 > 1.0f ? 0x1p-60f : 0x1p100f);
 }
+// The largest key m of a race as the others are compared with it: times the power of two `scale` it lies in [1, 2)
+// and a key r weighs 2^((lg2(r scale) - lg2_top) / T). The largest then weighs exactly 2^0, so that a choice that is
+// certain leaves no rounding in psi; through a reciprocal of m it weighed 1 to an ulp or two.
+struct KeyTop {
+    float scale, lg2_top;
+    __device__ __forceinline__ float lg2(float r) const { return lg2_approx(r * scale) - lg2_top; }
+};
+__device__ __forceinline__ KeyTop key_top(float m)
+{
+    KeyTop t;
+    t.scale = __uint_as_float(0x7f000000u - (__float_as_uint(m) & 0x7f800000u));
+    t.lg2_top = m > 0.0f ? lg2_approx(m * t.scale) : 0.0f;
+    return t;
+}
 // Two keys within this of each other, relatively, count as a possible tie (a key is a few units in the last place
 // off, and so is the comparison of products that decides the race).
 constexpr float kTieMargin = 0x1p-15f;

@@ -381,11 +381,11 @@ __device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const floa
     rmax = warp_max_nonneg(rmax);
     E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
     if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(rounds, a, k, z, a0, key);
-    const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
+    const KeyTop top = key_top(rmax);
     float Zp = 0.0f;
     for (int c = 0; c < rounds; ++c) {
         const float4 kv = key4[32 * c + lane];
-        auto weight = [&](float v) { return ex2_approx(lg2_approx(v * inv_rmax) * p.invT); };
+        auto weight = [&](float v) { return ex2_approx(top.lg2(v) * p.invT); };
         const float4 q = make_float4(weight(kv.x), weight(kv.y), weight(kv.z), weight(kv.w));
         key4[32 * c + lane] = q;
         Zp += (q.x + q.y) + (q.z + q.w);
@@ -884,17 +884,18 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                 rmax = warp_max_nonneg(rmax);
                 if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f)) rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, key);
                 __syncwarp();
-                const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
-                const bool k_tops = key[jk + 1] * inv_rmax >= 1.0f - kTieMargin;
+                const KeyTop top = key_top(rmax);
+                const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
+                const bool k_tops = key[jk + 1] >= top_edge;
                 // pass 2: soft-sample weights q_j = (key_j / largest)^(1/T), Z = sum q, W = sum q w with
                 // w_j = +lam_s (production of s) or -lam_s (degradation of s)
                 float Zp = 0.0f, Wp = 0.0f;
                 int near = 0;  // keys within the tie margin of the largest
                 float qp[NS > 0 ? NS : 1], qd[NS > 0 ? NS : 1];
                 each_species([&](int c, int s) {
-                    const float rp = key[s + 1] * inv_rmax, rd = key[nd + s + 1] * inv_rmax;
-                    near += (rp >= 1.0f - kTieMargin) + (rd >= 1.0f - kTieMargin);
-                    const float q1 = ex2_approx(lg2_approx(rp) * invT), q2 = ex2_approx(lg2_approx(rd) * invT);
+                    const float rp = key[s + 1], rd = key[nd + s + 1];
+                    near += (rp >= top_edge) + (rd >= top_edge);
+                    const float q1 = ex2_approx(top.lg2(rp) * invT), q2 = ex2_approx(top.lg2(rd) * invT);
                     Zp += q1 + q2;
                     Wp = fmaf(q1 - q2, lam(c), Wp);
                     if (NS > 0) {

@@ -764,10 +764,10 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
                 jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
             }
             mism += (jb != jk);
-            const float inv_m1 = m1 > 0.0f ? __fdividef(1.0f, m1) : 0.0f;
+            const KeyTop top = key_top(m1);
             float lg2_key[JM];
 #pragma unroll
-            for (int j = 0; j < JM; ++j) lg2_key[j] = lg2_approx(key[j] * inv_m1);
+            for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
             JitCoef coef;
             jit_coef(X, kr, a, h, coef);
             // The walk's divisions by a0 (tau = E0/a0 and d tau/d a0 = -tau/a0) take one approximate

@@ -961,8 +961,9 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             rmax = warp_max_nonneg(rmax);
             if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, rj);
             __syncwarp();
-            const float inv_rmax = rmax > 0.0f ? __fdividef(1.0f, rmax) : 0.0f;
-            const bool k_tops = rj[jk + 1] * inv_rmax >= 1.0f - kTieMargin;
+            const KeyTop top = key_top(rmax);
+            const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
+            const bool k_tops = rj[jk + 1] >= top_edge;
             const float tau = waiting_time(E0, a0);
             tau_k = tau;
             const int4 rk = tab.rx[jpos(jk, nb)];
@@ -1007,9 +1008,8 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
                     const int4 *el = tab.ent + 128 * c + lane;
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
-                        const float rel = qv[q] * inv_rmax;
-                        near += rel >= 1.0f - kTieMargin;
-                        qv[q] = ex2_approx(lg2_approx(rel) * invT);
+                        near += qv[q] >= top_edge;
+                        qv[q] = ex2_approx(top.lg2(qv[q]) * invT);
                         const int4 en = el[32 * q];
                         float w = ent_change(en.x) * at(en.x);
                         w = __fmaf_rn(ent_change(en.y), at(en.y), w);
