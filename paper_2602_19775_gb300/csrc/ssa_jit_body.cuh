@@ -172,13 +172,13 @@ __device__ __forceinline__ void jit_bin_init(const FwdParams &p, bool bad_obs, f
     }
 }
 
-// Coalesced sample stores. A trajectory's samples are one row of obs [n_traj][S][n_obs], written one at a
-// time as its clock passes them, so a warp's per-thread stores land in 32 different rows. Instead each
-// thread collects a window of W = 16 / n_obs consecutive samples (n_obs <= 4) in its row of a per-block
-// shared buffer; at the top of every step the warp's active lanes copy the completed windows together, two
-// windows per store instruction (consecutive words of two rows). A lane whose window fills
-// while it still has samples to write in the same step, and every lane after its last step, writes its own
-// window. The values and their places are those of direct stores.
+// Sample stores. A trajectory's samples are one row of obs [n_traj][S][n_obs], made one at a time as its clock passes
+// them, so a warp's stores of single values land in 32 rows, a sector each. Instead each thread collects a window of
+// 16 / n_obs consecutive samples (n_obs <= 4) in its row of a per-block shared buffer and writes it when it is full, in
+// 8-byte pieces where the row allows. The values and their places are those of direct stores.
+// The windows are written by their threads: gathered over the warp, two windows an instruction, a write cost every step
+// a vote and two steps in five some sixty instructions of shuffles and indices. 2A <-> B, 50 samples, forward: 1,048,576
+// trajectories 3.28 -> 3.04 ms, 1,024 trajectories 264 -> 237 us; the oscillator's 400 samples in 13.3 ms either way.
 constexpr int kJitFwdBlock = 64;    // threads per block of the specialised forwards
 constexpr int kStageWords = 16;     // words of a thread's sample window
 
@@ -188,7 +188,6 @@ struct SampleStage {
     int64_t base;    // first word of this trajectory's row
     int n_obs, W, S;
     int lo, cnt;     // the window holds samples lo .. lo + cnt - 1
-    bool ready;      // complete and not yet copied
 };
 
 __device__ __forceinline__ void stage_own_flush(SampleStage &g)
@@ -204,63 +203,16 @@ __device__ __forceinline__ void stage_own_flush(SampleStage &g)
     }
     g.lo += g.cnt;
     g.cnt = 0;
-    g.ready = false;
 }
 
 // one sample s (the next in order) of n_obs values
 template <class VAL>
 __device__ __forceinline__ void stage_put(SampleStage &g, int s, const VAL &val)
 {
-    if (g.ready) stage_own_flush(g);  // a second window completes within one step
     uint32_t *w = g.row + g.cnt * g.n_obs;
     for (int c = 0; c < g.n_obs; ++c) w[c] = val(c);
     ++g.cnt;
-    if (g.cnt == g.W || s + 1 == g.S) g.ready = true;
-}
-
-// the warp's active lanes copy every completed window, two at a time
-__device__ __forceinline__ void stage_warp_flush(SampleStage &g, const uint32_t *s_stage)
-{
-    const unsigned m = __activemask();
-    unsigned rd = __ballot_sync(m, g.ready);
-    if (!rd) return;
-    const int lane = threadIdx.x & 31;
-    const int first = threadIdx.x & ~31;
-    const int rank = __popc(m & ((1u << lane) - 1u)), nm = __popc(m);
-    const int64_t dst = g.base + (int64_t)g.lo * g.n_obs;
-    const int words = g.cnt * g.n_obs;
-    __syncwarp(m);
-    while (rd) {
-        const int a = __ffs(rd) - 1;
-        rd &= rd - 1;
-        int b = -1;
-        if (rd) {
-            b = __ffs(rd) - 1;
-            rd &= rd - 1;
-        }
-        const long long da = __shfl_sync(m, (long long)dst, a);
-        const int wa = __shfl_sync(m, words, a);
-        long long db = 0;
-        int wb = 0;
-        if (b >= 0) {
-            db = __shfl_sync(m, (long long)dst, b);
-            wb = __shfl_sync(m, words, b);
-        }
-        // the words of window a, then of window b, shared out over the participating lanes in the order of
-        // their lane numbers (lanes that have left the step loop take no part): one store instruction when all
-        // 32 lanes take part, a few otherwise
-        for (int pw = rank; pw < wa + wb; pw += nm) {
-            const bool in_a = pw < wa;
-            const int q = in_a ? pw : pw - wa;
-            g.out[(in_a ? da : db) + q] = s_stage[(first + (in_a ? a : b)) * kStageWords + q];
-        }
-    }
-    __syncwarp(m);
-    if (g.ready) {
-        g.lo += g.cnt;
-        g.cnt = 0;
-        g.ready = false;
-    }
+    if (g.cnt == g.W) stage_own_flush(g);
 }
 
 template <int READOUT, bool RECORD>
@@ -307,10 +259,9 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
     const bool staged = READOUT != SSA_READOUT_BIN && p.n_obs >= 1 && p.n_obs <= 4 && blockDim.x <= kJitFwdBlock;
     SampleStage stg{s_stage + threadIdx.x * kStageWords, static_cast<uint32_t *>(p.obs_out), i * p.S * p.n_obs,
-                    p.n_obs, staged ? kStageWords / p.n_obs : 1, p.S, 0, 0, false};
+                    p.n_obs, staged ? kStageWords / p.n_obs : 1, p.S, 0, 0};
 
     while (!bad_input) {
-        if (staged) stage_warp_flush(stg, s_stage);
         if (k >= max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
         jit_noise(E0n, cn, (uint32_t)(k + 1), c2, c3, key0, key1);  // next step, state-independent
         float a[JM], h[JM];
