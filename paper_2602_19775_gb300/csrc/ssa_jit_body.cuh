@@ -582,6 +582,10 @@ template <int READOUT, bool WIDE = false, int NT = 1>
 __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&kr)[JM], const int64_t i, const int st,
                                              float (&dAr)[NT][JM], int &sc, const BinChunks chunks, const int *s_chg)
 {
+    auto adj_noise = [](auto &v, uint32_t k, uint32_t c2, uint32_t c3, uint32_t key0, uint32_t key1) {
+        if constexpr (WIDE) step_noise<JM + 1>(v, k, c2, c3, key0, key1);
+        else step_noise_inv<JM + 1>(v, k, c2, c3, key0, key1);
+    };
     static_assert(!WIDE || NT == 1, "the wide-range walk takes one temperature");
     sc = 0;
     float inj = 1.0f;  // 2^-sc: the factor of every upstream-gradient term
@@ -652,7 +656,7 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
     constexpr int NQ = JM + 1;
     float E[NQ], En[NQ];
     const bool draw_last = st == SSA_TRAJ_OK;
-    step_noise_inv<NQ>(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
+    adj_noise(E, (uint32_t)(draw_last ? L : (L > 0 ? L - 1 : 0)), c2, c3, key0, key1);
     const bool few = p.n_obs <= kBinMaxObs;  // their species in registers
 
     // BIN readout (NT = 1): gq = g of the bin that contains t_{k+1}, xo = X_{k+1} at the observables
@@ -701,36 +705,51 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
         }
         float tau_k = 0.0f;
         if (draw) {
-            if (k > 0) step_noise_inv<NQ>(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
+            if (k > 0) adj_noise(En, (uint32_t)(k - 1), c2, c3, key0, key1);  // prefetch
             float a[JM], h[JM], key[JM];
             jit_props(X, kr, a, h);
             // pass 1: a0 and the race's keys a_j / E_j, with the two largest
-            float a0 = 0.0f, m1 = 0.0f, m2 = 0.0f;
+            float a0 = 0.0f;
             int jb = -1;
             const float E0 = E[0];
-#pragma unroll
-            for (int j = 0; j < JM; ++j) a0 = __fadd_rn(a0, a[j]);
-            const float sc_key = key_scale(a0);
-#pragma unroll
-            for (int j = 0; j < JM; ++j) {
-                key[j] = (a[j] * sc_key) * E[j + 1];
-                jb = key[j] > m1 ? j : jb;
-                m2 = fmaxf(m2, fminf(m1, key[j]));
-                m1 = fmaxf(m1, key[j]);
-            }
-            // the recorded reaction won the race if its key is the largest by more than the keys' error; near ties are
-            // raced again
-            if (m2 >= m1 * (1.0f - kTieMargin)) {
-                JitRates r;
-#pragma unroll
-                for (int j = 0; j < JM; ++j) r.a[j] = a[j];
-                jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
-            }
-            mism += (jb != jk);
-            const KeyTop top = key_top(m1);
             float lg2_key[JM];
 #pragma unroll
-            for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
+            for (int j = 0; j < JM; ++j) a0 = __fadd_rn(a0, a[j]);
+            // Over the ~1e6 steps of a wide walk the bias of the keys' approximations adds up (the oscillator's gradient
+            // at t = 400: 2.2e-3 from binary64 with them): their logarithms are taken of the accurate variates.
+            if constexpr (WIDE) {
+                float ab = 0.0f, Eb = 1.0f, lg2_top = -CUDART_INF_F;
+#pragma unroll
+                for (int j = 0; j < JM; ++j) {
+                    race(a[j], E[j + 1], j, ab, Eb, jb);
+                    lg2_key[j] = a[j] > 0.0f ? __log2f(a[j]) - __log2f(E[j + 1]) : -CUDART_INF_F;
+                    lg2_top = fmaxf(lg2_top, lg2_key[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < JM; ++j) lg2_key[j] -= lg2_top;
+            } else {
+                float m1 = 0.0f, m2 = 0.0f;
+                const float sc_key = key_scale(a0);
+#pragma unroll
+                for (int j = 0; j < JM; ++j) {
+                    key[j] = (a[j] * sc_key) * E[j + 1];
+                    jb = key[j] > m1 ? j : jb;
+                    m2 = fmaxf(m2, fminf(m1, key[j]));
+                    m1 = fmaxf(m1, key[j]);
+                }
+                // the recorded reaction won the race if its key is the largest by more than the keys' error; near ties are
+                // raced again
+                if (m2 >= m1 * (1.0f - kTieMargin)) {
+                    JitRates r;
+#pragma unroll
+                    for (int j = 0; j < JM; ++j) r.a[j] = a[j];
+                    jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
+                }
+                const KeyTop top = key_top(m1);
+#pragma unroll
+                for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
+            }
+            mism += (jb != jk);
             JitCoef coef;
             jit_coef(X, kr, a, h, coef);
             // The walk's divisions by a0 (tau = E0/a0 and d tau/d a0 = -tau/a0) take one approximate
