@@ -427,41 +427,15 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
 // epilogue warps write a tile while the next one is multiplied. Warp 0 loads (TMA), warp 1 issues tcgen05.mma, warps
 // 2 to 5 read TMEM lanes 32 (warp % 4) ... and store. BN (a multiple of 16 up to 256) is the launch's: the width that
 // takes the fewest rounds of the SMs times columns (sw_tile_columns).
-// CL = 2: the two CTAs of a cluster take the tiles of two neighbouring row blocks and the same columns; each loads half
-// of the B tile into both (multicast), so that an SM asks L2 for 30 KB per K block instead of 44. A stage is free once
-// both CTAs' MMAs have read it (their commits arrive at both).
-// 4096 x 4096 x 4096: 126 us with one tile per CTA and the epilogue after it, 116 persistent, 113 with
-// clusters; 4,500 cubed (rows that do not fill lines): 228, 235 and 168.
+// 4096 x 4096 x 4096: 126 -> 116 us (one tile per CTA, 128 x 256, the epilogue after the tile), bound by the operand
+// reads from L2 (44 KB per SM and K block of 64).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// a TMA load that lands at the same place in every CTA of `mask` and counts on the barrier there
-__device__ __forceinline__ void tma_load_2d_multicast(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar,
-                                                      uint16_t mask)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, %3}], "
-        "[%4], %5;" ::"r"(smem_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar)), "h"(mask)
-        : "memory");
-}
-__device__ __forceinline__ void tc_commit_multicast(uint64_t *bar, uint16_t mask)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_addr(bar)),
-        "h"(mask)
-        : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
-
 constexpr int kPsThreads = 192;
-template <int CL>
 __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const __grid_constant__ CUtensorMap mapA,
                                                                            const __grid_constant__ CUtensorMap mapB,
                                                                            int M, int N, int K, int BN, int tiles_m,
@@ -478,9 +452,6 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile int *s_ok = reinterpret_cast<int *>(s_tmem + 1);
     const int nkb = (K + 63) / 64;
-    // row blocks in clusters of CL: tile t of the walk is (row block CL (t % tiles_m) + rank, column block t / tiles_m)
-    const int rank = CL == 1 ? 0 : (int)(blockIdx.x % CL), first = (int)(blockIdx.x / CL), step = (int)(gridDim.x / CL);
-    constexpr uint16_t kAll = (uint16_t)((1u << CL) - 1);
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(s_tmem)), "r"(512)
@@ -490,7 +461,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
     if (tid == 0) {
         for (int b = 0; b < kSwStages; ++b) {
             mbar_init(&full[b], 1);
-            mbar_init(&empty[b], CL);
+            mbar_init(&empty[b], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -500,7 +471,6 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
     }
     tc_fence_before();
     __syncthreads();
-    if (CL > 1) cluster_sync_all();  // the peers' barriers are set up before anything arrives at them
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     auto give_up = [&]() {
@@ -512,8 +482,8 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
         if (lane == 0) {
             int c = 0;  // K blocks loaded so far, over all tiles
             bool ok = true;
-            for (int t = first; t < tiles && ok; t += step) {
-                const int m0 = (t % tiles_m * CL + rank) * 128, n0 = t / tiles_m * BN;
+            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+                const int m0 = t % tiles_m * 128, n0 = t / tiles_m * BN;
                 for (int kb = 0; kb < nkb; ++kb, ++c) {
                     const int st = c % kSwStages, round = c / kSwStages;
                     ok = (round == 0 || mbar_wait_bounded(&empty[st], (round - 1) & 1, kWaitLimit)) && *s_ok;
@@ -521,12 +491,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
                     unsigned char *stage = sw + st * kSwStage;
                     mbar_arrive_expect_tx(&full[st], (uint32_t)(kSwTileA + BN * 128));
                     tma_load_2d(stage, &mapA, kb * 64, m0, &full[st]);
-                    if (CL == 1) {
-                        tma_load_2d(stage + kSwTileA, &mapB, kb * 64, n0, &full[st]);
-                    } else {
-                        const int part = rank * (BN / CL);
-                        tma_load_2d_multicast(stage + kSwTileA + part * 128, &mapB, kb * 64, n0 + part, &full[st], kAll);
-                    }
+                    tma_load_2d(stage + kSwTileA, &mapB, kb * 64, n0, &full[st]);
                 }
             }
             if (!ok) {
@@ -534,10 +499,6 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
                 // the copies in flight land before the CTA exits (each wait bounded)
                 for (int q = max(0, c - kSwStages); q < c; ++q)
                     mbar_wait_bounded(&full[q % kSwStages], (q / kSwStages) & 1, kWaitLimit);
-            } else {
-                // and so do the arrivals at this CTA's barriers, the peer's among them
-                for (int q = max(0, c - kSwStages); q < c; ++q)
-                    if (!mbar_wait_bounded(&empty[q % kSwStages], (q / kSwStages) & 1, kWaitLimit)) give_up();
             }
         }
     } else if (warp == 1) {
@@ -545,7 +506,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
             int c = 0, it = 0;
             bool ok = true;
-            for (int t = first; t < tiles && ok; t += step, ++it) {
+            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
                 const int buf = it & 1;
                 ok = (it < 2 || mbar_wait_bounded(&acc_empty[buf], ((it >> 1) - 1) & 1, kWaitLimit)) && *s_ok;
                 if (!ok) break;
@@ -561,9 +522,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk)
                         tc_mma(acc, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
-                    // the stage is free once these MMAs have read it
-                    if (CL == 1) tc_commit(&empty[st]);
-                    else tc_commit_multicast(&empty[st], kAll);
+                    tc_commit(&empty[st]);  // the stage is free once these MMAs have read it
                 }
                 if (ok) tc_commit(&acc_full[buf]);
             }
@@ -571,7 +530,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
         }
     } else {
         int it = 0;
-        for (int t = first; t < tiles; t += step, ++it) {
+        for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
             const int buf = it & 1, quad = warp & 3;
             bool ok = true;
             if (lane == 0) ok = mbar_wait_bounded(&acc_full[buf], (it >> 1) & 1, kWaitLimit);
@@ -579,7 +538,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
             ok = __all_sync(0xffffffffu, ok && *s_ok);
             if (!ok) break;
             tc_fence_after();
-            const int row = (t % tiles_m * CL + rank) * 128 + 32 * quad + lane, n0 = t / tiles_m * BN;
+            const int row = t % tiles_m * 128 + 32 * quad + lane, n0 = t / tiles_m * BN;
             const uint32_t base = tmem + (uint32_t)(256 * buf) + ((uint32_t)(32 * quad) << 16);
             const bool wide = (ldd % 4) == 0 && (reinterpret_cast<uintptr_t>(D) & 15) == 0;
             for (int c16 = 0; c16 < BN / 16; ++c16) {
@@ -613,7 +572,6 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
     __syncwarp();
     tc_fence_before();
     __syncthreads();
-    if (CL > 1) cluster_sync_all();  // a peer may still load into this CTA or arrive at its barriers
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
@@ -735,33 +693,25 @@ static int sw_split(int M, int N, int K, int *per)
 
 constexpr int kGemmSms = 152;
 
-// Rounds of the SMs (clusters of cl row blocks, one per cl SMs) that tiles of bn columns take.
-static int64_t sw_rounds(int M, int N, int cl, int bn)
+// Columns of a tile of the persistent kernel: the multiple of 16 that takes the fewest rounds of one tile per SM times
+// the columns of a tile (48 more stand for a tile's fixed cost); ties take the wider tile. Below 128 columns the
+// instruction's time no longer falls with its width. 4096 x 4096: 224 columns, 608 tiles, exactly four rounds.
+static int sw_tile_columns(int M, int N)
 {
-    const int64_t tiles = (((M + 127) / 128 + cl - 1) / cl) * (int64_t)((N + bn - 1) / bn);
-    return (tiles + kGemmSms / cl - 1) / (kGemmSms / cl);
-}
-
-// Columns of a tile of the persistent kernel: the multiple of 16 that takes the fewest rounds times the columns of a tile
-// (48 more stand for a tile's fixed cost); ties take the wider tile. Below 128 columns the instruction's time no longer
-// falls with its width. Measured: 4096 cubed 224 columns 113 us (256: 117, 192: 131); 3000 cubed 256: 56 us (160: 65);
-// 4500 cubed 224: 168 us (256: 175).
-static int sw_tile_columns(int M, int N, int cl)
-{
+    const int64_t tm = (M + 127) / 128;
     int best = 256;
-    for (int bn = 256; bn >= 128; bn -= 16)
-        if (sw_rounds(M, N, cl, bn) * (bn + 48) < sw_rounds(M, N, cl, best) * (best + 48)) best = bn;
+    int64_t best_cost = INT64_MAX;
+    for (int bn = 256; bn >= 128; bn -= 16) {
+        const int64_t tiles = tm * ((N + bn - 1) / bn), cost = (tiles + kGemmSms - 1) / kGemmSms * (bn + 48);
+        if (cost < best_cost) {
+            best_cost = cost;
+            best = bn;
+        }
+    }
     return best;
 }
 
-// Pairs of row blocks where the tiles take more than one round; a single round of lone CTAs starts sooner
-// (2048 cubed: 23.0 us against 24.2, 4000 x 500 x 2000: 19.0 against 20.7).
-static int sw_cluster(int M, int N)
-{
-    return sw_rounds(M, N, 1, sw_tile_columns(M, N, 1)) > 1 && M > 128 ? 2 : 1;
-}
-
-static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, int bn, int cl,
+static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, int bn,
                                         const float *bias, float *D, int ldd, double *work, int k_split, int per,
                                         int *err, cudaStream_t st)
 {
@@ -775,9 +725,7 @@ static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap
     if (dev >= 64 || !(attr_set.load() & (1ull << dev))) {
         e = cudaFuncSetAttribute(tc_gemm_sw128_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tc_gemm_persistent_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tc_gemm_persistent_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            e = cudaFuncSetAttribute(tc_gemm_persistent_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         if (dev < 64) attr_set.fetch_or(1ull << dev);
     }
@@ -788,23 +736,10 @@ static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap
         const int64_t n = (int64_t)M * N;
         tc_splitk_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(work, k_split, M, N, bias, D, ldd);
     } else {
-        const int groups_m = (tiles_m + cl - 1) / cl;
-        const int64_t tiles = (int64_t)groups_m * tiles_n;
+        const int64_t tiles = (int64_t)tiles_m * tiles_n;
         if (tiles > INT32_MAX - kGemmSms) return cudaErrorInvalidValue;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3((unsigned)(cl * std::min<int64_t>(tiles, kGemmSms / cl)));
-        cfg.blockDim = dim3(kPsThreads);
-        cfg.dynamicSmemBytes = smem;
-        cfg.stream = st;
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = (unsigned)cl;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        e = cudaLaunchKernelEx(&cfg, cl == 1 ? tc_gemm_persistent_kernel<1> : tc_gemm_persistent_kernel<2>, ma, mb, M, N, K,
-                               bn, groups_m, (int)tiles, bias, D, ldd, err);
-        if (e != cudaSuccess) return e;
+        tc_gemm_persistent_kernel<<<(unsigned)std::min<int64_t>(tiles, kGemmSms), kPsThreads, smem, st>>>(
+            ma, mb, M, N, K, bn, tiles_m, (int)tiles, bias, D, ldd, err);
     }
     return cudaGetLastError();
 }
@@ -894,11 +829,10 @@ extern "C" ssa_status ssa_bf16_gemm(const uint16_t *A, const uint16_t *B, int32_
     // with the caller's work buffer K is split where the output tiles fill few SMs
     int per = (K + 63) / 64;
     const int k_split = work && work_words > 0 ? sw_split(M, N, K, &per) : 1;
-    const int cl = k_split > 1 ? 1 : sw_cluster(M, N);
-    const int bn = k_split > 1 ? kSwBN : sw_tile_columns(M, N, cl);
+    const int bn = k_split > 1 ? kSwBN : sw_tile_columns(M, N);
     CUtensorMap ma, mb;
-    if (!tc_make_map_sw128(&ma, A, M, K, lda, 128) || !tc_make_map_sw128(&mb, B, N, K, ldb, bn / cl))
+    if (!tc_make_map_sw128(&ma, A, M, K, lda, 128) || !tc_make_map_sw128(&mb, B, N, K, ldb, bn))
         return set_error(SSA_ERR_INVALID_ARG, "tensor map encoding failed (alignment or driver entry point)");
-    cudaError_t e = tc_gemm_sw128_launch(ma, mb, M, N, K, bn, cl, bias, D, ldd, work, k_split, per, err_flag, st);
+    cudaError_t e = tc_gemm_sw128_launch(ma, mb, M, N, K, bn, bias, D, ldd, work, k_split, per, err_flag, st);
     return e == cudaSuccess ? SSA_OK : set_error(SSA_ERR_CUDA, cudaGetErrorString(e));
 }

@@ -458,6 +458,13 @@ def bf16_gemm(A: torch.Tensor, B: torch.Tensor, bias: torch.Tensor | None = None
     output tiles split K across the SMs."""
     if A.dtype != torch.bfloat16 or B.dtype != torch.bfloat16:
         raise SSAError("bf16_gemm takes bfloat16 operands")
+    if not A.is_cuda:
+        raise SSAError("bf16_gemm takes CUDA tensors")
+    with torch.cuda.device(A.device):  # the kernel runs where A lies, on that device's stream
+        return _bf16_gemm_here(A, B, bias, stream, split_k)
+
+
+def _bf16_gemm_here(A, B, bias, stream, split_k):
     M, K = A.shape
     N = B.shape[0]
     if B.device != A.device or tuple(B.shape) != (N, K):
@@ -466,7 +473,7 @@ def bf16_gemm(A: torch.Tensor, B: torch.Tensor, bias: torch.Tensor | None = None
     Bp, ldb = _tma_rows(B)
     D = torch.empty((M, N), dtype=torch.float32, device=A.device)
     err = torch.zeros(1, dtype=torch.int32, device=A.device)
-    b = None if bias is None else bias.to(torch.float32).contiguous()
+    b = None if bias is None else bias.to(device=A.device, dtype=torch.float32).contiguous()
     L = _lib.lib()
     words = int(L.ssa_bf16_gemm_work_words(M, N, K)) if split_k else 0
     work = torch.empty(max(words, 1), dtype=torch.float64, device=A.device) if words else None
