@@ -688,10 +688,11 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
     bt->unit_begin[1] = n_thread_units;
     bt->n_units[1] = (int)sorted.size() - n_thread_units;
     bt->n_red_blocks = (int)blk_item.size();
-    int maxNw = 1, maxMpw = 4;  // largest warp-variant network
+    int maxNw = 1, maxMpw = 4, maxMpq = 4;  // largest warp-variant network
     for (int it = 0; it < n_items; ++it)
         if (bt->variant[it] != 1) {
             maxNw = std::max(maxNw, bt->items[it].net->N);
+            maxMpq = std::max(maxMpq, bt->items[it].net->Mp);
             maxMpw = std::max(maxMpw, bt->soft ? bt->items[it].net->Mp : wide_len(bt->items[it].net->M));
         }
     const int maxNpad = (maxNw + 3) & ~3;
@@ -720,7 +721,9 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
                             : (ro == 0 ? (const void *)batch_adj_kernel<0, 32>
                                        : ro == 1 ? (const void *)batch_adj_kernel<1, 32> : (const void *)batch_adj_kernel<2, 32>)};
     for (int v = 0; v < 2; ++v) {
-        // a block of four warps, of fewer where the arrays of the largest network leave no room for four
+        // A block of four warps, of three where the padding of the arrays by word leaves no room for four. What a batch
+        // takes is set by four warps' arrays without that padding: about 7,200 species, well inside the sizes that have
+        // a second table region.
         const size_t words = kItemWords + (size_t)std::max(bt->x_words[v], bt->w_words[v]);
         bt->warps[v] = kBatchWarps;
         if (v == 1 && !bt->soft)
@@ -728,7 +731,9 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
         bt->fwd_smem[v] = (size_t)bt->warps[v] * (kItemWords + bt->x_words[v]) * 4;
         bt->adj_smem[v] = (size_t)bt->warps[v] * (kItemWords + bt->w_words[v]) * 4;
         if (bt->n_units[v] == 0) continue;
-        if (bt->fwd_smem[v] > (size_t)limit || bt->adj_smem[v] > (size_t)limit)
+        const size_t unpadded = kItemWords + 2 * (size_t)maxNpad + 4 * (size_t)maxMpq;
+        if (bt->fwd_smem[v] > (size_t)limit || bt->adj_smem[v] > (size_t)limit ||
+            (v == 1 && !bt->soft && 4 * kBatchWarps * unpadded > (size_t)limit))
             return set_error(SSA_ERR_UNSUPPORTED, "a network in the batch is too large for the batch kernels");
         int per_sm_f = 0, per_sm_a = 0;
         CUDA_TRY_B(cudaFuncSetAttribute(fk[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bt->fwd_smem[v]));
