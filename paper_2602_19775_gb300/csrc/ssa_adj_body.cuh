@@ -53,7 +53,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
     const uint64_t gid = p.traj_offset + (uint64_t)i;
     const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32);
     const uint32_t key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
-    const float invT = p.invT;
+    const float invT = p.invT, invT_q = weight_factor(invT);
     const float *gl = p.dl_dobs + i * p.dl_stride;
 
     int row_cached = -1;
@@ -207,7 +207,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 float wr[MC];
 #pragma unroll
                 for (int j = 0; j < MC; ++j) {
-                    const float q = ex2_approx(top.lg2(lr[j]) * invT);
+                    const float q = ex2_approx(top.lg2(lr[j]) * invT_q);
                     lr[j] = q;
                     wr[j] = stoich_dot(s_rx[j], s_st, lam, B);
                     Z += q;
@@ -225,7 +225,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 }
             } else {
                 for (int j = 0; j < M; ++j) {
-                    const float q = ex2_approx(top.lg2(qbuf[j * B]) * invT);
+                    const float q = ex2_approx(top.lg2(qbuf[j * B]) * invT_q);
                     qbuf[j * B] = q;
                     if (q > 0.0f) {
                         Z += q;

@@ -241,6 +241,9 @@ __device__ __forceinline__ KeyTop key_top(float m)
     t.lg2_top = m > 0.0f ? lg2_approx(m * t.scale) : 0.0f;
     return t;
 }
+// The factor of the log2 keys in the soft weights: 1/T, or at an infinite T the smallest normal number, under which every
+// reaction with a positive key still weighs 1 and one with key 0 still weighs 0.
+__device__ __forceinline__ float weight_factor(float invT) { return fmaxf(invT, 0x1p-126f); }
 // Two keys within this of each other, relatively, count as a possible tie (a key is a few units in the last place
 // off, and so is the comparison of products that decides the race).
 constexpr float kTieMargin = 0x1p-15f;

@@ -837,7 +837,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
         __syncwarp();
         const uint64_t gid = p.traj_offset + (uint64_t)i;
         const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-        const float invT = p.invT;
+        const float invT = p.invT, invT_q = weight_factor(invT);
         const float *gl = p.dl_dobs + i * p.dl_stride;
         int row_cached = -1;
         uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                 each_species([&](int c, int s) {
                     const float rp = key[s + 1], rd = key[nd + s + 1];
                     near += (rp >= top_edge) + (rd >= top_edge);
-                    const float q1 = ex2_approx(top.lg2(rp) * invT), q2 = ex2_approx(top.lg2(rd) * invT);
+                    const float q1 = ex2_approx(top.lg2(rp) * invT_q), q2 = ex2_approx(top.lg2(rd) * invT_q);
                     Zp += q1 + q2;
                     Wp = fmaf(q1 - q2, lam(c), Wp);
                     if (NS > 0) {

@@ -871,7 +871,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
     warp_propensities_all<true>(tab, X, ad);
     const uint64_t gid = p.traj_offset + (uint64_t)i;
     const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-    const float invT = p.invT;
+    const float invT = p.invT, invT_q = weight_factor(invT);
     const float *gl = p.dl_dobs + i * p.dl_stride;
     int row_cached = -1;
     uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -1009,7 +1009,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         near += qv[q] >= top_edge;
-                        qv[q] = ex2_approx(top.lg2(qv[q]) * invT);
+                        qv[q] = ex2_approx(top.lg2(qv[q]) * invT_q);
                         const int4 en = el[32 * q];
                         float w = ent_change(en.x) * at(en.x);
                         w = __fmaf_rn(ent_change(en.y), at(en.y), w);
