@@ -887,6 +887,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                 const KeyTop top = key_top(rmax);
                 const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
                 const bool k_tops = key[jk + 1] >= top_edge;
+                if (NS == 0) __syncwarp();  // every lane has read that key before its owner puts a weight in its place
                 // pass 2: soft-sample weights q_j = (key_j / largest)^(1/T), Z = sum q, W = sum q w with
                 // w_j = +lam_s (production of s) or -lam_s (degradation of s)
                 float Zp = 0.0f, Wp = 0.0f;
