@@ -17,7 +17,8 @@
 // commits each stage to an mbarrier that frees it; warp 0 allocates the TMEM columns; after the
 // last commit every warp reads its 32 TMEM lanes (tcgen05.ld 32x32b) for the epilogue.
 // Terms either share one accumulator or keep one each (`separate`); separate accumulators are
-// summed in binary64 in the epilogue. Every wait is bounded and reports a timeout in `err`.
+// summed in binary64 in the epilogue. Every wait is bounded and reports a timeout in `err`; a CTA that gives up waits
+// (again bounded) for its own copies and tensor-core instructions in flight before it frees its TMEM and exits.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -31,6 +32,13 @@ namespace ssa {
 namespace {
 
 constexpr int kErrTcTimeout = 8;
+
+// Polls of a wait inside the pipelines; a build for tests sets 0, and every product gives up at once. The waits for what
+// is in flight keep kWaitLimit.
+#ifndef SSA_TC_WAIT_LIMIT
+#define SSA_TC_WAIT_LIMIT kWaitLimit
+#endif
+constexpr uint32_t kPipeWait = SSA_TC_WAIT_LIMIT;
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int x, int y, uint64_t *bar)
 {
@@ -118,9 +126,9 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
     constexpr int kTileB = NT * 64 * 2;
     const int stage_bytes = args.n_a * kTileA + args.n_b * kTileB;
     unsigned char *stage0 = tc_smem;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(tc_smem + 2 * stage_bytes);  // full[2], empty[2]
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + 4);
-    int *s_ok = reinterpret_cast<int *>(bars + 5);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(tc_smem + 2 * stage_bytes);  // full[2], empty[2], drain
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(bars + 5);
+    int *s_ok = reinterpret_cast<int *>(bars + 6);
 
     const int m0 = blockIdx.x * 128, n0 = blockIdx.y * NT;
     const int n_acc = args.separate ? args.n_terms : 1;
@@ -138,7 +146,7 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int b = 0; b < 4; ++b) mbar_init(&bars[b], 1);
+        for (int b = 0; b < 5; ++b) mbar_init(&bars[b], 1);
         *s_ok = 1;
     }
     tc_fence_before();
@@ -163,13 +171,15 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
         };
         bool ok = true;
         issue(0);
+        int issued = 1;
         for (int ch = 0; ch < n_chunks && ok; ++ch) {
             if (ch + 1 < n_chunks) {
-                if (ch + 1 >= 2) ok = mbar_wait_bounded(&bars[2 + ((ch + 1) & 1)], ((ch - 1) >> 1) & 1, kWaitLimit);
+                if (ch + 1 >= 2) ok = mbar_wait_bounded(&bars[2 + ((ch + 1) & 1)], ((ch - 1) >> 1) & 1, kPipeWait);
                 if (!ok) break;
                 issue(ch + 1);
+                ++issued;
             }
-            ok = mbar_wait_bounded(&bars[ch & 1], (ch >> 1) & 1, kWaitLimit);
+            ok = mbar_wait_bounded(&bars[ch & 1], (ch >> 1) & 1, kPipeWait);
             if (!ok) break;
             tc_fence_after();
             unsigned char *st = stage0 + (ch & 1) * stage_bytes;
@@ -187,12 +197,14 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_kernel(const __grid_constant__
             }
             tc_commit(&bars[2 + (ch & 1)]);
         }
-        if (ok) ok = mbar_wait_bounded(&bars[2 + ((n_chunks - 1) & 1)], ((n_chunks - 1) >> 1) & 1, kWaitLimit);
+        if (ok) ok = mbar_wait_bounded(&bars[2 + ((n_chunks - 1) & 1)], ((n_chunks - 1) >> 1) & 1, kPipeWait);
         if (!ok) {
             atomicOr(args.err, kErrTcTimeout);
-            // let anything still in flight land before the CTA releases its TMEM and exits
-            mbar_wait_bounded(&bars[2 + ((n_chunks - 1) & 1)], ((n_chunks - 1) >> 1) & 1, kWaitLimit);
             *s_ok = 0;
+            // what is in flight ends before the CTA releases its TMEM and exits
+            for (int q = max(0, issued - 2); q < issued; ++q) mbar_wait_bounded(&bars[q & 1], (q >> 1) & 1, kWaitLimit);
+            tc_commit(&bars[4]);
+            mbar_wait_bounded(&bars[4], 0, kWaitLimit);
         }
     }
     tc_fence_before();
@@ -354,9 +366,10 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
 
     if (tid == 0) {
         // TMA producer: wait for the stage to be free, then load both operands of k block kb
-        for (int kb = 0; kb < nkb; ++kb) {
+        int kb = 0;
+        for (; kb < nkb; ++kb) {
             const int st = kb % kSwStages, round = kb / kSwStages;
-            if (round > 0 && !mbar_wait_bounded(&empty[st], (round - 1) & 1, kWaitLimit)) {
+            if (round > 0 && !mbar_wait_bounded(&empty[st], (round - 1) & 1, kPipeWait)) {
                 atomicOr(err, kErrTcTimeout);
                 *s_ok = 0;
                 break;
@@ -367,13 +380,16 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
             tma_load_2d(stage, &mapA, (kb0 + kb) * 64, m0, &full[st]);
             tma_load_2d(stage + kSwTileA, &mapB, (kb0 + kb) * 64, n0, &full[st]);
         }
+        // the copies in flight land before the CTA exits, also where the MMA thread no longer waits for them
+        for (int q = max(0, kb - kSwStages); q < kb; ++q)
+            mbar_wait_bounded(&full[q % kSwStages], (q / kSwStages) & 1, kWaitLimit);
     } else if (tid == 32) {
         // MMA issuer: four K = 16 steps per block, advancing the descriptors by 32 bytes inside the atom
         const uint32_t idesc = tc_idesc(128, kSwBN);
         bool ok = true;
         for (int kb = 0; kb < nkb && ok; ++kb) {
             const int st = kb % kSwStages, round = kb / kSwStages;
-            ok = mbar_wait_bounded(&full[st], round & 1, kWaitLimit) && *(volatile int *)s_ok;
+            ok = mbar_wait_bounded(&full[st], round & 1, kPipeWait) && *(volatile int *)s_ok;
             if (!ok) break;
             tc_fence_after();
             const unsigned char *stage = sw + st * kSwStage;
@@ -383,11 +399,11 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
                 tc_mma(tmem, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), idesc, (kb > 0 || kk > 0) ? 1u : 0u);
             tc_commit(&empty[st]);  // the stage is free once these MMAs have read it
         }
-        if (ok) tc_commit(done);
-        else {
+        if (!ok) {
             atomicOr(err, kErrTcTimeout);
             *(volatile int *)s_ok = 0;
         }
+        tc_commit(done);  // also of a product given up: what was issued of it ends before the TMEM is freed
     }
     __syncwarp();
     // epilogue: wait for the last MMA, then every warp reads its 32 TMEM lanes
@@ -449,7 +465,8 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
     uint64_t *empty = full + kSwStages;
     uint64_t *acc_full = empty + kSwStages;  // [2]
     uint64_t *acc_empty = acc_full + 2;      // [2], one arrival per epilogue warp
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(acc_empty + 2);
+    uint64_t *drain = acc_empty + 2;         // every MMA issued has ended
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *s_ok = reinterpret_cast<int *>(s_tmem + 1);
     const int nkb = (K + 63) / 64;
 
@@ -467,6 +484,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 4);
         }
+        mbar_init(drain, 1);
         *s_ok = 1;
     }
     tc_fence_before();
@@ -486,7 +504,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
                 const int m0 = t % tiles_m * 128, n0 = t / tiles_m * BN;
                 for (int kb = 0; kb < nkb; ++kb, ++c) {
                     const int st = c % kSwStages, round = c / kSwStages;
-                    ok = (round == 0 || mbar_wait_bounded(&empty[st], (round - 1) & 1, kWaitLimit)) && *s_ok;
+                    ok = (round == 0 || mbar_wait_bounded(&empty[st], (round - 1) & 1, kPipeWait)) && *s_ok;
                     if (!ok) break;
                     unsigned char *stage = sw + st * kSwStage;
                     mbar_arrive_expect_tx(&full[st], (uint32_t)(kSwTileA + BN * 128));
@@ -494,12 +512,10 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
                     tma_load_2d(stage + kSwTileA, &mapB, kb * 64, n0, &full[st]);
                 }
             }
-            if (!ok) {
-                give_up();
-                // the copies in flight land before the CTA exits (each wait bounded)
-                for (int q = max(0, c - kSwStages); q < c; ++q)
-                    mbar_wait_bounded(&full[q % kSwStages], (q / kSwStages) & 1, kWaitLimit);
-            }
+            if (!ok) give_up();
+            // the copies in flight land before the CTA exits, also where the MMA warp no longer waits for them
+            for (int q = max(0, c - kSwStages); q < c; ++q)
+                mbar_wait_bounded(&full[q % kSwStages], (q / kSwStages) & 1, kWaitLimit);
         }
     } else if (warp == 1) {
         if (lane == 0) {
@@ -508,13 +524,13 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
             bool ok = true;
             for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
                 const int buf = it & 1;
-                ok = (it < 2 || mbar_wait_bounded(&acc_empty[buf], ((it >> 1) - 1) & 1, kWaitLimit)) && *s_ok;
+                ok = (it < 2 || mbar_wait_bounded(&acc_empty[buf], ((it >> 1) - 1) & 1, kPipeWait)) && *s_ok;
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(256 * buf);
                 for (int kb = 0; kb < nkb; ++kb, ++c) {
                     const int st = c % kSwStages;
-                    ok = mbar_wait_bounded(&full[st], (c / kSwStages) & 1, kWaitLimit) && *s_ok;
+                    ok = mbar_wait_bounded(&full[st], (c / kSwStages) & 1, kPipeWait) && *s_ok;
                     if (!ok) break;
                     tc_fence_after();
                     const unsigned char *stage = sw + st * kSwStage;
@@ -527,13 +543,16 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
                 if (ok) tc_commit(&acc_full[buf]);
             }
             if (!ok) give_up();
+            // no MMA reads shared memory or writes TMEM after this, whichever warp gave up
+            tc_commit(drain);
+            if (!mbar_wait_bounded(drain, 0, kWaitLimit)) give_up();
         }
     } else {
         int it = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {
             const int buf = it & 1, quad = warp & 3;
             bool ok = true;
-            if (lane == 0) ok = mbar_wait_bounded(&acc_full[buf], (it >> 1) & 1, kWaitLimit);
+            if (lane == 0) ok = mbar_wait_bounded(&acc_full[buf], (it >> 1) & 1, kPipeWait);
             if (!ok) give_up();
             ok = __all_sync(0xffffffffu, ok && *s_ok);
             if (!ok) break;
