@@ -54,6 +54,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
     const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32);
     const uint32_t key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
     const float invT = p.invT, invT_q = weight_factor(invT);
+    const bool hot = hot_weights(invT);
     const float *gl = p.dl_dobs + i * p.dl_stride;
 
     int row_cached = -1;
@@ -120,7 +121,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
             const int jk = event_at(k);
             float a0 = 0.0f, E0, m1 = 0.0f, m2 = 0.0f;
             int jb = -1;
-            float ar[MC > 0 ? MC : 1], lr[MC > 0 ? MC : 1];
+            float ar[MC > 0 ? MC : 1], lr[MC > 0 ? MC : 1], lg2_max = -CUDART_INF_F;  // of log2 keys (hot)
             // pass 1: the forward's propensities and a0; the race's keys a_j / E_j with the two largest
             auto enter = [&](float key, int j) {
                 jb = key > m1 ? j : jb;
@@ -157,6 +158,10 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                     const float key = (a * sc_key) * inv_exp_of_word(word_of(cache, q & 3));
                     enter(key, j);
                     qbuf[j * B] = key;
+                    if (hot) {
+                        qbuf[j * B] = key_log2(a, inv_exp_of_word(word_of(cache, q & 3)));
+                        lg2_max = fmaxf(lg2_max, qbuf[j * B]);
+                    }
                 }
             }
             // the recorded reaction won the race if its key is the largest by more than the keys' error; near ties are
@@ -205,9 +210,13 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
             float Z = 0.0f, Wq = 0.0f;
             if constexpr (MC > 0) {
                 float wr[MC];
+                if (hot) {
+#pragma unroll
+                    for (int j = 0; j < MC; ++j) lg2_max = fmaxf(lg2_max, key_log2(ar[j], E[j + 1]));
+                }
 #pragma unroll
                 for (int j = 0; j < MC; ++j) {
-                    const float q = ex2_approx(top.lg2(lr[j]) * invT_q);
+                    const float q = ex2_approx((hot ? key_log2(ar[j], E[j + 1]) - lg2_max : top.lg2(lr[j])) * invT_q);
                     lr[j] = q;
                     wr[j] = stoich_dot(s_rx[j], s_st, lam, B);
                     Z += q;
@@ -225,7 +234,7 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
                 }
             } else {
                 for (int j = 0; j < M; ++j) {
-                    const float q = ex2_approx(top.lg2(qbuf[j * B]) * invT_q);
+                    const float q = ex2_approx((hot ? qbuf[j * B] - lg2_max : top.lg2(qbuf[j * B])) * invT_q);
                     qbuf[j * B] = q;
                     if (q > 0.0f) {
                         Z += q;

@@ -380,12 +380,14 @@ __device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const floa
     const float a0 = warp_sum(a0p);
     rmax = warp_max_nonneg(rmax);
     E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
-    if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(rounds, a, k, z, a0, key);
+    const bool hot = hot_weights(p.invT);
+    if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f) || hot) rmax = warp_keys_scaled(rounds, a, k, z, a0, hot, key);
+    const float invT_q = hot ? 8.0f * p.invT : p.invT;
     const KeyTop top = key_top(rmax);
     float Zp = 0.0f;
     for (int c = 0; c < rounds; ++c) {
         const float4 kv = key4[32 * c + lane];
-        auto weight = [&](float v) { return ex2_approx(top.lg2(v) * p.invT); };
+        auto weight = [&](float v) { return ex2_approx(top.lg2(v) * invT_q); };
         const float4 q = make_float4(weight(kv.x), weight(kv.y), weight(kv.z), weight(kv.w));
         key4[32 * c + lane] = q;
         Zp += (q.x + q.y) + (q.z + q.w);
@@ -837,7 +839,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
         __syncwarp();
         const uint64_t gid = p.traj_offset + (uint64_t)i;
         const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-        const float invT = p.invT, invT_q = weight_factor(invT);
+        const float invT = p.invT, invT_q = weight_factor(hot_weights(invT) ? 8.0f * invT : invT);
         const float *gl = p.dl_dobs + i * p.dl_stride;
         int row_cached = -1;
         uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -882,7 +884,8 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                     key4[b] = kv;
                 }
                 rmax = warp_max_nonneg(rmax);
-                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f)) rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, key);
+                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f) || hot_weights(invT))
+                    rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, hot_weights(invT), key);
                 __syncwarp();
                 const KeyTop top = key_top(rmax);
                 const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest

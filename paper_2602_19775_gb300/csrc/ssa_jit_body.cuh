@@ -608,6 +608,9 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
     float invT[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) invT[t] = NT == 1 ? p.invT : p.invT_multi[t];
+    bool hot = false;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) hot |= hot_weights(invT[t]);
     const float *gl = p.dl_dobs + i * p.dl_stride;
 
     // The walk's loads are issued well before their use (a load consumed where it is issued stalls the
@@ -745,9 +748,17 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
                     for (int j = 0; j < JM; ++j) r.a[j] = a[j];
                     jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
                 }
-                const KeyTop top = key_top(m1);
+                if (hot) {
+                    float lg2_top = -CUDART_INF_F;
 #pragma unroll
-                for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
+                    for (int j = 0; j < JM; ++j) lg2_top = fmaxf(lg2_top, lg2_key[j] = key_log2(a[j], E[j + 1]));
+#pragma unroll
+                    for (int j = 0; j < JM; ++j) lg2_key[j] -= lg2_top;
+                } else {
+                    const KeyTop top = key_top(m1);
+#pragma unroll
+                    for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
+                }
             }
             mism += (jb != jk);
             JitCoef coef;

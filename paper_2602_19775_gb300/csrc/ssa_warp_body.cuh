@@ -826,9 +826,32 @@ __device__ __forceinline__ void warp_soft_adj_body(const AdjParams &p, const int
 }
 
 // The keys of a step whose a0 lies where a_j / E_j could leave the binary32 range, scaled by a power of two (all
-// that follows uses ratios of keys); returns the largest.
-static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *ad, int k, WarpNoise z, float a0, float *rj)
+// that follows uses ratios of keys); returns the largest. hot (hot_weights): the eighth root of each key's ratio to the
+// largest instead, from its log2, so that no positive key flushes; the weights' exponent is then 8/T.
+static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *ad, int k, WarpNoise z, float a0, bool hot,
+                                                      float *rj)
 {
+    if (hot) {
+        const int lane = threadIdx.x & 31;
+        float top = -CUDART_INF_F;
+        for (int c = 0; c < rounds; ++c) {
+            const uint4 r = philox4x32_10(make_uint4((uint32_t)(32 * c + lane), (uint32_t)k, z.c2, z.c3), z.key0, z.key1);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int w = 4 * (32 * c + lane) + q;
+                rj[w] = key_log2(fmaxf(ad[w], 0.0f), inv_exp_of_word(word_of(r, q)));
+                top = fmaxf(top, rj[w]);
+            }
+        }
+        top = warp_max(top);
+        for (int c = 0; c < rounds; ++c)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int w = 4 * (32 * c + lane) + q;
+                rj[w] = ex2_approx((rj[w] - top) * 0.125f);
+            }
+        return 1.0f;
+    }
     const float sc = key_scale(a0);
     const int lane = threadIdx.x & 31;
     float rmax = 0.0f;
@@ -871,7 +894,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
     warp_propensities_all<true>(tab, X, ad);
     const uint64_t gid = p.traj_offset + (uint64_t)i;
     const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-    const float invT = p.invT, invT_q = weight_factor(invT);
+    const float invT = p.invT, invT_q = weight_factor(hot_weights(invT) ? 8.0f * invT : invT);
     const float *gl = p.dl_dobs + i * p.dl_stride;
     int row_cached = -1;
     uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -959,7 +982,8 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             const float a0 = warp_sum(a0p);
             const float E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
             rmax = warp_max_nonneg(rmax);
-            if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, rj);
+            if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f) || hot_weights(invT))
+                rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, hot_weights(invT), rj);
             __syncwarp();
             const KeyTop top = key_top(rmax);
             const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
