@@ -587,6 +587,9 @@ struct AdjParams {
     float invT_multi[4];
     const int4 *wtab;  // as in FwdParams
     uint32_t wtab_bytes;
+    // BIN readout with a gradient per trajectory, specialised kernels: bits of the chunks of bins whose sums the launch
+    // has shared memory for, 0: none
+    int chunk_shift;
 };
 
 
@@ -650,12 +653,12 @@ __device__ __forceinline__ void bin_held_run(const FwdParams &p, int64_t i, int 
 // run by broadcast instead of passing it from a lane's local array by shuffles. The ninth entry takes the held tail.
 // Ion channel (262,144 trajectories, 800 bins, recorded): 345 -> 320 us with 44% fewer instructions; what is left are
 // the stores (839 MB, 250 us at half the copy rate; 16-byte stores make no difference).
-constexpr int kRunWords = 2 + kBinMaxObs;
 struct BinRunsShared {
     int n, slots;
-    int *col;    // word w of run q at col[(q * kRunWords + w) * stride]
+    int *col;    // word w of run q at col[(q * words + w) * stride]
+    int words;   // of a run: 2 and one per observable
     int stride;  // threads of the block
-    __device__ __forceinline__ int *word(int q, int w, int lanes_off = 0) const { return col + (q * kRunWords + w) * stride + lanes_off; }
+    __device__ __forceinline__ int *word(int q, int w, int lanes_off = 0) const { return col + (q * words + w) * stride + lanes_off; }
     template <class XF>
     __device__ __forceinline__ void put(int lo, int hi, const XF &value, int no)
     {

@@ -8,6 +8,7 @@
 // in the same order), so both give the same trajectories bit for bit; only the table lookups and
 // the shared-memory traffic go away. The generated source is compiled once per distinct network and
 // process (cached for its lifetime) for sm_103a and loaded as a context-independent CUDA library.
+#include <algorithm>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -339,6 +340,18 @@ const JitKernels *jit_load(const ssa_network *net, bool soft, std::string &why)
 const JitKernels *jit_kernels(const ssa_network *net, std::string &why) { return jit_load(net, false, why); }
 const JitKernels *jit_soft_kernels(const ssa_network *net, std::string &why) { return jit_load(net, true, why); }
 
+// Bits of the chunk size for the bin readout's chunk sums, 0: none. One observable, a gradient per trajectory, at most
+// kChunkRows chunks a row (28 KB a block), a chunk no wider than a warp's loads.
+constexpr int kChunkRows = 56;
+static int jit_chunk_shift(const AdjParams &p, int readout)
+{
+    if (readout != SSA_READOUT_BIN || p.bin_prefix || p.n_obs != 1 || p.S < 32) return 0;
+    int shift = 4;
+    while (((p.S - 1) >> shift) >= kChunkRows) ++shift;
+    const bool pieces = (p.S & 3) == 0 && (p.dl_stride & 3) == 0 && (reinterpret_cast<uintptr_t>(p.dl_dobs) & 15) == 0;
+    return shift <= (pieces ? 7 : 5) ? shift : 0;
+}
+
 cudaError_t jit_launch_forward(const JitKernels *k, const FwdParams &p, int readout, bool record, int selector,
                                int block, cudaStream_t st)
 {
@@ -347,15 +360,19 @@ cudaError_t jit_launch_forward(const JitKernels *k, const FwdParams &p, int read
     void *args[] = {const_cast<FwdParams *>(&p)};
     const int r = readout;  // SSA_READOUT_HOLD, _LINEAR, _BIN index the tables
     const cudaKernel_t f = selector == SSA_SELECT_DIRECT ? k->fwd_direct[r] : k->fwd[r][record ? 1 : 0];
-    return cudaLaunchKernel(reinterpret_cast<const void *>(f), dim3(grid), dim3((unsigned)block), args, 0, st);
+    const size_t smem = readout == SSA_READOUT_BIN ? (size_t)4 * (kBinRuns + 1) * (2 + p.n_obs) * block : 0;
+    return cudaLaunchKernel(reinterpret_cast<const void *>(f), dim3(grid), dim3((unsigned)block), args, smem, st);
 }
 
 cudaError_t jit_launch_backward(const JitKernels *k, const AdjParams &p, int readout, int block, int64_t grid,
                                 cudaStream_t st)
 {
     if (grid == 0) return cudaSuccess;
-    void *args[] = {const_cast<AdjParams *>(&p)};
-    const size_t smem = (size_t)4 * p.M * block;
+    AdjParams q = p;
+    q.chunk_shift = jit_chunk_shift(p, readout);
+    void *args[] = {&q};
+    const size_t rows = q.chunk_shift ? ((p.S - 1) >> q.chunk_shift) + 1 : 0;
+    const size_t smem = (size_t)4 * std::max<size_t>(p.M, rows) * block;
     return cudaLaunchKernel(reinterpret_cast<const void *>(k->adj[readout]),
                             dim3((unsigned)grid), dim3((unsigned)block), args, smem, st);
 }

@@ -156,10 +156,13 @@ __device__ __forceinline__ void jit_lam_add2(float (&lam)[JN], float (&lo)[JN], 
         if (s == sp) acc2(lam[s], lo[s], v);
 }
 
-// The bin readout's held runs in shared memory, one column per thread (kJitFwdBlock threads at most).
-#define SSA_JIT_BIN_RUNS(R)                                                                               \
-    __shared__ int s_runs[(R) == SSA_READOUT_BIN ? (kBinRuns + 1) * kRunWords * kJitFwdBlock : 1];        \
-    BinRunsShared bruns{0, 0, s_runs + threadIdx.x, kJitFwdBlock}
+// The bin readout's held runs in shared memory, one column per thread; the launch gives (kBinRuns + 1) (2 + n_obs) words
+// a thread, no more than the call's observables need. One observable, 2A <-> B, 16,384 trajectories x 1,500 bins: 1.53 ms
+// with the runs in local arrays, 1.82 with room for four observables (13.8 KB a block, which set the resident blocks), 1.45
+// so; the relaxed forward, 65,536 x 50, 0.678, 0.719 and 0.679.
+#define SSA_JIT_BIN_RUNS()                                                                                \
+    extern __shared__ int s_runs[];                                                                       \
+    BinRunsShared bruns{0, 0, s_runs + threadIdx.x, 2 + p.n_obs, (int)blockDim.x}
 
 // BIN readout state of a forward: cleared integrals, observed species (0 where the list is invalid)
 __device__ __forceinline__ void jit_bin_init(const FwdParams &p, bool bad_obs, float (&bacc)[kBinMaxObs],
@@ -251,7 +254,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     float E0, E0n, c[JM], cn[JM];
     jit_noise(E0, c, 0u, c2, c3, key0, key1);
     float bacc[kBinMaxObs];
-    SSA_JIT_BIN_RUNS(READOUT);
+    SSA_JIT_BIN_RUNS();
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     const bool few = p.n_obs <= kBinMaxObs;  // their species in registers
@@ -420,7 +423,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
     uint4 r = philox4x32_10(make_uint4(0u, 0u, c2, c3), key0, key1);
     float E0 = neg_log_unit(u01(r.x)), U1 = u01(r.y);
     float bacc[kBinMaxObs];
-    SSA_JIT_BIN_RUNS(READOUT);
+    SSA_JIT_BIN_RUNS();
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
@@ -505,22 +508,12 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
 // every trajectory's row, formed before the walk by the warp's lanes side by side along the row; the walk then sums
 // the whole bins of an interval from chunks and the loose bins at its ends. Summed bin by bin in the walk, a row per
 // lane, the loads set the time. A row that starts and ends on 16 bytes is read in 16-byte pieces, others (of up to
-// 32 bins a chunk) by the float. s_chunk [kChunkRows][kJitAdjBlock]; from kChunkMinBins bins on (below, a row is a line
-// or two and the intervals hold no long runs).
+// 32 bins a chunk) by the float. s_chunk [rows][kJitAdjBlock], a row a chunk; whether they are formed is the launch's
+// choice (jit_chunk_shift). Where intervals hold few bins they neither cost nor save (2A <-> B, 200 bins in 250 steps).
 // Ion channel, 262,144 trajectories x 800 bins, the adjoint: 2,050 us bin by bin; 800 with the sum of every interval
 // formed by the warp beforehand (a reduction per interval and row); 395 so.
+// The chunk sums share the block sums' memory (28 KB of their own, also where unused: relaxed 2A <-> B 0.79 -> 0.86 ms).
 constexpr int kJitAdjBlock = 128;
-constexpr int kChunkRows = 56, kChunkMinBins = 32;
-
-// bits of the chunk size for S bins, 0: no chunks
-__device__ __forceinline__ int jit_chunk_shift(const AdjParams &p)
-{
-    if (p.bin_prefix || p.n_obs != 1 || p.S < kChunkMinBins || (int)blockDim.x != kJitAdjBlock) return 0;
-    int shift = 4;
-    while (((p.S - 1) >> shift) >= kChunkRows) ++shift;
-    const bool pieces = (p.S & 3) == 0 && (p.dl_stride & 3) == 0 && (reinterpret_cast<uintptr_t>(p.dl_dobs) & 15) == 0;
-    return shift <= (pieces ? 7 : 5) ? shift : 0;
-}
 
 __device__ __forceinline__ void jit_bin_chunk_sums(const AdjParams &p, int64_t i, bool active, int shift, float *s_chunk)
 {
@@ -1008,7 +1001,7 @@ __device__ __forceinline__ void jit_fwd_soft(const FwdParams &p)
     float E[NQ], En[NQ];
     step_noise<NQ>(E, 0u, c2, c3, key0, key1);
     float bacc[kBinMaxObs];
-    SSA_JIT_BIN_RUNS(READOUT);
+    SSA_JIT_BIN_RUNS();
     int osp[kBinMaxObs];
     jit_bin_init(p, bad_obs, bacc, osp);
     auto xobs = [&](int c) { return jit_fsel(X, osp[c]); };
@@ -1239,7 +1232,8 @@ __device__ __forceinline__ void jit_adj_soft_traj(const AdjParams &p, const floa
 template <int READOUT, bool SOFT, bool WIDE = false, int NT = 1>
 __device__ __forceinline__ void jit_adj(const AdjParams &p)
 {
-    extern __shared__ float s_dA[];  // [NT][JM][blockDim.x] (WIDE: binary64)
+    // the block's sums [NT][JM][blockDim.x] (WIDE: binary64); during the walk of a bin readout the chunk sums
+    extern __shared__ float s_dA[];
     __shared__ int s_len[256], s_perm[256];
     SSA_JIT_CHANGES();
     const int B = blockDim.x, tid = threadIdx.x;
@@ -1271,11 +1265,10 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
     int sc = 0;
     BinChunks chunks{nullptr, 0, kJitAdjBlock};
     if constexpr (READOUT == SSA_READOUT_BIN) {
-        __shared__ float s_chunk[kChunkRows * kJitAdjBlock];
-        chunks.shift = jit_chunk_shift(p);
-        if (chunks.shift) {
-            jit_bin_chunk_sums(p, i, active, chunks.shift, s_chunk);
-            chunks.sum = s_chunk + tid;
+        if (p.chunk_shift) {  // the launch has made room for them
+            chunks.shift = p.chunk_shift;
+            jit_bin_chunk_sums(p, i, active, chunks.shift, s_dA);
+            chunks.sum = s_dA + tid;
         }
     }
     if (active) {
@@ -1300,6 +1293,7 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
         }
         return;
     }
+    if constexpr (READOUT == SSA_READOUT_BIN) __syncthreads();  // every warp is done with its chunk sums
 #pragma unroll
     for (int t = 0; t < NT; ++t)
 #pragma unroll
