@@ -35,7 +35,7 @@ __device__ __forceinline__ float stoich_dot(const int4 rx, const int *s_st, cons
 // Per-trajectory body of the thread adjoint. X, lam, dlam point at this trajectory's column (stride B);
 // q and dA at its column of the runtime-size buffers [M][B] (MC == 0); dAr holds the per-reaction
 // adjoints in registers when MC > 0.
-template <int READOUT, int MC>
+template <int READOUT, int MC, bool HOT>
 __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *s_rx, const int *s_st,
                                                 const float *s_k, int *X, float *lam, float *dlam, float *qbuf,
                                                 float *dA, const int B, const int64_t i, const int st,
@@ -53,8 +53,8 @@ __device__ __forceinline__ void thread_adj_body(const AdjParams &p, const int4 *
     const uint64_t gid = p.traj_offset + (uint64_t)i;
     const uint32_t c2 = (uint32_t)gid, c3 = (uint32_t)(gid >> 32);
     const uint32_t key0 = (uint32_t)p.seed, key1 = (uint32_t)(p.seed >> 32);
-    const float invT = p.invT, invT_q = weight_factor(invT);
-    const bool hot = hot_weights(invT);
+    const float invT = p.invT, invT_q = HOT ? weight_factor(invT) : invT;
+    constexpr bool hot = HOT;
     const float *gl = p.dl_dobs + i * p.dl_stride;
 
     int row_cached = -1;

@@ -46,6 +46,7 @@ struct JitKernels;
 bool jit_eligible(const ssa_network *net);
 const JitKernels *jit_kernels(const ssa_network *net, std::string &why);
 const JitKernels *jit_soft_kernels(const ssa_network *net, std::string &why);
+const JitKernels *jit_hot_kernels(const ssa_network *net, std::string &why);
 cudaError_t jit_launch_forward(const JitKernels *k, const FwdParams &p, int readout, bool record, int selector,
                                int block, cudaStream_t st);
 cudaError_t jit_launch_backward(const JitKernels *k, const AdjParams &p, int readout, int block, int64_t grid,
@@ -596,10 +597,11 @@ extern "C" ssa_status ssa_forward_replay(const ssa_network *net, const float *lo
 }
 
 // Everything ssa_backward and ssa_backward_wide share: argument checks, the kernel variant and launch
-// shape, and the adjoint parameters (the per-block sums are left unset).
+// shape, and the adjoint parameters (the per-block sums are left unset). hot: a temperature of the walk is one at which
+// hot_weights holds.
 static ssa_status backward_setup(ssa_run *run, const float *dl_dobs, int64_t dl_traj_stride, float temperature,
-                                 const void *dl_dlog_rates, cudaStream_t st, AdjParams &p, const JitKernels *&jit,
-                                 int &block, int64_t &grid)
+                                 const void *dl_dlog_rates, cudaStream_t st, bool hot, AdjParams &p,
+                                 const JitKernels *&jit, int &block, int64_t &grid)
 {
     if (run && dl_traj_stride != 0 && dl_traj_stride < (int64_t)run->S * run->n_obs)
         return fail(SSA_ERR_INVALID_ARG, "dl_traj_stride must be 0 or >= n_samples * n_obs");
@@ -621,7 +623,7 @@ static ssa_status backward_setup(ssa_run *run, const float *dl_dobs, int64_t dl_
         return fail(SSA_ERR_INVALID_ARG, "the gradient of a soft forward is taken at the forward's temperature");
     if (run->variant == 2) {
         std::string why;
-        jit = soft ? jit_soft_kernels(net, why) : jit_kernels(net, why);
+        jit = soft ? jit_soft_kernels(net, why) : hot ? jit_hot_kernels(net, why) : jit_kernels(net, why);
         if (!jit) return fail(SSA_ERR_STATE, "specialised kernels unavailable: %s", why.c_str());
         block = kJitAdjBlock;
         grid = (run->n_traj + block - 1) / block;
@@ -686,7 +688,8 @@ extern "C" ssa_status ssa_backward(ssa_run *run, const float *dl_dobs, int64_t d
     const JitKernels *jit = nullptr;
     int block = 0;
     int64_t grid = 0;
-    const ssa_status s = backward_setup(run, dl_dobs, dl_traj_stride, temperature, dl_dlog_rates, st, p, jit, block, grid);
+    const ssa_status s = backward_setup(run, dl_dobs, dl_traj_stride, temperature, dl_dlog_rates, st,
+                                        hot_weights(1.0f / temperature), p, jit, block, grid);
     if (s != SSA_OK) return s;
     const ssa_network *net = run->net;
     unsigned char *ws = run->ws;
@@ -741,7 +744,10 @@ extern "C" ssa_status ssa_backward_multi(ssa_run *run, const float *dl_dobs, int
         const JitKernels *jit = nullptr;
         int block = 0;
         int64_t grid = 0;
-        const ssa_status s = backward_setup(run, dl_dobs, dl_traj_stride, temperatures[t0], out, st, p, jit, block, grid);
+        bool hot = false;
+        for (int t = 0; t < nt; ++t) hot |= hot_weights(1.0f / temperatures[t0 + t]);
+        const ssa_status s =
+            backward_setup(run, dl_dobs, dl_traj_stride, temperatures[t0], out, st, hot, p, jit, block, grid);
         if (s != SSA_OK) return s;
         for (int t = 0; t < nt; ++t) p.invT_multi[t] = 1.0f / temperatures[t0 + t];
         p.partial = reinterpret_cast<float *>(ws + run->L.partial);
@@ -766,7 +772,7 @@ extern "C" ssa_status ssa_backward_wide(ssa_run *run, const float *dl_dobs, int6
     const JitKernels *jit = nullptr;
     int block = 0;
     int64_t grid = 0;
-    const ssa_status s = backward_setup(run, dl_dobs, dl_traj_stride, temperature, dl_dlog_rates, st, p, jit, block, grid);
+    const ssa_status s = backward_setup(run, dl_dobs, dl_traj_stride, temperature, dl_dlog_rates, st, false, p, jit, block, grid);
     if (s != SSA_OK) return s;
     const ssa_network *net = run->net;
     unsigned char *ws = run->ws;

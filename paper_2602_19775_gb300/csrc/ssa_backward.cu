@@ -23,7 +23,7 @@
 
 namespace ssa {
 
-template <int READOUT, int MC>
+template <int READOUT, int MC, bool HOT>
 __global__ void __launch_bounds__(256) adj_thread_kernel(const AdjParams p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(256) adj_thread_kernel(const AdjParams p)
         for (int j = 0; j < M; ++j) s_dA[j * B + tid] = 0.0f;
 
     if (active)
-        thread_adj_body<READOUT, MC>(p, s_rx, s_st, s_k, s_X + tid, s_lam + tid, s_dlam + tid, s_q + tid, s_dA + tid, B, i,
+        thread_adj_body<READOUT, MC, HOT>(p, s_rx, s_st, s_k, s_X + tid, s_lam + tid, s_dlam + tid, s_q + tid, s_dA + tid, B, i,
                                      st, dAr);
     if (MC > 0) {
 #pragma unroll
@@ -135,7 +135,7 @@ __global__ void map_params64_kernel(const double *dA, int M, const int *rate_ind
 template <int R, int MC>
 static cudaError_t launch_adj_t(const AdjParams &p, int block, size_t smem, int64_t grid, cudaStream_t st)
 {
-    auto kern = adj_thread_kernel<R, MC>;
+    auto kern = hot_weights(p.invT) ? adj_thread_kernel<R, MC, true> : adj_thread_kernel<R, MC, false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, block, smem, st>>>(p);

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
     }
 }
 
-template <int READOUT, int MC>
+template <int READOUT, int MC, bool HOT>
 __device__ __forceinline__ void batch_adj_thread_unit(const BatchItem &b, const BatchUnit &u, float *wsm)
 {
     const AdjParams &p = b.a;
@@ -196,8 +196,8 @@ __device__ __forceinline__ void batch_adj_thread_unit(const BatchItem &b, const 
     if (lane < u.count) stt = p.status[i];
     const bool active = stt == SSA_TRAJ_OK || stt == SSA_TRAJ_ABSORBED || stt == SSA_TRAJ_STEP_CAP;
     if (active)
-        thread_adj_body<READOUT, MC>(p, rx, st, p.k_rates, X + lane, lam + lane, dlam + lane, nullptr, nullptr, 32, i,
-                                     stt, dAr);
+        thread_adj_body<READOUT, MC, HOT>(p, rx, st, p.k_rates, X + lane, lam + lane, dlam + lane, nullptr, nullptr, 32, i,
+                                          stt, dAr);
     // fixed-order sum over the lanes (butterfly: every lane holds the same bits), lane 0 writes the slot
     float *slot = p.partial + b.slot_off + (int64_t)u.slot * p.M;
 #pragma unroll
@@ -207,7 +207,7 @@ __device__ __forceinline__ void batch_adj_thread_unit(const BatchItem &b, const 
     }
 }
 
-template <int READOUT, int VARIANT, bool SOFT = false>
+template <int READOUT, int VARIANT, bool SOFT = false, bool HOT = false>
 __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWarpBlocks) batch_adj_kernel(const BatchItem *items, const BatchUnit *units,
                                                                     int n_units, int *counter, int w_words)
 {
@@ -224,10 +224,10 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
         const BatchItem &b = s_items[wib];
         if constexpr (VARIANT == 1) {
             switch (b.mc) {
-            case 2: batch_adj_thread_unit<READOUT, 2>(b, u, wsm); break;
-            case 4: batch_adj_thread_unit<READOUT, 4>(b, u, wsm); break;
-            case 8: batch_adj_thread_unit<READOUT, 8>(b, u, wsm); break;
-            default: batch_adj_thread_unit<READOUT, 16>(b, u, wsm); break;
+            case 2: batch_adj_thread_unit<READOUT, 2, HOT>(b, u, wsm); break;
+            case 4: batch_adj_thread_unit<READOUT, 4, HOT>(b, u, wsm); break;
+            case 8: batch_adj_thread_unit<READOUT, 8, HOT>(b, u, wsm); break;
+            default: batch_adj_thread_unit<READOUT, 16, HOT>(b, u, wsm); break;
             }
         } else {
             const AdjParams &p = b.a;
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(32 * kBatchWarps, VARIANT == 1 ? 1 : kBatchWar
                     const int64_t i = u.traj_begin + c;
                     const int stt = p.status[i];
                     if (stt == SSA_TRAJ_OK || stt == SSA_TRAJ_ABSORBED || stt == SSA_TRAJ_STEP_CAP)
-                        warp_adj_body<READOUT>(p, tab, X, lam, aj, lj, ct, dA, i, stt);
+                        warp_adj_body<READOUT, HOT>(p, tab, X, lam, aj, lj, ct, dA, i, stt);
                     __syncwarp();
                 }
             }
@@ -324,6 +324,8 @@ __global__ void batch_params_kernel(const BatchItem *items, int n_items)
 // =============================================================================================
 using namespace ssa;
 
+using BatchAdjKernel = void (*)(const BatchItem *, const BatchUnit *, int, int *, int);
+
 struct ssa_batch {
     std::vector<ssa_batch_item> items;
     std::vector<int> variant, mc, K;
@@ -346,6 +348,7 @@ struct ssa_batch {
     int fwd_blocks[2] = {0, 0}, adj_blocks[2] = {0, 0};
     size_t fwd_smem[2] = {0, 0}, adj_smem[2] = {0, 0};
     int warps[2] = {0, 0};  // per block
+    bool hot() const { return hot_weights(1.0f / temperature); }
     std::vector<BatchItem> h_items;
     cudaGraphExec_t graph = nullptr;
     bool ready = false;
@@ -537,6 +540,22 @@ extern "C" ssa_status ssa_batch_set_soft(ssa_batch *bt, int32_t soft)
 
 extern "C" size_t ssa_batch_workspace_bytes(const ssa_batch *bt) { return bt ? batch_layout(bt).total : 0; }
 
+// the adjoint kernel of a variant (soft: of the relaxed model, whose keys keep their range at every temperature)
+template <int R>
+static BatchAdjKernel batch_adj_of_r(int variant, bool soft, bool hot)
+{
+    if (variant == 1) return hot ? batch_adj_kernel<R, 1, false, true> : batch_adj_kernel<R, 1, false, false>;
+    if (soft) return batch_adj_kernel<R, 32, true>;
+    return hot ? batch_adj_kernel<R, 32, false, true> : batch_adj_kernel<R, 32, false, false>;
+}
+
+static const void *batch_adj_of(int readout, int variant, bool soft, bool hot)
+{
+    return (const void *)(readout == 0   ? batch_adj_of_r<0>(variant, soft, hot)
+                          : readout == 1 ? batch_adj_of_r<1>(variant, soft, hot)
+                                         : batch_adj_of_r<2>(variant, soft, hot));
+}
+
 static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cudaStream_t st)
 {
     const BatchLayout L = batch_layout(bt);
@@ -713,13 +732,7 @@ static ssa_status batch_build(ssa_batch *bt, void *workspace, size_t bytes, cuda
                                                  : (const void *)batch_fwd_kernel<2, 32, true>)
                             : (ro == 0 ? (const void *)batch_fwd_kernel<0, 32>
                                        : ro == 1 ? (const void *)batch_fwd_kernel<1, 32> : (const void *)batch_fwd_kernel<2, 32>)};
-    const void *ak[2] = {ro == 0 ? (const void *)batch_adj_kernel<0, 1>
-                                 : ro == 1 ? (const void *)batch_adj_kernel<1, 1> : (const void *)batch_adj_kernel<2, 1>,
-                         sf ? (ro == 0 ? (const void *)batch_adj_kernel<0, 32, true>
-                                       : ro == 1 ? (const void *)batch_adj_kernel<1, 32, true>
-                                                 : (const void *)batch_adj_kernel<2, 32, true>)
-                            : (ro == 0 ? (const void *)batch_adj_kernel<0, 32>
-                                       : ro == 1 ? (const void *)batch_adj_kernel<1, 32> : (const void *)batch_adj_kernel<2, 32>)};
+    const void *ak[2] = {batch_adj_of(ro, 1, false, bt->hot()), batch_adj_of(ro, 32, sf, bt->hot())};
     for (int v = 0; v < 2; ++v) {
         // A block of four warps, of three where the padding of the arrays by word leaves no room for four. What a batch
         // takes is set by four warps' arrays without that padding: about 7,200 species, well inside the sizes that have
@@ -759,7 +772,7 @@ static void batch_launch_kernels(const ssa_batch *bt, cudaStream_t st)
     if (bt->n_units[0] > 0) {  // thread units: forward then adjoint
         batch_fwd_kernel<R, 1><<<bt->fwd_blocks[0], blk, bt->fwd_smem[0], st>>>(bt->d_items, u0, bt->n_units[0],
                                                                               bt->d_counters, bt->x_words[0]);
-        batch_adj_kernel<R, 1><<<bt->adj_blocks[0], blk, bt->adj_smem[0], st>>>(bt->d_items, u0, bt->n_units[0],
+        batch_adj_of_r<R>(1, false, bt->hot())<<<bt->adj_blocks[0], blk, bt->adj_smem[0], st>>>(bt->d_items, u0, bt->n_units[0],
                                                                               bt->d_counters + 1, bt->w_words[0]);
     }
     if (bt->n_units[1] > 0 && bt->soft) {  // warp units of a soft batch
@@ -770,7 +783,7 @@ static void batch_launch_kernels(const ssa_batch *bt, cudaStream_t st)
     } else if (bt->n_units[1] > 0) {  // warp units
         batch_fwd_kernel<R, 32><<<bt->fwd_blocks[1], blkw, bt->fwd_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
                                                                                bt->d_counters + 2, bt->x_words[1]);
-        batch_adj_kernel<R, 32><<<bt->adj_blocks[1], blkw, bt->adj_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
+        batch_adj_of_r<R>(32, false, bt->hot())<<<bt->adj_blocks[1], blkw, bt->adj_smem[1], st>>>(bt->d_items, u1, bt->n_units[1],
                                                                                bt->d_counters + 3, bt->w_words[1]);
     }
 }

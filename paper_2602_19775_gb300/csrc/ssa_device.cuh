@@ -245,8 +245,9 @@ __device__ __forceinline__ KeyTop key_top(float m)
     return t;
 }
 // A key below 2^-126 of the largest flushes to 0. Up to T = 5 it would weigh less than 2^-25 of the largest; above, the
-// weights are formed from log2 keys taken of the two factors apart, over all of the binary32 range.
-__device__ __forceinline__ bool hot_weights(float invT) { return invT < 0.2f; }
+// weights are formed from log2 keys taken of the two factors apart, over all of the binary32 range, by kernels of their
+// own (HOT): a test per step in the others cost them 2 to 6%.
+__host__ __device__ __forceinline__ bool hot_weights(float invT) { return invT < 0.2f; }
 __device__ __forceinline__ float key_log2(float a, float inv_E) { return __log2f(a) + __log2f(inv_E); }
 // The factor of the log2 keys in the soft weights: 1/T, or at an infinite T the smallest normal number, under which every
 // reaction with a positive key still weighs 1 and one with key 0 still weighs 0.

@@ -358,6 +358,7 @@ __device__ __forceinline__ void grn_soft_outputs(const GrnParams &p, const float
 
 // one soft step at step k from the propensities a: the race's keys a_j / E_j, then the unnormalised weights
 // q_j = (key_j / largest)^(1/T) in their place; returns a0 and sets E0 and invZ = 1/sum q
+template <bool HOT>
 __device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const float *a, float *key, int k,
                                                   const WarpNoise &z, int lane, float &E0, float &invZ)
 {
@@ -380,9 +381,8 @@ __device__ __forceinline__ float grn_soft_weights(const GrnParams &p, const floa
     const float a0 = warp_sum(a0p);
     rmax = warp_max_nonneg(rmax);
     E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
-    const bool hot = hot_weights(p.invT);
-    if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f) || hot) rmax = warp_keys_scaled(rounds, a, k, z, a0, hot, key);
-    const float invT_q = hot ? 8.0f * p.invT : p.invT;
+    if (HOT || !(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(rounds, a, k, z, a0, HOT, key);
+    const float invT_q = HOT ? 8.0f * p.invT : p.invT;
     const KeyTop top = key_top(rmax);
     float Zp = 0.0f;
     for (int c = 0; c < rounds; ++c) {
@@ -412,6 +412,7 @@ __device__ __forceinline__ void grn_soft_update(const GrnParams &p, const float 
 
 }  // namespace
 
+template <bool HOT>
 __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, float *obs, int record)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(128) grn_soft_fwd_kernel(const GrnParams p, fl
     while (!bad_input) {
         if (k >= p.max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
         float E0, invZ;
-        const float a0 = grn_soft_weights(p, a, q, k, noise, lane, E0, invZ);
+        const float a0 = grn_soft_weights<HOT>(p, a, q, k, noise, lane, E0, invZ);
         if (!(a0 < CUDART_INF_F)) { status = SSA_TRAJ_BAD_RATE; break; }
         if (a0 == 0.0f) { status = SSA_TRAJ_ABSORBED; break; }
         const float tau = waiting_time(E0, a0);
@@ -524,7 +525,7 @@ __host__ __device__ inline size_t grn_soft_adj_words(int nh, int no)
 
 // NS rounds of species (n_dyn <= 32 NS) read a step's weights and state into registers together, one wait for memory a
 // step; NS = 0: any number, read where they are used.
-template <int NS>
+template <int NS, bool HOT>
 __global__ void __launch_bounds__(128, 4) grn_soft_adj_kernel(const GrnParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -606,7 +607,7 @@ __global__ void __launch_bounds__(128, 4) grn_soft_adj_kernel(const GrnParams p)
                 if (kk < L) {
                     grn_soft_outputs(p, s_W2, s_b2, X, aO, lane);
                     float E0, invZ;
-                    grn_soft_weights(p, a, q, kk, noise, lane, E0, invZ);
+                    grn_soft_weights<HOT>(p, a, q, kk, noise, lane, E0, invZ);
                     for (int o = lane; o < no; o += 32) row[ndp + o] = aO[o];
                     for (int j = lane; j < M; j += 32) row[ndp + nop + j] = q[j + 1];
                     if (lane == 0) row[ndp + nop + Mq] = invZ;
@@ -744,7 +745,7 @@ __host__ __device__ inline size_t grn_adj_words(int nh, int no, bool shared_sums
 // six with the sums in shared memory 77.
 constexpr int kGrnAdjBlocks = 4;
 // NF: the first rounds of species that are full (n_dyn >= 32 NF).
-template <int NS, int NF>
+template <int NS, int NF, bool HOT>
 __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnParams p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -839,7 +840,7 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
         __syncwarp();
         const uint64_t gid = p.traj_offset + (uint64_t)i;
         const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-        const float invT = p.invT, invT_q = weight_factor(hot_weights(invT) ? 8.0f * invT : invT);
+        const float invT = p.invT, invT_q = HOT ? weight_factor(8.0f * invT) : invT;
         const float *gl = p.dl_dobs + i * p.dl_stride;
         int row_cached = -1;
         uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -884,8 +885,8 @@ __global__ void __launch_bounds__(128, kGrnAdjBlocks) grn_adj_kernel(const GrnPa
                     key4[b] = kv;
                 }
                 rmax = warp_max_nonneg(rmax);
-                if (!(rmax >= 0x1p-60f && rmax <= 0x1p120f) || hot_weights(invT))
-                    rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, hot_weights(invT), key);
+                if (HOT || !(rmax >= 0x1p-60f && rmax <= 0x1p120f))
+                    rmax = warp_keys_scaled(rounds, a, k, noise, rmax > 1.0f ? 0x1p110f : 0.0f, HOT, key);
                 __syncwarp();
                 const KeyTop top = key_top(rmax);
                 const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
@@ -1336,8 +1337,9 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
         p.invT = 1.0f / opts->temperature;
         const int wpb = grn_soft_warps(g);
         const size_t smem = grn_soft_fwd_smem(g, wpb);
-        GRN_CUDA_TRY(cudaFuncSetAttribute(grn_soft_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_soft_fwd_kernel<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
+        auto kern = hot_weights(p.invT) ? grn_soft_fwd_kernel<true> : grn_soft_fwd_kernel<false>;
+        GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(
             p, reinterpret_cast<float *>(obs_out), opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
@@ -1432,19 +1434,23 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     p.n_ckpt = L.n_ckpt;
     p.seg = soft ? reinterpret_cast<float *>(ws + L.soft_seg) : nullptr;
     const int wpb = soft ? grn_soft_warps(g) : grn_warps(g);
+    const bool hot = hot_weights(p.invT);
     const int64_t nblk = (n + wpb - 1) / wpb;
     float *red = reinterpret_cast<float *>(ws + L.red);
     if (n > 0 && soft) {
         const size_t smem = grn_soft_adj_smem(g, wpb);
-        auto kern = grn_sums_in_registers(g) ? grn_soft_adj_kernel<9> : grn_soft_adj_kernel<0>;
+        auto kern = grn_sums_in_registers(g) ? (hot ? grn_soft_adj_kernel<9, true> : grn_soft_adj_kernel<9, false>)
+                                             : (hot ? grn_soft_adj_kernel<0, true> : grn_soft_adj_kernel<0, false>);
         GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
         const size_t smem = grn_adj_smem(g, wpb);
         const int nd = g->n_dyn;
-        auto kern = !grn_sums_in_registers(g) ? grn_adj_kernel<0, 0>
-                    : nd > 192 ? grn_adj_kernel<9, 6> : nd > 96 ? grn_adj_kernel<6, 3> : grn_adj_kernel<3, 0>;
+        auto kern = !grn_sums_in_registers(g) ? (hot ? grn_adj_kernel<0, 0, true> : grn_adj_kernel<0, 0, false>)
+                    : nd > 192                ? (hot ? grn_adj_kernel<9, 6, true> : grn_adj_kernel<9, 6, false>)
+                    : nd > 96                 ? (hot ? grn_adj_kernel<6, 3, true> : grn_adj_kernel<6, 3, false>)
+                                              : (hot ? grn_adj_kernel<3, 0, true> : grn_adj_kernel<3, 0, false>);
         GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<(unsigned)nblk, 32 * wpb, smem, st>>>(p);
         GRN_CUDA_TRY(cudaGetLastError());

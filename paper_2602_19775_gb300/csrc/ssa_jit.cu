@@ -278,16 +278,17 @@ bool jit_eligible(const ssa_network *net)
 }
 
 namespace {
-// Kernels of `net` (soft: the soft-forward program of the same text), compiling and loading them on
+// Kernels of `net` (soft: the soft-forward program of the same text; hot: the adjoints at temperatures at which
+// hot_weights holds, their forwards' and wide walks' entries empty), compiling and loading them on
 // first use. Returns nullptr (with the reason in `why`) if the network is not eligible or compilation
 // failed.
-const JitKernels *jit_load(const ssa_network *net, bool soft, std::string &why)
+const JitKernels *jit_load(const ssa_network *net, bool soft, bool hot, std::string &why)
 {
     if (!jit_eligible(net)) {
         why = "network above the specialisation limits (24 species, 24 reactions, 96 stoichiometric entries)";
         return nullptr;
     }
-    const std::string src = (soft ? std::string("#define SSA_JIT_SOFT 1\n") : std::string()) + jit_source(net);
+    const std::string src = (soft ? "#define SSA_JIT_SOFT 1\n" : hot ? "#define SSA_JIT_HOT 1\n" : "") + jit_source(net);
     std::lock_guard<std::mutex> lock(g_jit_mu);
     auto f = g_jit_failed.find(src);
     if (f != g_jit_failed.end()) {
@@ -313,15 +314,15 @@ const JitKernels *jit_load(const ssa_network *net, bool soft, std::string &why)
     bool ok = true;
     for (int r = 0; r < 3; ++r) {
         const std::string base = std::string(rname[r]) + (soft ? "_soft" : "");
-        for (int rec = 0; rec < 2; ++rec) {
+        for (int rec = 0; rec < 2 && !hot; ++rec) {
             const std::string nm = "ssa_jit_fwd_" + base + (rec ? "_rec" : "");
             ok &= cudaLibraryGetKernel(&k.fwd[r][rec], lib, nm.c_str()) == cudaSuccess;
         }
         ok &= cudaLibraryGetKernel(&k.adj[r], lib, ("ssa_jit_adj_" + base).c_str()) == cudaSuccess;
-        if (!soft)
+        if (!soft && !hot)
             ok &= cudaLibraryGetKernel(&k.fwd_direct[r], lib, ("ssa_jit_fwd_" + base + "_direct").c_str()) == cudaSuccess;
         if (!soft && r < 2) {
-            ok &= cudaLibraryGetKernel(&k.adj_wide[r], lib, ("ssa_jit_adj_" + base + "_wide").c_str()) == cudaSuccess;
+            ok &= hot || cudaLibraryGetKernel(&k.adj_wide[r], lib, ("ssa_jit_adj_" + base + "_wide").c_str()) == cudaSuccess;
             for (int nt = 2; nt <= 3; ++nt)
                 ok &= cudaLibraryGetKernel(&k.adj_multi[r][nt - 2], lib,
                                            ("ssa_jit_adj_" + base + "_t" + std::to_string(nt)).c_str()) == cudaSuccess;
@@ -337,8 +338,9 @@ const JitKernels *jit_load(const ssa_network *net, bool soft, std::string &why)
 }
 }  // namespace
 
-const JitKernels *jit_kernels(const ssa_network *net, std::string &why) { return jit_load(net, false, why); }
-const JitKernels *jit_soft_kernels(const ssa_network *net, std::string &why) { return jit_load(net, true, why); }
+const JitKernels *jit_kernels(const ssa_network *net, std::string &why) { return jit_load(net, false, false, why); }
+const JitKernels *jit_soft_kernels(const ssa_network *net, std::string &why) { return jit_load(net, true, false, why); }
+const JitKernels *jit_hot_kernels(const ssa_network *net, std::string &why) { return jit_load(net, false, true, why); }
 
 // Bits of the chunk size for the bin readout's chunk sums, 0: none. One observable, a gradient per trajectory, at most
 // kChunkRows chunks a row (28 KB a block), a chunk no wider than a warp's loads.

@@ -601,9 +601,6 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
     float invT[NT];
 #pragma unroll
     for (int t = 0; t < NT; ++t) invT[t] = NT == 1 ? p.invT : p.invT_multi[t];
-    bool hot = false;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) hot |= hot_weights(invT[t]);
     const float *gl = p.dl_dobs + i * p.dl_stride;
 
     // The walk's loads are issued well before their use (a load consumed where it is issued stalls the
@@ -741,17 +738,17 @@ __device__ __forceinline__ void jit_adj_traj(const AdjParams &p, const float (&k
                     for (int j = 0; j < JM; ++j) r.a[j] = a[j];
                     jb = jit_race_exact(r, (uint32_t)k, c2, c3, key0, key1);
                 }
-                if (hot) {
-                    float lg2_top = -CUDART_INF_F;
+#ifdef SSA_JIT_HOT  // the program for temperatures at which hot_weights holds
+                float lg2_top = -CUDART_INF_F;
 #pragma unroll
-                    for (int j = 0; j < JM; ++j) lg2_top = fmaxf(lg2_top, lg2_key[j] = key_log2(a[j], E[j + 1]));
+                for (int j = 0; j < JM; ++j) lg2_top = fmaxf(lg2_top, lg2_key[j] = key_log2(a[j], E[j + 1]));
 #pragma unroll
-                    for (int j = 0; j < JM; ++j) lg2_key[j] -= lg2_top;
-                } else {
-                    const KeyTop top = key_top(m1);
+                for (int j = 0; j < JM; ++j) lg2_key[j] -= lg2_top;
+#else
+                const KeyTop top = key_top(m1);
 #pragma unroll
-                    for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
-                }
+                for (int j = 0; j < JM; ++j) lg2_key[j] = top.lg2(key[j]);
+#endif
             }
             mism += (jb != jk);
             JitCoef coef;
@@ -1314,6 +1311,7 @@ __device__ __forceinline__ void jit_adj(const AdjParams &p)
 }  // namespace ssa
 
 #ifndef SSA_JIT_SOFT
+#ifndef SSA_JIT_HOT
 extern "C" __global__ void __launch_bounds__(256) ssa_jit_fwd_hold(const ssa::FwdParams p)
 {
     ssa::jit_fwd<SSA_READOUT_HOLD, false>(p);
@@ -1350,6 +1348,7 @@ extern "C" __global__ void __launch_bounds__(256) ssa_jit_fwd_linear_direct(cons
 {
     ssa::jit_fwd_direct<SSA_READOUT_LINEAR>(p);
 }
+#endif
 extern "C" __global__ void __launch_bounds__(256) ssa_jit_adj_hold(const ssa::AdjParams p)
 {
     ssa::jit_adj<SSA_READOUT_HOLD, false>(p);
@@ -1378,6 +1377,7 @@ extern "C" __global__ void __launch_bounds__(256) ssa_jit_adj_linear_t3(const ss
 {
     ssa::jit_adj<SSA_READOUT_LINEAR, false, false, 3>(p);
 }
+#ifndef SSA_JIT_HOT
 extern "C" __global__ void __launch_bounds__(256) ssa_jit_adj_hold_wide(const ssa::AdjParams p)
 {
     ssa::jit_adj<SSA_READOUT_HOLD, false, true>(p);
@@ -1386,6 +1386,7 @@ extern "C" __global__ void __launch_bounds__(256) ssa_jit_adj_linear_wide(const 
 {
     ssa::jit_adj<SSA_READOUT_LINEAR, false, true>(p);
 }
+#endif
 #else  // the soft-forward program of the same network
 extern "C" __global__ void __launch_bounds__(256) ssa_jit_fwd_hold_soft(const ssa::FwdParams p)
 {

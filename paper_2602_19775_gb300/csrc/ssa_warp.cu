@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(256) adj_warp_soft_kernel(const AdjParams p, c
     }
 }
 
-template <int READOUT, bool STAGED>
+template <int READOUT, bool STAGED, bool HOT>
 __global__ void __launch_bounds__(128, kWarpAdjBlocks) adj_warp_kernel(const AdjParams p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(128, kWarpAdjBlocks) adj_warp_kernel(const Adj
     int st = -1;
     if (i < n) st = p.status[i];
     const bool active = st == SSA_TRAJ_OK || st == SSA_TRAJ_ABSORBED || st == SSA_TRAJ_STEP_CAP;
-    if (active) warp_adj_body<READOUT>(p, tab, X, lam, ad, rj, ct, dA, i, st);
+    if (active) warp_adj_body<READOUT, HOT>(p, tab, X, lam, ad, rj, ct, dA, i, st);
     __syncthreads();
     // fixed-order reduction over the block's warps
     for (int j = threadIdx.x; j < M; j += blockDim.x) {
@@ -249,13 +249,13 @@ cudaError_t launch_backward_warp_soft(const AdjParams &p, const int *upd, uint32
     return launch_adj_soft_w<1>(p, upd, upd_words, warps, smem, grid, st);
 }
 
-template <int R>
+template <int R, bool HOT>
 static cudaError_t launch_adj_w(const AdjParams &p, int warps, size_t limit, int64_t grid, cudaStream_t st)
 {
     const size_t own = (size_t)warps * (2 * ((p.N + 3) & ~3) + 4 * (size_t)wide_len(p.M)) * 4;
     const size_t full = own + staged_bytes(p.inc_off, p.k_bytes, p.wtab_bytes);
     const bool staged = full <= limit;
-    auto kern = staged ? adj_warp_kernel<R, true> : adj_warp_kernel<R, false>;
+    auto kern = staged ? adj_warp_kernel<R, true, HOT> : adj_warp_kernel<R, false, HOT>;
     const size_t smem = staged ? full : own;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -267,10 +267,14 @@ cudaError_t launch_backward_warp(const AdjParams &p, int readout, int warps, siz
                                  cudaStream_t st)
 {
     if (grid == 0) return cudaSuccess;
+    const bool hot = hot_weights(p.invT);
     switch (readout) {
-    case SSA_READOUT_HOLD: return launch_adj_w<0>(p, warps, limit, grid, st);
-    case SSA_READOUT_LINEAR: return launch_adj_w<1>(p, warps, limit, grid, st);
-    default: return launch_adj_w<2>(p, warps, limit, grid, st);
+    case SSA_READOUT_HOLD:
+        return hot ? launch_adj_w<0, true>(p, warps, limit, grid, st) : launch_adj_w<0, false>(p, warps, limit, grid, st);
+    case SSA_READOUT_LINEAR:
+        return hot ? launch_adj_w<1, true>(p, warps, limit, grid, st) : launch_adj_w<1, false>(p, warps, limit, grid, st);
+    default:
+        return hot ? launch_adj_w<2, true>(p, warps, limit, grid, st) : launch_adj_w<2, false>(p, warps, limit, grid, st);
     }
 }
 

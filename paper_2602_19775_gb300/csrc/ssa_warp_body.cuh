@@ -876,7 +876,7 @@ static __device__ __noinline__ float warp_keys_scaled(int rounds, const float *a
 // proportional to the count of each plain reactant, so lambda_s += (1/X_s) sum g_j over the reactions of s, a
 // homodimer's share carries (2 X - 1) / (X (X - 1)), and where a reactant is absent (a_j = 0) only the
 // waiting-time path remains, dL/da0 D_j. One division per species replaces two per reaction.
-template <int READOUT>
+template <int READOUT, bool HOT>
 __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab &tab, int *X, float *lam, float *ad,
                                               float *rj, float *ct, float *dA, const int64_t i, const int st)
 {
@@ -894,7 +894,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
     warp_propensities_all<true>(tab, X, ad);
     const uint64_t gid = p.traj_offset + (uint64_t)i;
     const WarpNoise noise{(uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)p.seed, (uint32_t)(p.seed >> 32)};
-    const float invT = p.invT, invT_q = weight_factor(hot_weights(invT) ? 8.0f * invT : invT);
+    const float invT = p.invT, invT_q = HOT ? weight_factor(8.0f * invT) : invT;
     const float *gl = p.dl_dobs + i * p.dl_stride;
     int row_cached = -1;
     uint4 row = make_uint4(0, 0, 0, 0), row_below = row;  // the log row below is loaded ahead of its use
@@ -982,8 +982,7 @@ __device__ __forceinline__ void warp_adj_body(const AdjParams &p, const WarpTab 
             const float a0 = warp_sum(a0p);
             const float E0 = neg_log_unit(u01(__shfl_sync(0xffffffffu, x0, 0)));
             rmax = warp_max_nonneg(rmax);
-            if (!(a0 >= 0x1p-60f && a0 <= 0x1p100f) || hot_weights(invT))
-                rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, hot_weights(invT), rj);
+            if (HOT || !(a0 >= 0x1p-60f && a0 <= 0x1p100f)) rmax = warp_keys_scaled(n_rounds, ad, k, noise, a0, HOT, rj);
             __syncwarp();
             const KeyTop top = key_top(rmax);
             const float top_edge = rmax * (1.0f - kTieMargin);  // keys from here on may be the largest
