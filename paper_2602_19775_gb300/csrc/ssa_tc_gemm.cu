@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(kPsThreads, 1) tc_gemm_persistent_kernel(const
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+            const uint32_t idesc = tc_idesc(128, BN);
             int c = 0, it = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++it) {
@@ -710,18 +710,16 @@ static int sw_split(int M, int N, int K, int *per)
     return (total + *per - 1) / *per;  // every split non-empty
 }
 
-constexpr int kGemmSms = 152;
-
 // Columns of a tile of the persistent kernel: the multiple of 16 that takes the fewest rounds of one tile per SM times
 // the columns of a tile (48 more stand for a tile's fixed cost); ties take the wider tile. Below 128 columns the
-// instruction's time no longer falls with its width. 4096 x 4096: 224 columns, 608 tiles, exactly four rounds.
-static int sw_tile_columns(int M, int N)
+// instruction's time no longer falls with its width. 4096 x 4096 on 152 SMs: 224 columns, 608 tiles, exactly four rounds.
+static int sw_tile_columns(int M, int N, int sms)
 {
     const int64_t tm = (M + 127) / 128;
     int best = 256;
     int64_t best_cost = INT64_MAX;
     for (int bn = 256; bn >= 128; bn -= 16) {
-        const int64_t tiles = tm * ((N + bn - 1) / bn), cost = (tiles + kGemmSms - 1) / kGemmSms * (bn + 48);
+        const int64_t tiles = tm * ((N + bn - 1) / bn), cost = (tiles + sms - 1) / sms * (bn + 48);
         if (cost < best_cost) {
             best_cost = cost;
             best = bn;
@@ -730,7 +728,7 @@ static int sw_tile_columns(int M, int N)
     return best;
 }
 
-static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, int bn,
+static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap &mb, int M, int N, int K, int bn, int sms,
                                         const float *bias, float *D, int ldd, double *work, int k_split, int per,
                                         int *err, cudaStream_t st)
 {
@@ -756,8 +754,8 @@ static cudaError_t tc_gemm_sw128_launch(const CUtensorMap &ma, const CUtensorMap
         tc_splitk_reduce_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(work, k_split, M, N, bias, D, ldd);
     } else {
         const int64_t tiles = (int64_t)tiles_m * tiles_n;
-        if (tiles > INT32_MAX - kGemmSms) return cudaErrorInvalidValue;
-        tc_gemm_persistent_kernel<<<(unsigned)std::min<int64_t>(tiles, kGemmSms), kPsThreads, smem, st>>>(
+        if (tiles > INT32_MAX - sms) return cudaErrorInvalidValue;
+        tc_gemm_persistent_kernel<<<(unsigned)std::min<int64_t>(tiles, sms), kPsThreads, smem, st>>>(
             ma, mb, M, N, K, bn, tiles_m, (int)tiles, bias, D, ldd, err);
     }
     return cudaGetLastError();
@@ -848,10 +846,14 @@ extern "C" ssa_status ssa_bf16_gemm(const uint16_t *A, const uint16_t *B, int32_
     // with the caller's work buffer K is split where the output tiles fill few SMs
     int per = (K + 63) / 64;
     const int k_split = work && work_words > 0 ? sw_split(M, N, K, &per) : 1;
-    const int bn = k_split > 1 ? kSwBN : sw_tile_columns(M, N);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return set_error(SSA_ERR_CUDA, cudaGetErrorString(e));
+    const int bn = k_split > 1 ? kSwBN : sw_tile_columns(M, N, sms);
     CUtensorMap ma, mb;
     if (!tc_make_map_sw128(&ma, A, M, K, lda, 128) || !tc_make_map_sw128(&mb, B, N, K, ldb, bn))
         return set_error(SSA_ERR_INVALID_ARG, "tensor map encoding failed (alignment or driver entry point)");
-    cudaError_t e = tc_gemm_sw128_launch(ma, mb, M, N, K, bn, bias, D, ldd, work, k_split, per, err_flag, st);
+    e = tc_gemm_sw128_launch(ma, mb, M, N, K, bn, sms, bias, D, ldd, work, k_split, per, err_flag, st);
     return e == cudaSuccess ? SSA_OK : set_error(SSA_ERR_CUDA, cudaGetErrorString(e));
 }
