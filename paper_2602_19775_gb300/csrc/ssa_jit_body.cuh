@@ -189,7 +189,7 @@ struct SampleStage {
     uint32_t *row;   // this thread's window in shared memory
     uint32_t *out;   // obs_out as 32-bit words
     int64_t base;    // first word of this trajectory's row
-    int n_obs, W, S;
+    int n_obs, W;
     int lo, cnt;     // the window holds samples lo .. lo + cnt - 1
 };
 
@@ -208,9 +208,9 @@ __device__ __forceinline__ void stage_own_flush(SampleStage &g)
     g.cnt = 0;
 }
 
-// one sample s (the next in order) of n_obs values
+// the next sample, n_obs values
 template <class VAL>
-__device__ __forceinline__ void stage_put(SampleStage &g, int s, const VAL &val)
+__device__ __forceinline__ void stage_put(SampleStage &g, const VAL &val)
 {
     uint32_t *w = g.row + g.cnt * g.n_obs;
     for (int c = 0; c < g.n_obs; ++c) w[c] = val(c);
@@ -262,7 +262,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     auto xobs = [&](int c) { return jit_xsel(X, osp[c]); };
     const bool staged = READOUT != SSA_READOUT_BIN && p.n_obs >= 1 && p.n_obs <= 4 && blockDim.x <= kJitFwdBlock;
     SampleStage stg{s_stage + threadIdx.x * kStageWords, static_cast<uint32_t *>(p.obs_out), i * p.S * p.n_obs,
-                    p.n_obs, staged ? kStageWords / p.n_obs : 1, p.S, 0, 0};
+                    p.n_obs, staged ? kStageWords / p.n_obs : 1, 0, 0};
 
     while (!bad_input) {
         if (k >= max_steps) { status = SSA_TRAJ_STEP_CAP; break; }
@@ -304,7 +304,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
                 while (s < p.S && gt_nonneg(t_next, thr)) {
                     if (READOUT == SSA_READOUT_HOLD) {
                         if (staged) {
-                            stage_put(stg, s, [&](int c) { return (uint32_t)jit_xsel(X, species(c)); });
+                            stage_put(stg, [&](int c) { return (uint32_t)jit_xsel(X, species(c)); });
                         } else {
                             int *o = static_cast<int *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                             for (int c = 0; c < p.n_obs; ++c) o[c] = jit_xsel(X, p.obs_sp[c]);
@@ -316,7 +316,7 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
                             return __fmaf_rn(alpha, (float)jit_dv(s_chg, jb, sp), (float)jit_xsel(X, sp));
                         };
                         if (staged) {
-                            stage_put(stg, s, [&](int c) { return __float_as_uint(lin(c)); });
+                            stage_put(stg, [&](int c) { return __float_as_uint(lin(c)); });
                         } else {
                             float *o = static_cast<float *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                             for (int c = 0; c < p.n_obs; ++c) o[c] = lin(c);
@@ -353,14 +353,14 @@ __device__ __forceinline__ void jit_fwd(const FwdParams &p)
     for (; READOUT != SSA_READOUT_BIN && s < p.S; ++s) {
         if (READOUT == SSA_READOUT_HOLD) {
             if (staged) {
-                stage_put(stg, s, [&](int c) { return (uint32_t)(bad_obs ? 0 : jit_xsel(X, p.obs_sp[c])); });
+                stage_put(stg, [&](int c) { return (uint32_t)(bad_obs ? 0 : jit_xsel(X, p.obs_sp[c])); });
             } else {
                 int *o = static_cast<int *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                 for (int c = 0; c < p.n_obs; ++c) o[c] = bad_obs ? 0 : jit_xsel(X, p.obs_sp[c]);
             }
         } else {
             if (staged) {
-                stage_put(stg, s, [&](int c) { return __float_as_uint(bad_obs ? 0.0f : (float)jit_xsel(X, p.obs_sp[c])); });
+                stage_put(stg, [&](int c) { return __float_as_uint(bad_obs ? 0.0f : (float)jit_xsel(X, p.obs_sp[c])); });
             } else {
                 float *o = static_cast<float *>(p.obs_out) + ((int64_t)i * p.S + s) * p.n_obs;
                 for (int c = 0; c < p.n_obs; ++c) o[c] = bad_obs ? 0.0f : (float)jit_xsel(X, p.obs_sp[c]);
