@@ -55,10 +55,11 @@ struct BatchUnit {
 
 constexpr int kBatchWarps = 4;
 constexpr int kBatchThreadMaxN = 16;  // thread variant inside a batch: N <= 16 and M <= 16
-// Resident blocks per SM the warp-unit kernels are compiled for (a tuning constant: more blocks hide more
-// latency, fewer let each trajectory run faster, which counts where one long trajectory ends a launch, and leave
-// more of the SM's 256 KB to L1, through which the batch kernels read their tables). 24 networks, 9,468
-// trajectories with up to 32,768 draws: 6 blocks 380 ms, 5 300, 4 240, 3 221.
+// Resident blocks per SM the warp-unit kernels are compiled for: more hide more latency, fewer let each trajectory run
+// faster, which counts where one long trajectory ends a launch, and leave more of the SM's 256 KB to L1, through which the
+// batch kernels read their tables. Milliseconds at 3, 4 and 5 blocks: 24 uneven networks (up to 32,768 draws) 177-191,
+// 174-184, 200-208; 12 of them x 512 trajectories to t = 1 32.0, 27.6, 32.6; 40 networks of 30 to 100 reactions x 512 33.2,
+// 27.4, 25.6 (bin readout 34.7, 29.6, 30.5).
 #ifndef SSA_BATCH_WARP_BLOCKS
 #define SSA_BATCH_WARP_BLOCKS 4
 #endif
