@@ -443,7 +443,8 @@ def _tma_rows(x: torch.Tensor):
     Anything else is copied into rows padded to 8 elements (the maps end at column K: the padding is never read).
     At 4096 x 4096 x 4096 the zeroed and copied operands took 90 of a call's 262 us."""
     rows, K = x.shape
-    if K > 0 and rows > 0 and x.stride(1) == 1 and x.stride(0) % 8 == 0 and x.stride(0) >= K and x.data_ptr() % 16 == 0:
+    if (K > 0 and rows > 0 and x.stride(1) == 1 and x.stride(0) % 8 == 0 and K <= x.stride(0) < 1 << 31  # lda is an int32
+            and x.data_ptr() % 16 == 0):
         return x, x.stride(0)
     ld = (K + 7) // 8 * 8
     out = torch.empty((rows, ld), dtype=x.dtype, device=x.device)

@@ -47,3 +47,12 @@ def test_gemm_refuses_host_operands():
     a = torch.zeros((8, 8), dtype=torch.bfloat16)
     with pytest.raises(SSAError):
         ssa.bf16_gemm(a, a)
+
+
+def test_rows_too_far_apart_for_the_call_are_copied():
+    """The call's row strides are 32-bit: columns of a matrix with 2^31 of them are copied together."""
+    x = torch.empty_strided((3, 64), (2 ** 31, 1), dtype=torch.bfloat16, device="meta")
+    rows, ld = ssa._tma_rows(x)
+    assert ld == 64 and rows.shape == (3, 64) and rows.stride(0) == 64
+    x = torch.empty_strided((3, 64), (2 ** 31 - 8, 1), dtype=torch.bfloat16, device="meta")
+    assert ssa._tma_rows(x)[1] == 2 ** 31 - 8
