@@ -192,25 +192,28 @@ __global__ void grn_prepare_kernel(const uint16_t *W1, const uint16_t *W2, const
 // The warp-per-trajectory forward's step (ssa_warp_body.cuh) over propensities kept by word: those of the hidden
 // productions are constant, an event changes one degradation and, for a hidden gene, the output productions. Bound
 // by instruction issue: 1,620 -> 796 warp instructions per step at 784-256-10.
+// W2S: W2 in shared memory; else its columns are read through L1 (networks where it leaves room for fewer warps).
+template <bool W2S>
 __global__ void __launch_bounds__(128, 6) grn_fwd_kernel(const GrnParams p, int record)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, W = blockDim.x >> 5;
     const int nh = p.n_hid, no = p.n_out, nd = p.n_dyn;
     int *s_W2fix = reinterpret_cast<int *>(smem);
-    float *s_d = reinterpret_cast<float *>(s_W2fix + no * nh);
+    const int w2_words = W2S ? no * nh : 0;
+    float *s_d = reinterpret_cast<float *>(s_W2fix + w2_words);
     float *s_b2 = s_d + nd;
     const int ndp = (nd + 3) & ~3, wide = wide_len(p.M), rounds = wide >> 7;
     const int nop = (no + 3) & ~3;
     const size_t per_warp = (size_t)ndp + wide + 2 * (size_t)nop;  // X, a, E2acc (2 words each)
     // offsets from the shared array itself (not through an integer round trip), so that every access below
     // compiles to a shared-memory load or store with 32-bit addressing
-    unsigned char *wb = smem + ((4 * ((size_t)no * nh + nd + ((no + 3) & ~3)) + 15) & ~(size_t)15);
+    unsigned char *wb = smem + ((4 * ((size_t)w2_words + nd + ((no + 3) & ~3)) + 15) & ~(size_t)15);
     int *X = reinterpret_cast<int *>(wb) + wib * per_warp;
     float *a = reinterpret_cast<float *>(X + ndp);
     long long *E2acc = reinterpret_cast<long long *>(a + wide);
 
-    for (int q = threadIdx.x; q < no * nh; q += blockDim.x) s_W2fix[q] = p.W2fix[q];
+    for (int q = threadIdx.x; q < w2_words; q += blockDim.x) s_W2fix[q] = p.W2fix[q];
     for (int q = threadIdx.x; q < nd; q += blockDim.x) s_d[q] = p.dvec[q];
     for (int q = threadIdx.x; q < no; q += blockDim.x) s_b2[q] = p.b2[q];
     __syncthreads();
@@ -281,7 +284,7 @@ __global__ void __launch_bounds__(128, 6) grn_fwd_kernel(const GrnParams p, int 
         }
         if (sp < nh) {
             for (int o = lane; o < no; o += 32) {
-                E2acc[o] += (long long)delta * s_W2fix[o * nh + sp];
+                E2acc[o] += (long long)delta * (W2S ? s_W2fix[o * nh + sp] : __ldg(p.W2fix + o * nh + sp));
                 a[nh + o + 1] = p.k_max * sigmoid_f(e2_value(E2acc[o], scale, s_b2[o]));
             }
         }
@@ -1069,12 +1072,12 @@ int grn_dw1_nt(const ssa_grn *g) { return (g->n_in % 112 == 0) ? 112 : 64; }
 // shared memory one CTA may hold on sm_103a
 constexpr size_t kGrnMaxSmem = 227 * 1024;
 
-size_t grn_fwd_smem(const ssa_grn *g, int warps)
+size_t grn_fwd_smem(const ssa_grn *g, int warps)  // without W2
 {
     const int ndp = (g->n_dyn + 3) & ~3, nop = (g->n_out + 3) & ~3;
-    return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop) + 16 +
-           4 * (size_t)warps * (ndp + wide_len(g->M) + 2 * (size_t)nop);
+    return 4 * ((size_t)g->n_dyn + nop) + 16 + 4 * (size_t)warps * (ndp + wide_len(g->M) + 2 * (size_t)nop);
 }
+size_t grn_fwd_smem_w2(const ssa_grn *g, int warps) { return grn_fwd_smem(g, warps) + 4 * (size_t)g->n_out * g->n_hid; }
 
 bool grn_sums_in_registers(const ssa_grn *g) { return g->n_dyn <= kGrnRegSpecies; }  // 288 = 9 rounds
 
@@ -1085,11 +1088,14 @@ size_t grn_adj_smem(const ssa_grn *g, int warps)
            4 * (size_t)warps * grn_adj_words(g->n_hid, g->n_out, !grn_sums_in_registers(g));
 }
 
-// warps per block of the exact forward and its adjoint
-int grn_warps(const ssa_grn *g)
+// Warps per block: four, or as many as the kernel's own per-warp arrays leave room for. The exact forward gives up W2's place
+// in shared memory before it gives up a warp: 1,024 trajectories of 3,000-10, a forward to t = 0.3 in 29.3 ms with two
+// warps beside W2, 15.9 with four and W2 through L1 (28.0 with four and W2 before the propensities were kept); 3,800-4 76.5
+// with the adjoint's one warp, 23.9 with four.
+int grn_warps(size_t (*smem)(const ssa_grn *, int), const ssa_grn *g)
 {
     int w = kGrnWarps;
-    while (w > 1 && std::max(grn_fwd_smem(g, w), grn_adj_smem(g, w)) > kGrnMaxSmem) --w;
+    while (w > 1 && smem(g, w) > kGrnMaxSmem) --w;
     return w;
 }
 
@@ -1115,13 +1121,6 @@ size_t grn_soft_adj_smem(const ssa_grn *g, int warps)
 {
     const size_t nop = (g->n_out + 3) & ~3;
     return 4 * ((size_t)g->n_out * g->n_hid + g->n_dyn + nop + warps * grn_soft_adj_words(g->n_hid, g->n_out)) + 16;
-}
-
-int grn_soft_warps(const ssa_grn *g)
-{
-    int w = kGrnWarps;
-    while (w > 1 && std::max(grn_soft_fwd_smem(g, w), grn_soft_adj_smem(g, w)) > kGrnMaxSmem) --w;
-    return w;
 }
 
 WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, const ssa_fwd_opts *o)
@@ -1164,7 +1163,7 @@ WsLayout grn_layout(const ssa_grn *g, int64_t n_img, int64_t tpi, int32_t S, con
         const int K = o->selector == SSA_SELECT_SOFT ? kGrnSoftK : o->ckpt_interval > 0 ? o->ckpt_interval : 64;
         L.ev_rows = (o->max_steps + 7) / 8;
         L.n_ckpt = o->max_steps / K + 1;
-        const int wpb = o->selector == SSA_SELECT_SOFT ? grn_soft_warps(g) : grn_warps(g);
+        const int wpb = grn_warps(o->selector == SSA_SELECT_SOFT ? grn_soft_adj_smem : grn_adj_smem, g);
         L.max_blocks = (n + wpb - 1) / wpb;
         L.xfinal = take((size_t)g->n_dyn * n * 4);
         L.ev = take((size_t)L.ev_rows * n * sizeof(uint4));
@@ -1335,7 +1334,7 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
     }
     if (n > 0 && soft) {
         p.invT = 1.0f / opts->temperature;
-        const int wpb = grn_soft_warps(g);
+        const int wpb = grn_warps(grn_soft_fwd_smem, g);
         const size_t smem = grn_soft_fwd_smem(g, wpb);
         auto kern = hot_weights(p.invT) ? grn_soft_fwd_kernel<true> : grn_soft_fwd_kernel<false>;
         GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -1343,10 +1342,13 @@ extern "C" ssa_status ssa_grn_forward(const ssa_grn *g, const uint16_t *W1, cons
             p, reinterpret_cast<float *>(obs_out), opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     } else if (n > 0) {
-        const int wpb = grn_warps(g);
-        const size_t smem = grn_fwd_smem(g, wpb);
-        GRN_CUDA_TRY(cudaFuncSetAttribute(grn_fwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        grn_fwd_kernel<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(p, opts->record);
+        const int wpb = grn_warps(grn_fwd_smem, g);
+        // (a network whose W2 leaves no room for one warp is refused by the launch, as it always was)
+        const bool w2s = grn_fwd_smem_w2(g, wpb) <= kGrnMaxSmem || grn_fwd_smem_w2(g, 1) > kGrnMaxSmem;
+        const size_t smem = w2s ? grn_fwd_smem_w2(g, wpb) : grn_fwd_smem(g, wpb);
+        auto kern = w2s ? grn_fwd_kernel<true> : grn_fwd_kernel<false>;
+        GRN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kern<<<(unsigned)((n + wpb - 1) / wpb), 32 * wpb, smem, st>>>(p, opts->record);
         GRN_CUDA_TRY(cudaGetLastError());
     }
     if (n > 0 && draws_out) GRN_CUDA_TRY(cudaMemcpyAsync(draws_out, p.draws, (size_t)n * 4, cudaMemcpyDeviceToDevice, st));
@@ -1433,7 +1435,7 @@ extern "C" ssa_status ssa_grn_backward(ssa_run *run, const float *dl_dobs, int64
     p.err = flag + 1;
     p.n_ckpt = L.n_ckpt;
     p.seg = soft ? reinterpret_cast<float *>(ws + L.soft_seg) : nullptr;
-    const int wpb = soft ? grn_soft_warps(g) : grn_warps(g);
+    const int wpb = grn_warps(soft ? grn_soft_adj_smem : grn_adj_smem, g);
     const bool hot = hot_weights(p.invT);
     const int64_t nblk = (n + wpb - 1) / wpb;
     float *red = reinterpret_cast<float *>(ws + L.red);
