@@ -652,7 +652,7 @@ __device__ __forceinline__ void bin_held_run(const FwdParams &p, int64_t i, int 
 
 // The same with the runs in shared memory, one column per thread (the network-specialised kernels): the warp reads a
 // run by broadcast instead of passing it from a lane's local array by shuffles. The ninth entry takes the held tail.
-// Ion channel (262,144 trajectories, 800 bins, recorded): 345 -> 320 us with 44% fewer instructions; what is left are
+// Ion channel (262,144 trajectories, 800 bins, recorded): 345 -> 307 us with 44% fewer instructions; what is left are
 // the stores (839 MB, 250 us at half the copy rate; 16-byte stores make no difference).
 struct BinRunsShared {
     int n, slots;

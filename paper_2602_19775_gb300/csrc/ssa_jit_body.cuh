@@ -511,7 +511,7 @@ __device__ __forceinline__ void jit_fwd_direct(const FwdParams &p)
 // 32 bins a chunk) by the float. s_chunk [rows][kJitAdjBlock], a row a chunk; whether they are formed is the launch's
 // choice (jit_chunk_shift). Where intervals hold few bins they neither cost nor save (2A <-> B, 200 bins in 250 steps).
 // Ion channel, 262,144 trajectories x 800 bins, the adjoint: 2,050 us bin by bin; 800 with the sum of every interval
-// formed by the warp beforehand (a reduction per interval and row); 395 so.
+// formed by the warp beforehand (a reduction per interval and row); 387 so.
 // The chunk sums share the block sums' memory (28 KB of their own, also where unused: relaxed 2A <-> B 0.79 -> 0.86 ms).
 constexpr int kJitAdjBlock = 128;
 

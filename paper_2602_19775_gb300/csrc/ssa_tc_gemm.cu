@@ -443,8 +443,9 @@ __global__ void __launch_bounds__(128, 1) tc_gemm_sw128_kernel(const __grid_cons
 // epilogue warps write a tile while the next one is multiplied. Warp 0 loads (TMA), warp 1 issues tcgen05.mma, warps
 // 2 to 5 read TMEM lanes 32 (warp % 4) ... and store. BN (a multiple of 16 up to 256) is the launch's: the width that
 // takes the fewest rounds of the SMs times columns (sw_tile_columns).
-// 4096 x 4096 x 4096: 126 -> 116 us (one tile per CTA, 128 x 256, the epilogue after the tile), bound by the operand
-// reads from L2 (44 KB per SM and K block of 64).
+// One tile per CTA (128 x 256) with the epilogue after it, and so: 4096 cubed 128 and 117 us, 8192 cubed 819 and 800, 3000
+// cubed 72 and 73, 2304 cubed 44 and 37, 2048 cubed 22 and 24, 4500 cubed (rows that fill no lines) 228 both. Bound by the
+// operand reads from L2 (44 KB per SM and K block of 64): the tensor pipe is active 55% of the time at 4096 cubed.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
@@ -711,7 +712,8 @@ static int sw_split(int M, int N, int K, int *per)
 }
 
 // Columns of a tile of the persistent kernel: the multiple of 16 that takes the fewest rounds of one tile per SM times
-// the columns of a tile (48 more stand for a tile's fixed cost); ties take the wider tile. Below 128 columns the
+// the columns of a tile (48 more stand for a tile's fixed cost: 3000 cubed takes 256 columns and 73 us, with 16 more 160
+// columns and 78); ties take the wider tile. Below 128 columns the
 // instruction's time no longer falls with its width. 4096 x 4096 on 152 SMs: 224 columns, 608 tiles, exactly four rounds.
 static int sw_tile_columns(int M, int N, int sms)
 {
