@@ -169,10 +169,7 @@ __device__ __forceinline__ float ex2_approx(float v)
 // 1/E = -1/ln u of the uniform of a Philox word, for the adjoints' soft weights (the forward's clock and race use
 // neg_log_unit). With v = 1 - u, 1/E = 1/v - P(v) where P = 1/v + 1/ln(1 - v) is smooth (1/2 + v/12 + v^2/24 + ...):
 // below v = 1/2 a degree-6 fit of P (weighted least squares towards the smallest relative error of 1/E, 2^-25.9)
-// and one approximate reciprocal; above it ln u is away from 0 and the hardware log2 is accurate in relative terms. That
-// log2 comes out nearer to 0 than it is, by 1.1e-7 of a log2 key on average over the words: ln 2 is taken one unit in the
-// last place up, which leaves -2e-8 (the half below: 8e-9). With the bias the gradients of 2A <-> B (250 steps, T = 0.1)
-// were 6.2e-7 from binary64, without it 4.2e-7; with logf and log2 keys 4.4e-7.
+// and one approximate reciprocal; above it ln u is away from 0 and the hardware log2 is accurate in relative terms.
 // 16 issue slots against 32 of logf and a division.
 __device__ __forceinline__ float inv_exp_of_word(uint32_t x)
 {
@@ -184,7 +181,7 @@ __device__ __forceinline__ float inv_exp_of_word(uint32_t x)
     p = __fmaf_rn(p, v, 0x1.63387p-5f);
     p = __fmaf_rn(p, v, 0x1.54e3ecp-4f);
     p = __fmaf_rn(p, v, 0x1.00004ep-1f);
-    const float near = rcp_approx(v) - p, far = rcp_approx(lg2_approx(1.0f - v) * -0x1.62e432p-1f);
+    const float near = rcp_approx(v) - p, far = rcp_approx(lg2_approx(1.0f - v) * -0x1.62e430p-1f);
     float r;  // a select, never a branch
     asm("{\n\t.reg .pred p;\n\tsetp.lt.f32 p, %3, 0f3F000000;\n\tselp.f32 %0, %1, %2, p;\n\t}"
         : "=f"(r) : "f"(near), "f"(far), "f"(v));
