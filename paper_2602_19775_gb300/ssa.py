@@ -461,6 +461,8 @@ def bf16_gemm(A: torch.Tensor, B: torch.Tensor, bias: torch.Tensor | None = None
         raise SSAError("bf16_gemm takes bfloat16 operands")
     if not A.is_cuda:
         raise SSAError("bf16_gemm takes CUDA tensors")
+    if A.device.index == torch.cuda.current_device():
+        return _bf16_gemm_here(A, B, bias, stream, split_k)
     with torch.cuda.device(A.device):  # the kernel runs where A lies, on that device's stream
         return _bf16_gemm_here(A, B, bias, stream, split_k)
 

@@ -37,6 +37,7 @@ def test_gemm_runs_on_the_device_of_its_operand(monkeypatch):
         seen.append(("leave", d))
 
     monkeypatch.setattr(torch.cuda, "device", device)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     monkeypatch.setattr(ssa, "_bf16_gemm_here", lambda *a: seen.append(("run", a[0].device)))
     here = torch.device("cuda:1")
     ssa.bf16_gemm(_On(here), _On(here))
