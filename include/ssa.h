@@ -187,6 +187,8 @@ ssa_status ssa_forward_replay(const ssa_network *net, const float *log_rates, in
  *                  [n_traj][n_samples][n_obs] array, or 0 when every trajectory has the same
  *                  upstream gradient (a loss on ensemble means, Section 3.5).
  *   temperature    T > 0 (Eq. 3); for a soft forward (SSA_SELECT_SOFT) the forward's T.
+ *                  Above T = 5 the network-specialised adjoint is a program of its own, compiled at the
+ *                  first such call of a network (as the soft forward's is at its first).
  *   dl_dlog_rates  device float [P], overwritten with dL/dtheta summed over trajectories
  *                  (deterministic reduction order).
  * Trajectories whose status is not OK/ABSORBED/STEP_CAP contribute nothing. Callable any number
