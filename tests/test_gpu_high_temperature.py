@@ -123,3 +123,22 @@ def test_relaxed_classifier_slow_degradation_keeps_its_weight():
     assert same.mean() > 0.95
     err = np.abs(fw.obs.double().cpu().numpy() - orc.obs)[same]
     assert err.max() <= 1e-3 * np.abs(orc.obs).max()
+
+
+def test_first_high_temperature_gradient_inside_a_capture():
+    """The specialised kernels' program for high temperatures is compiled at its first use, which may be in a capture."""
+    from paper_2602_19775_gb300 import ssa
+    spec, n = _slow_reaction(4), 64
+    fw = ssa.forward(ssa.Network(spec), torch.tensor(spec.log_rates.astype(np.float32), device="cuda"), n, spec.x0, 3.0,
+                     [1.5, 3.0], [0, 1], 3, readout="linear", record=True, max_steps=512)
+    dl = torch.tensor(W.seeded_dl_dobs(4, n, 2, 2, scale=1.0 / n), dtype=torch.float32, device="cuda")
+    out = torch.zeros(spec.n_params, device="cuda")
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        graph.capture_begin()
+        ssa.backward(fw, dl, 20.0, out=out)
+        graph.capture_end()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, ssa.backward(fw, dl, 20.0)) and torch.count_nonzero(out) > 0
